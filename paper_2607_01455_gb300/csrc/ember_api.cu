@@ -29,12 +29,11 @@ Layout make_layout(int64_t V, int64_t D, int64_t max_sparse_N)
     L.colpart = take(sizeof(float) * (size_t)kPartRows * (size_t)D);
     if (max_sparse_N > 0) {
         const size_t N = (size_t)max_sparse_N;
-        const size_t Npad = (N + kSortTile - 1) / kSortTile * kSortTile;
         const size_t nslices = (size_t)((D + kThreads - 1) / kThreads);
-        L.sp_keys = take(sizeof(uint64_t) * Npad);
-        L.sp_rank = take(sizeof(int32_t) * Npad);
-        L.sp_sorted = take(sizeof(uint64_t) * N);
-        L.sp_tilecnt = take(sizeof(int32_t) * 2 * (Npad / kSortTile));
+        L.sp_arr = take(sizeof(int32_t) * N);
+        L.sp_rng = take(sizeof(int32_t) * kScanCounters);
+        L.sp_long = take(sizeof(int32_t) * (N / kLongRun + 1));
+        L.sp_placed = take(sizeof(int32_t) * N);
         L.sp_perm = take(sizeof(int32_t) * N);
         L.sp_segidx = take(sizeof(int32_t) * N);
         L.sp_uniq = take(sizeof(int32_t) * N);
@@ -161,10 +160,12 @@ ember_status ember_bind_workspace(ember_handle *h, void *workspace, size_t bytes
     if (cudaMemsetAsync((unsigned char *)workspace + L.scalars, 0, sizeof(DevScalars),
                         (cudaStream_t)stream) != cudaSuccess)
         return EMBER_ERR_CUDA;
-    // the sparse step expects an all-zero slot map and leaves it all-zero
+    // the sparse step expects an all-zero slot map and counters and leaves them all-zero
     if (max_sparse_N > 0 &&
-        cudaMemsetAsync((unsigned char *)workspace + L.sp_slot, 0, sizeof(int32_t) * (size_t)h->V,
-                        (cudaStream_t)stream) != cudaSuccess)
+        (cudaMemsetAsync((unsigned char *)workspace + L.sp_slot, 0, sizeof(int32_t) * (size_t)h->V,
+                         (cudaStream_t)stream) != cudaSuccess ||
+         cudaMemsetAsync((unsigned char *)workspace + L.sp_rng, 0, sizeof(int32_t) * kScanCounters,
+                         (cudaStream_t)stream) != cudaSuccess))
         return EMBER_ERR_CUDA;
     h->ws = (unsigned char *)workspace;
     h->ws_bytes = bytes;

@@ -28,12 +28,10 @@ constexpr int kPartRows = kSparseCtas > kGridCtas ? kSparseCtas : kGridCtas;
 // warps, so that each warp adds few per-CTA partial rows).  Its row pass runs
 // up to kMaxRowCtas CTAs: about one row per thread for the LM-head step (whose
 // rows each sum ceil(D/256) slices) and for a dense step in column panels
-// (one slice per panel), and kRowBatch rows per thread for the sparse step
-// (whose untouched rows only decay).
+// (one slice per panel), and one touched row per thread for the sparse step.
 constexpr int kStateCols = 32;
 constexpr int kStateThreads = 512;
 constexpr int kMaxRowCtas = 1024;
-constexpr int kRowBatch = 8;
 constexpr int kRsumParts = kMaxRowCtas > kGridCtas ? kMaxRowCtas : kGridCtas;
 
 // Bits of the sticky device flag.
@@ -53,10 +51,19 @@ struct DevScalars {
     int32_t n_valid;   // sparse step: number of ids inside [0, V)
 };
 
-// Sparse step: ids are sorted in tiles of kSortTile keys by kSortThreads
-// threads.
-constexpr int kSortTile = 1024;
-constexpr int kSortThreads = 256;
+// Sparse step, dedup kernels: kSpThreads threads (kOrderThreads in the last),
+// kCountKeys occurrences per CTA of the count.  The
+// ids are split into at most kScanCtas equal ranges of at least kScanMin ids,
+// one CTA of the scan each (two per SM; smaller ranges would add up more
+// counts of ranges before them than they hold ids).  A run longer than
+// kLongRun occurrences is put in order by a CTA, a shorter one by its threads.
+constexpr int kSpThreads = 256;
+constexpr int kOrderThreads = 512;
+constexpr int kCountKeys = 1024;
+constexpr int kScanCtas = kGridCtas;
+constexpr int kScanMin = 256;
+constexpr int kScanCounters = 2 * kScanCtas + 1;  // two per range, then the number of long runs
+constexpr int kLongRun = 128;
 
 // Workspace layout (byte offsets, each 256-byte aligned).
 struct Layout {
@@ -64,12 +71,11 @@ struct Layout {
     size_t rsum_part;   // float[kRsumParts]            sum of new r per CTA
     size_t csum_part;   // float[ceil(D/32)]            sum of new c per 32-column group
     size_t colpart;     // float[kPartRows * D]     column sums of g^2 per CTA
-    // sparse step (present when max_sparse_N > 0); N = max_sparse_N,
-    // Npad = N rounded up to kSortTile
-    size_t sp_keys;     // uint64[Npad]  (id << 32 | occurrence), sorted within tiles
-    size_t sp_rank;     // int32[Npad]   global rank of each tile-sorted key
-    size_t sp_sorted;   // uint64[N]     keys in (id, occurrence) order
-    size_t sp_tilecnt;  // int32[2 * Npad / kSortTile]  heads and valid ids per tile
+    // sparse step (present when max_sparse_N > 0), N = max_sparse_N
+    size_t sp_arr;      // int32[N]      arrival number of each occurrence within its id
+    size_t sp_rng;      // int32[kScanCounters]  counts per id range and of long runs; zero between steps
+    size_t sp_long;     // int32[N / kLongRun + 1]  distinct-id index of each long run
+    size_t sp_placed;   // int32[N]      occurrences in id order, unordered within a run
     size_t sp_perm;     // int32[N]      occurrence index at each sorted position
     size_t sp_segidx;   // int32[N]      distinct-id index at each sorted position
     size_t sp_uniq;     // int32[N]      distinct ids, ascending

@@ -12,19 +12,15 @@
 //   - only the touched rows of W change.
 //
 // Kernels, in launch order:
-//   sort      k_sp_tile_sort, k_sp_rank, k_sp_scatter: the N keys
-//             (id << 32 | occurrence) in ascending order, without atomics on
-//             floating-point data: 1024-key tiles are bitonic-sorted in shared
-//             memory, then every key's global rank is its rank in its tile
-//             plus its lower bound in every other tile (integer atomics, so
-//             the rank is exact and the order deterministic).  The same
-//             searches find the run heads: a key heads its id's run unless
-//             some tile holds a smaller key of the same id, which is then the
-//             key just below it in that tile.  The scatter counts the heads
-//             and the valid ids of every tile of sorted positions.
-//   dedup     k_sp_segments: the distinct ids (ascending), where each id's
-//             run starts, and a V-entry map from a touched row to its
-//             distinct-id index.
+//   dedup     a counting sort by id, linear in N and V, in integer atomics:
+//             k_sp_count counts each id's occurrences in the V-entry map and
+//             hands every occurrence an arrival number; k_sp_scan turns the
+//             counts into the distinct ids (ascending) and where each id's run
+//             starts, and decays r on the rows whose count is zero; k_sp_place
+//             puts every occurrence at its run's start plus its arrival
+//             number; k_sp_order sorts each run by occurrence, so that
+//             arrival order (the only thing that varies from run to run)
+//             leaves no trace.
 //   segsum    k_sp_segsum, k_sp_carry: the summed gradient row of every
 //             distinct id, adding its occurrences in increasing occurrence
 //             order (compensated fp32 sums); per (id, column slice) sums of
@@ -35,8 +31,8 @@
 //             a run that crosses worker boundaries leaves one piece per
 //             worker, which k_sp_carry adds in worker order.
 //   state     the dense step's column/normaliser pass, whose launch also runs
-//             the row pass: r for all V rows, the sums of new r per CTA, and
-//             the touched-row map cleared for the next step.
+//             the row pass: r for the touched rows, the sums of new r per
+//             CTA, and the touched-row map cleared for the next step.
 //   apply     k_sp_apply: the update of the touched rows only (once per
 //             column panel for tables wider than a CTA holds).
 //
@@ -53,295 +49,270 @@ namespace {
 
 using namespace dev;
 
-constexpr uint64_t kPad = ~0ull;
-// Bit of a key's rank word set when the key is not the head of its id's run
-// (ranks stay below 2^30: N <= INT32_MAX / 2).
-constexpr int kNotHead = 1 << 30;
-constexpr int kKeysPerThread = kSortTile / kSortThreads;
-
-// keys a <= b afterwards when `up`, a >= b otherwise
-__device__ __forceinline__ void cmp_swap(uint64_t &a, uint64_t &b, bool up)
+// Inclusive scan of x over a warp.
+__device__ __forceinline__ int warp_scan(int x, int lane)
 {
-    if ((a > b) == up) {
-        const uint64_t x = a;
-        a = b;
-        b = x;
-    }
-}
-
-__device__ __forceinline__ uint64_t shfl_xor_u64(uint64_t x, int m)
-{
-    const uint32_t lo = __shfl_xor_sync(0xffffffffu, (uint32_t)x, m);
-    const uint32_t hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(x >> 32), m);
-    return ((uint64_t)hi << 32) | lo;
-}
-
-// Bitonic sort of one tile of kSortTile keys, thread t holding keys
-// 4t .. 4t + 3.  For the compare-exchange of keys i and i ^ j at merge size
-// k, both holders keep min or max by the same rule: the lower index of the
-// pair keeps the min when the block (i & k) sorts ascending.  Partners at
-// distance 1 or 2 are in the same thread, distance 4 .. 64 in the same warp
-// (shuffles), and only distances 128 .. 512 go through shared memory.
-template <typename IdT>
-__global__ void __launch_bounds__(kSortThreads)
-k_sp_tile_sort(const IdT *__restrict__ ids, int64_t N, int64_t V, uint64_t *__restrict__ keys,
-               int32_t *__restrict__ rank, int32_t *__restrict__ tilecnt, DevScalars *sc)
-{
-    static_assert(kSortTile == 4 * kSortThreads, "four keys per thread");
-    __shared__ uint64_t s[kSortTile];
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    const int t = threadIdx.x;
-    grid_dep_wait();  // first kernel of a step: returns at once
-    grid_dep_launch();
-    bool bad = false;
-    uint64_t key[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int64_t k = base + 4 * t + q;
-        key[q] = kPad;
-        if (k < N) {
-            int64_t id = (int64_t)ids[k];
-            if (id < 0 || id >= V) {  // skipped: sorts after every valid id
-                bad = true;
-                id = V;
-            }
-            key[q] = ((uint64_t)id << 32) | (uint64_t)k;
-        }
-    }
-    if (bad)
-        atomicOr(&sc->flags, kFlagIdRange);
-
-    for (int k = 2; k <= kSortTile; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= 128) {  // partner in another warp
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    s[4 * t + q] = key[q];
-                __syncthreads();
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int i = 4 * t + q;
-                    const uint64_t o = s[i ^ j];
-                    const bool keep_min = ((i & j) == 0) == ((i & k) == 0);
-                    key[q] = keep_min ? (key[q] < o ? key[q] : o) : (key[q] > o ? key[q] : o);
-                }
-                __syncthreads();
-            } else if (j >= 4) {  // partner in this warp
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int i = 4 * t + q;
-                    const uint64_t o = shfl_xor_u64(key[q], j >> 2);
-                    const bool keep_min = ((i & j) == 0) == ((i & k) == 0);
-                    key[q] = keep_min ? (key[q] < o ? key[q] : o) : (key[q] > o ? key[q] : o);
-                }
-            } else {  // partner in this thread: pairs (0,1),(2,3) or (0,2),(1,3)
-                const bool up = ((4 * t) & k) == 0;  // for k >= 4 the same for all four keys
-                if (j == 1) {
-                    cmp_swap(key[0], key[1], k == 2 ? (((4 * t) & 2) == 0) : up);
-                    cmp_swap(key[2], key[3], k == 2 ? (((4 * t + 2) & 2) == 0) : up);
-                } else {
-                    cmp_swap(key[0], key[2], up);
-                    cmp_swap(key[1], key[3], up);
-                }
-            }
-        }
-    }
-    // rank within the tile, and kNotHead where the key before it in the
-    // tile has the same id; the scatter's counts of this tile start at zero
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        s[4 * t + q] = key[q];
-    if (t < 2)
-        tilecnt[2 * blockIdx.x + t] = 0;
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int i = 4 * t + q;
-        const bool same = i > 0 && (s[i - 1] >> 32) == (key[q] >> 32);
-        keys[base + i] = key[q];
-        rank[base + i] = i | (same ? kNotHead : 0);
-    }
-}
-
-// CTA (own, other): add to each key of tile `own` the number of keys of tile
-// `other` below it.  Keys are unique, so the ranks form a permutation.  A key
-// whose lower bound in `other` follows a key of the same id is not the head
-// of its id's run.
-__global__ void __launch_bounds__(kSortThreads)
-k_sp_rank(const uint64_t *__restrict__ keys, int32_t *__restrict__ rank)
-{
-    const int own = blockIdx.x, other = blockIdx.y;
-    grid_dep_wait();  // tile-sorted keys
-    grid_dep_launch();
-    if (own == other)
-        return;
-    __shared__ uint64_t s[kSortTile];
-#pragma unroll
-    for (int q = 0; q < kKeysPerThread; ++q) {
-        const int i = threadIdx.x + q * kSortThreads;
-        s[i] = keys[(int64_t)other * kSortTile + i];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kKeysPerThread; ++q) {
-        const int64_t at = (int64_t)own * kSortTile + threadIdx.x + q * kSortThreads;
-        const uint64_t x = keys[at];
-        if (x == kPad)
-            continue;
-        int lo = 0, hi = kSortTile;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (s[mid] < x)
-                lo = mid + 1;
-            else
-                hi = mid;
-        }
-        if (lo) {
-            atomicAdd(&rank[at], lo);
-            if ((s[lo - 1] >> 32) == (x >> 32))
-                atomicOr(&rank[at], kNotHead);
-        }
-    }
-}
-
-// Keys to their sorted positions, and per tile of sorted positions the
-// number of run heads and of valid ids (counted per warp, then one integer
-// atomic per tile a warp touches).  npad is a multiple of the warp size, so
-// every lane of a warp takes the same iterations.
-__global__ void k_sp_scatter(const uint64_t *__restrict__ keys, const int32_t *__restrict__ rank,
-                             int64_t npad, int64_t V, uint64_t *__restrict__ sorted, int32_t *__restrict__ tilecnt)
-{
-    grid_dep_wait();  // ranks
-    grid_dep_launch();
-    const int lane = threadIdx.x & 31;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < npad;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t x = keys[q];
-        const int rk = rank[q];
-        const bool real = x != kPad;
-        const int pos = rk & ~kNotHead;
-        if (real)
-            sorted[pos] = x;
-        const bool valid = real && (int64_t)(x >> 32) < V;
-        const bool head = valid && !(rk & kNotHead);
-        const int tile = real ? pos / kSortTile : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, tile);
-        const int nh = __popc(__ballot_sync(0xffffffffu, head) & peers);
-        const int nv = __popc(__ballot_sync(0xffffffffu, valid) & peers);
-        if (real && lane == __ffs(peers) - 1) {
-            if (nh)
-                atomicAdd(&tilecnt[2 * tile], nh);
-            if (nv)
-                atomicAdd(&tilecnt[2 * tile + 1], nv);
-        }
-    }
-}
-
-__device__ __forceinline__ int block_sum_int(int x, int *sh)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1)
-        x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0)
-        sh[w] = x;
-    __syncthreads();
-    int t = 0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q)
-        t += sh[q];
-    __syncthreads();
-    return t;
-}
-
-// Distinct ids and their runs.  Thread t of tile b owns sorted positions
-// kSortTile b + 4 t .. + 3; an exclusive scan of run heads numbers the ids.
-__global__ void __launch_bounds__(kSortThreads)
-k_sp_segments(const uint64_t *__restrict__ sorted, int64_t N, int64_t V,
-              const int32_t *__restrict__ tilecnt, int32_t *__restrict__ uniq,
-              int32_t *__restrict__ segoff, int32_t *__restrict__ perm, int32_t *__restrict__ segidx,
-              int32_t *__restrict__ slot, int32_t *__restrict__ single, DevScalars *sc)
-{
-    __shared__ int pre[2];
-    __shared__ int wsum[kSortThreads / 32];
-    __shared__ int sh[kSortThreads / 32];
-    grid_dep_wait();  // per-tile counts
-    grid_dep_launch();
-    {
-        // run heads and valid ids of the tiles before this one: a thread per
-        // tile, then the block's sums (one trip to L2, not one per tile)
-        int a = 0, b = 0;
-        for (int t = threadIdx.x; t < (int)blockIdx.x; t += kSortThreads) {
-            a += tilecnt[2 * t];
-            b += tilecnt[2 * t + 1];
-        }
-        a = block_sum_int(a, sh);
-        b = block_sum_int(b, sh);
-        if (threadIdx.x == 0) {
-            pre[0] = a;
-            pre[1] = b;
-        }
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t p0 = (int64_t)blockIdx.x * kSortTile + (int64_t)threadIdx.x * kKeysPerThread;
-    uint64_t key[kKeysPerThread];
-    bool valid[kKeysPerThread], head[kKeysPerThread];
-    int nh = 0, nv = 0;
-#pragma unroll
-    for (int q = 0; q < kKeysPerThread; ++q) {
-        const int64_t p = p0 + q;
-        valid[q] = head[q] = false;
-        key[q] = kPad;
-        if (p < N) {
-            key[q] = sorted[p];
-            const uint64_t id = key[q] >> 32;
-            valid[q] = (int64_t)id < V;
-            head[q] = valid[q] && (p == 0 || (sorted[p - 1] >> 32) != id);
-        }
-        nh += head[q];
-        nv += valid[q];
-    }
-    // exclusive scan of nh over the block
-    int x = nh;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o)
             x += y;
     }
-    if (lane == 31)
-        wsum[w] = x;
-    __syncthreads();
-    int before = 0;
-    for (int q = 0; q < w; ++q)
-        before += wsum[q];
-    int run = pre[0] + before + x - nh;  // heads before my first position
+    return x;
+}
+
+// ---------------------------------------------------------------------------
+// Dedup.  The cost is a few trips to L2 per kernel, whatever the number of
+// occurrences: sorting 1024-key tiles and ranking every key in every other
+// tile took 23.7 us for 32768 ids and 313 us for 262144, most of it the
+// ranks, which grow with the square of N.
+// ---------------------------------------------------------------------------
+
+// slot[id] <- how often the id occurs; arr[k] <- how many of its occurrences
+// arrived before occurrence k (any order: k_sp_order undoes it).  A CTA adds
+// up the equal ids of its kCountKeys occurrences in a hash table in shared
+// memory first and makes one global atomic per id: a frequent id's atomics
+// queue on one address at about 3 ns each (one per warp took 27 us on 262144
+// Zipf ids).  An id that finds its table entry taken goes to the map
+// directly.  rng[2 q], rng[2 q + 1]: distinct ids and occurrences in the ids
+// [q len, (q + 1) len).
+template <typename IdT>
+__global__ void __launch_bounds__(kSpThreads)
+k_sp_count(const IdT *__restrict__ ids, int64_t N, int64_t V, int32_t *__restrict__ slot,
+           int32_t *__restrict__ arr, int32_t *__restrict__ rng, unsigned len, int nrange, DevScalars *sc)
+{
+    constexpr int kTab = kCountKeys;  // a power of two
+    constexpr int kPer = kCountKeys / kSpThreads;
+    __shared__ int tag[kTab], num[kTab];
+    __shared__ int cnt[2 * kScanCtas];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t k0 = (int64_t)blockIdx.x * kCountKeys + tid;
+    int id[kPer];
+    bool bad = false;
 #pragma unroll
-    for (int q = 0; q < kKeysPerThread; ++q) {
-        const int64_t p = p0 + q;
-        if (head[q]) {
-            const int id = (int)(key[q] >> 32);
-            uniq[run] = id;
-            segoff[run] = (int)p;
-            slot[id] = run + 1;
-            // an id seen once: its summed row is that occurrence's row
-            const bool once = p + 1 >= N || (sorted[p + 1] >> 32) != (uint64_t)id;
-            single[run] = once ? (int)(key[q] & 0xffffffffu) : -1;
-            ++run;
-        }
-        if (valid[q]) {
-            segidx[p] = run - 1;
-            perm[p] = (int)(key[q] & 0xffffffffu);
+    for (int e = 0; e < kPer; ++e) {
+        const int64_t k = k0 + e * kSpThreads;
+        id[e] = -1;
+        if (k < N) {
+            const int64_t x = (int64_t)ids[k];
+            if (x >= 0 && x < V)
+                id[e] = (int)x;
+            else
+                bad = true;  // skipped
         }
     }
-    const int tot_h = block_sum_int(nh, sh);
-    const int tot_v = block_sum_int(nv, sh);
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        const int U = pre[0] + tot_h;
-        const int nvalid = pre[1] + tot_v;
-        sc->n_unique = U;
-        sc->n_valid = nvalid;
-        segoff[U] = nvalid;
+    for (int q = tid; q < kTab; q += kSpThreads) {
+        tag[q] = -1;
+        num[q] = 0;
     }
+    for (int q = tid; q < 2 * nrange; q += kSpThreads)
+        cnt[q] = 0;
+    grid_dep_wait();  // first kernel of a step: returns at once
+    grid_dep_launch();
+    __syncthreads();
+    if (__any_sync(0xffffffffu, bad) && lane == 0)
+        atomicOr(&sc->flags, kFlagIdRange);
+    auto count_in = [&](int x, int n, int before) {  // n occurrences of x reached the map, after `before`
+        const unsigned q = (unsigned)x / len;
+        atomicAdd(&cnt[2 * q + 1], n);
+        if (before == 0)
+            atomicAdd(&cnt[2 * q], 1);
+    };
+    int at[kPer], mine[kPer];  // table entry (-1: none), arrival number so far
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+        const unsigned peers = __match_any_sync(0xffffffffu, id[e]);
+        const int lead = __ffs(peers) - 1;
+        const int n = __popc(peers);
+        int h = -1, m = 0;
+        if (id[e] >= 0 && lane == lead) {
+            h = (int)(((unsigned)id[e] * 2654435761u) >> 16) & (kTab - 1);  // Fibonacci hashing
+            const int old = atomicCAS(&tag[h], -1, id[e]);
+            if (old == -1 || old == id[e]) {
+                m = atomicAdd(&num[h], n);
+            } else {
+                h = -1;
+                m = atomicAdd(&slot[id[e]], n);
+                count_in(id[e], n, m);
+            }
+        }
+        at[e] = __shfl_sync(0xffffffffu, h, lead);
+        mine[e] = __shfl_sync(0xffffffffu, m, lead) + __popc(peers & ((1u << lane) - 1u));
+    }
+    __syncthreads();
+    {
+        // the table's ids to the map, all of a thread's atomics in one trip
+        constexpr int kE = kTab / kSpThreads;
+        int n[kE], x[kE], before[kE];
+#pragma unroll
+        for (int e = 0; e < kE; ++e) {
+            n[e] = num[tid + e * kSpThreads];
+            x[e] = tag[tid + e * kSpThreads];
+        }
+#pragma unroll
+        for (int e = 0; e < kE; ++e)
+            before[e] = n[e] ? atomicAdd(&slot[x[e]], n[e]) : 0;
+#pragma unroll
+        for (int e = 0; e < kE; ++e)
+            if (n[e]) {
+                num[tid + e * kSpThreads] = before[e];
+                count_in(x[e], n[e], before[e]);
+            }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+        const int64_t k = k0 + e * kSpThreads;
+        if (k < N)
+            arr[k] = id[e] < 0 ? -1 : mine[e] + (at[e] >= 0 ? num[at[e]] : 0);
+    }
+    for (int q = tid; q < 2 * nrange; q += kSpThreads)
+        if (cnt[q])
+            atomicAdd(&rng[q], cnt[q]);
+}
+
+// CTA b numbers the distinct ids of [b len, (b + 1) len): uniq, segoff (the
+// run's first position among the occurrences in id order), slot <- 1 + the
+// number.  Runs longer than kLongRun are listed for k_sp_order (in any
+// order).  With r: the rows outside the batch decay, r_i <- beta2 r_i (their
+// g is 0), and the CTA's fp32 sum of them goes to rsum_part[b]; the touched
+// rows are left to the state pass.  A CTA's loads are one trip to L2 when
+// its range is one tile (V up to kScanCtas x kScanTile).
+constexpr int kScanPer = 4;                        // ids per thread of a tile
+constexpr int kScanTile = kSpThreads * kScanPer;
+__global__ void __launch_bounds__(kSpThreads)
+k_sp_scan(int32_t *__restrict__ slot, int64_t V, int64_t len, const int32_t *__restrict__ rng,
+          int32_t *__restrict__ uniq, int32_t *__restrict__ segoff, int32_t *__restrict__ longrun,
+          int32_t *__restrict__ nlong, DevScalars *sc, float *__restrict__ r, EmaPair ema,
+          float *__restrict__ rsum_part)
+{
+    constexpr int kW = kSpThreads / 32;
+    __shared__ int wh[2][kW], wv[2][kW];
+    __shared__ float wr[kW];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int64_t i0 = (int64_t)blockIdx.x * len;
+    const int64_t i1 = i0 + len < V ? i0 + len : V;
+    grid_dep_wait();  // the counts
+    grid_dep_launch();
+    // distinct ids and occurrences of the ranges before this one
+    int h = 0, v = 0;
+    for (int q = tid; q < (int)blockIdx.x; q += kSpThreads) {
+        h += __ldcg(rng + 2 * q);
+        v += __ldcg(rng + 2 * q + 1);
+    }
+    h = __reduce_add_sync(0xffffffffu, h);
+    v = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0) {
+        wh[1][w] = h;
+        wv[1][w] = v;
+    }
+    float rsum = 0.f;
+    int run = 0, pos = 0;  // of the next tile (tile 0: added from wh[1] and wv[1])
+    int buf = 0;
+    for (int64_t t0 = i0; t0 < i1; t0 += kScanTile) {
+        const int64_t i = t0 + (int64_t)tid * kScanPer;  // len and kScanPer are multiples of 4
+        int c[kScanPer];
+        float rr[kScanPer];
+        const int4 c4 = (i + 3 < i1) ? __ldcg(reinterpret_cast<const int4 *>(slot + i)) : make_int4(0, 0, 0, 0);
+        c[0] = c4.x;
+        c[1] = c4.y;
+        c[2] = c4.z;
+        c[3] = c4.w;
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+            if (i + 3 >= i1)
+                c[e] = (i + e < i1) ? __ldcg(slot + i + e) : 0;
+            rr[e] = (r && i + e < i1) ? r[i + e] : 0.f;
+        }
+        int nh = 0, nv = 0;
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+            nh += c[e] > 0;
+            nv += c[e];
+        }
+        const int xh = warp_scan(nh, lane), xv = warp_scan(nv, lane);
+        if (lane == 31) {
+            wh[buf][w] = xh;
+            wv[buf][w] = xv;
+        }
+        __syncthreads();
+        if (t0 == i0) {
+#pragma unroll
+            for (int q = 0; q < kW; ++q) {
+                run += wh[1][q];
+                pos += wv[1][q];
+            }
+            __syncthreads();  // before the next tile writes wh[1]
+        }
+        int u = run + xh - nh, p = pos + xv - nv;
+#pragma unroll
+        for (int q = 0; q < kW; ++q) {
+            u += q < w ? wh[buf][q] : 0;
+            p += q < w ? wv[buf][q] : 0;
+            run += wh[buf][q];
+            pos += wv[buf][q];
+        }
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+            if (c[e] > 0) {
+                uniq[u] = (int)(i + e);
+                segoff[u] = p;
+                if (c[e] > kLongRun)
+                    longrun[atomicAdd(nlong, 1)] = u;
+                ++u;
+                slot[i + e] = u;
+                p += c[e];
+            } else if (r && i + e < i1) {
+                const float rn = ema_pair(ema, rr[e], 0.f);
+                r[i + e] = rn;
+                rsum += rn;
+            }
+        }
+        buf ^= 1;
+    }
+    if (blockIdx.x == gridDim.x - 1 && tid == 0) {
+        sc->n_unique = run;
+        sc->n_valid = pos;
+        segoff[run] = pos;
+    }
+    if (r) {
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1)
+            rsum += __shfl_xor_sync(0xffffffffu, rsum, o);
+        if (lane == 0)
+            wr[w] = rsum;
+        __syncthreads();
+        if (tid == 0) {
+            float t = 0.f;
+            for (int q = 0; q < kW; ++q)
+                t += wr[q];
+            rsum_part[blockIdx.x] = t;
+        }
+    }
+}
+
+// Occurrence k of the id with number u to position segoff[u] + arr[k].
+template <typename IdT>
+__global__ void __launch_bounds__(kSpThreads)
+k_sp_place(const IdT *__restrict__ ids, int64_t N, const int32_t *__restrict__ slot,
+           const int32_t *__restrict__ segoff, const int32_t *__restrict__ arr, int32_t *__restrict__ placed,
+           int32_t *__restrict__ segidx, int32_t *__restrict__ single)
+{
+    const int64_t k = (int64_t)blockIdx.x * kSpThreads + threadIdx.x;
+    grid_dep_wait();  // runs and arrival numbers
+    grid_dep_launch();
+    if (k >= N)
+        return;
+    const int a = arr[k];
+    if (a < 0)
+        return;
+    const int u = slot[ids[k]] - 1;
+    const int s = segoff[u];
+    const bool once = segoff[u + 1] == s + 1;
+    placed[s + a] = (int)k;
+    segidx[s + a] = u;
+    if (a == 0)  // an id seen once: its summed row is that occurrence's row
+        single[u] = once ? (int)k : -1;
 }
 
 // Workers split the sorted occurrences into contiguous ranges of equal
@@ -355,35 +326,118 @@ __device__ __forceinline__ int64_t cost_target(int w, int nw, int64_t C)
     return ((int64_t)w * C) / nw;
 }
 
-// Smallest p in [0, n_valid] with p + segidx[p] >= T (position n_valid
-// counts as reaching every target).  Block-wide 256-way search: each round
-// probes kThreads evenly spaced positions and keeps the one interval that
-// holds the answer.
-__device__ int block_first_reaching(const int32_t *__restrict__ segidx, int n_valid, int64_t T)
+// Each run's occurrences in increasing order, and the workers' bounds.
+// A run of up to kLongRun occurrences: the thread of each position counts the
+// smaller ones in its run (a warp's positions mostly share a run, so the
+// loads broadcast).  A longer run, by a whole CTA: the occurrences of a
+// window of kWinBits are bits of a bitmap in shared memory, read back in
+// order; the first `nbig` CTAs take the (long run, window) pairs.  A long
+// run is bound by its trips to L2, so a thread has 16 occurrences in flight.
+constexpr int kWinWords = 2048;
+constexpr int kWinBits = 32 * kWinWords;
+__global__ void __launch_bounds__(kOrderThreads)
+k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segidx,
+           const int32_t *__restrict__ segoff, const int32_t *__restrict__ longrun,
+           const int32_t *__restrict__ nlong, const DevScalars *__restrict__ sc, int64_t N, int nbig,
+           int32_t *__restrict__ perm, int32_t *__restrict__ bounds, int nw)
 {
-    __shared__ int lo_hi[2];
-    int lo = 0, hi = n_valid;  // answer in [lo, hi]
-    while (lo < hi) {
-        const int64_t len = hi - lo;
-        const int t = threadIdx.x;
-        const int p = lo + (int)((len * t) / kThreads);
-        const bool reached = (int64_t)p + segidx[p] >= T;  // p < hi <= n_valid
-        const int below = __syncthreads_count(!reached);  // probes before the answer
-        if (t == 0) {
-            int nlo = lo, nhi = hi;
-            if (below > 0)
-                nlo = lo + (int)((len * (below - 1)) / kThreads) + 1;
-            if (below < kThreads)
-                nhi = lo + (int)((len * below) / kThreads);
-            lo_hi[0] = nlo;
-            lo_hi[1] = nhi;
+    constexpr int kW = kOrderThreads / 32;
+    constexpr int kPer = 16;
+    __shared__ unsigned bits[kWinWords];
+    __shared__ int wsum[2][kW];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    grid_dep_wait();  // placed occurrences
+    grid_dep_launch();
+    if ((int)blockIdx.x >= nbig) {
+        const int n_valid = sc->n_valid, U = sc->n_unique;
+        const int64_t p = (int64_t)((int)blockIdx.x - nbig) * kOrderThreads + tid;
+        if (p >= n_valid)
+            return;
+        const int u = segidx[p];
+        const int before = p > 0 ? segidx[p - 1] : 0;
+        const int x = placed[p];
+        const int s = segoff[u], e = segoff[u + 1];
+        if (e - s <= kLongRun) {
+            int below = 0;
+#pragma unroll 8
+            for (int q = s; q < e; ++q)
+                below += placed[q] < x;
+            perm[s + below] = x;
+        }
+        // the workers whose target lies above the position before this one
+        // and not above this one start here (and those above the last
+        // position at the end)
+        const int64_t C = (int64_t)n_valid + U;
+        const int64_t c1 = p + u;
+        const int64_t c0 = p > 0 ? p - 1 + before : -1;
+        for (int64_t q = ((c0 + 1) * nw + C - 1) / C; q < nw; ++q) {
+            const bool here = cost_target((int)q, nw, C) <= c1;
+            if (!here && p + 1 < n_valid)
+                break;
+            bounds[q] = here ? (int)p : n_valid;
+        }
+        if (p + 1 == n_valid)
+            bounds[nw] = n_valid;
+        return;
+    }
+    const int nwin = (int)((N + kWinBits - 1) / kWinBits);
+    const int64_t items = (int64_t)*nlong * nwin;
+    for (int64_t it = blockIdx.x; it < items; it += nbig) {
+        const int u = longrun[it / nwin];
+        const int64_t k0 = (it % nwin) * kWinBits;
+        const int words = (int)((N - k0 < kWinBits ? N - k0 : kWinBits) + 31) / 32;
+        const int s = segoff[u], e = segoff[u + 1];
+        for (int q = tid; q < words; q += kOrderThreads)
+            bits[q] = 0u;
+        __syncthreads();
+        int below = 0;  // occurrences before the window
+        for (int q0 = s + tid; q0 < e; q0 += kPer * kOrderThreads) {
+            int x[kPer];
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const int q = q0 + k * kOrderThreads;
+                x[k] = q < e ? placed[q] : -1;
+            }
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const int64_t b = x[k] - k0;
+                if (b >= 0 && b < kWinBits)
+                    atomicOr(&bits[b >> 5], 1u << (b & 31));
+                below += x[k] >= 0 && b < 0;
+            }
         }
         __syncthreads();
-        lo = lo_hi[0];
-        hi = lo_hi[1];
+        // warp w owns words [w0, w1), 32 of them at a time; the rank of its
+        // first bit is the number of bits in the words before them
+        const int per = ((words + kW - 1) / kW + 31) / 32 * 32;
+        const int w0 = w * per, w1 = w0 + per < words ? w0 + per : words;
+        int mine = 0;
+        for (int q = w0 + lane; q < w1; q += 32)
+            mine += __popc(bits[q]);
+        mine = __reduce_add_sync(0xffffffffu, mine);
+        below = __reduce_add_sync(0xffffffffu, below);
+        if (lane == 0) {
+            wsum[0][w] = mine;
+            wsum[1][w] = below;
+        }
         __syncthreads();
+        int at = s;
+#pragma unroll
+        for (int q = 0; q < kW; ++q)
+            at += wsum[1][q] + (q < w ? wsum[0][q] : 0);
+        for (int q = w0; q < w1; q += 32) {
+            unsigned m = q + lane < w1 ? bits[q + lane] : 0u;
+            const int n = __popc(m);
+            const int x = warp_scan(n, lane);
+            int o = at + x - n;
+            while (m) {
+                perm[o++] = (int)(k0 + (int64_t)(q + lane) * 32 + __ffs(m) - 1);
+                m &= m - 1;
+            }
+            at += __shfl_sync(0xffffffffu, x, 31);
+        }
+        __syncthreads();  // the bitmap is cleared for the next pair
     }
-    return lo;
 }
 
 // Worker whose range holds sorted position p of run u.
@@ -410,9 +464,8 @@ __global__ void __launch_bounds__(kThreads, kSparseCtasPerSm)
 k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
             const int32_t *__restrict__ segidx, const DevScalars *__restrict__ sc,
             float *__restrict__ S, float *__restrict__ rowpart, float *__restrict__ carry,
-            float *__restrict__ colpart, int32_t *__restrict__ bounds, int D, int NS,
-            float *__restrict__ r, const int32_t *__restrict__ slot, int64_t V, EmaPair ema,
-            float *__restrict__ rsum_part)
+            float *__restrict__ colpart, const int32_t *__restrict__ bounds, int D, int NS,
+            int32_t *__restrict__ counters, int ncounters)
 {
     using F = typename Vec<VEC>::F;
     constexpr int R = 8;  // rows in flight per thread
@@ -447,14 +500,8 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
     const bool worker = w < nw && n_valid > 0;
     int p0 = 0, p1 = 0;
     if (worker) {
-        const int64_t C = (int64_t)n_valid + sc->n_unique;
-        p0 = block_first_reaching(segidx, n_valid, cost_target(w, nw, C));
-        p1 = (w + 1 == nw) ? n_valid : block_first_reaching(segidx, n_valid, cost_target(w + 1, nw, C));
-        if (sigma == 0 && threadIdx.x == 0) {
-            bounds[w] = p0;
-            if (w + 1 == nw)
-                bounds[nw] = n_valid;
-        }
+        p0 = bounds[w];
+        p1 = bounds[w + 1];
         if (p0 == p1 && active) {
             // an empty range holds no piece of the run that spans it
             const F z = zero_vec<VEC>();
@@ -582,45 +629,10 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
         for (int e = 0; e < VEC; ++e)
             out[col * VEC + e] = colacc[e];
 
-    // The rows outside the batch: r_i <- beta2 r_i (their g is 0), this CTA's
-    // share of the table, kRowBatch rows per thread at a time with their map
-    // entries loaded together; the touched rows are left to the state pass.
-    // The CTA's fp32 sum of the decayed r goes to rsum_part[blockIdx.x].
-    {
-        const int64_t i0 = (int64_t)blockIdx.x * V / gridDim.x, i1 = (int64_t)(blockIdx.x + 1) * V / gridDim.x;
-        float rsum = 0.f;
-        for (int64_t ib = i0 + threadIdx.x; ib < i1; ib += (int64_t)kThreads * kRowBatch) {
-            int sl[kRowBatch];
-            float rr[kRowBatch];
-#pragma unroll
-            for (int k = 0; k < kRowBatch; ++k) {
-                const int64_t i = ib + (int64_t)k * kThreads;
-                sl[k] = (i < i1) ? slot[i] : 1;
-                rr[k] = (i < i1) ? r[i] : 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < kRowBatch; ++k) {
-                if (sl[k] != 0)
-                    continue;
-                const float rn = ema_pair(ema, rr[k], 0.f);
-                r[ib + (int64_t)k * kThreads] = rn;
-                rsum += rn;
-            }
-        }
-        __shared__ float rsh[kThreads / 32];
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1)
-            rsum += __shfl_xor_sync(0xffffffffu, rsum, o);
-        if (lane == 0)
-            rsh[warp] = rsum;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float t = 0.f;
-            for (int q = 0; q < kThreads / 32; ++q)
-                t += rsh[q];
-            rsum_part[blockIdx.x] = t;
-        }
-    }
+    // the dedup's range counts and list length start the next step at zero
+    if (blockIdx.x == 0)
+        for (int q = threadIdx.x; q < ncounters; q += kThreads)
+            counters[q] = 0;
 }
 
 // Runs cut by worker boundaries.  CTA b handles boundary bd = b / NS + 1
@@ -837,56 +849,79 @@ struct Tracer {
     }
 };
 
-// Sort the ids and number their runs (or record zero runs when N == 0).
-void launch_sort_dedup(const SparseArgs &a, Tracer &tr)
+// Ids per range of k_sp_count and k_sp_scan, and the number of ranges: a
+// function of V alone.
+int64_t scan_len(int64_t V)
+{
+    int64_t len = (V + kScanCtas - 1) / kScanCtas;
+    if (len < kScanMin)
+        len = kScanMin;
+    return (len + 3) / 4 * 4;
+}
+int scan_ranges(int64_t V) { return (int)((V + scan_len(V) - 1) / scan_len(V)); }
+
+// Count the ids and number the distinct ones; with r also decay the rows
+// outside the batch (their sums to rsum_part[0 .. scan_ranges)).
+template <typename IdT>
+void launch_count_scan(const SparseArgs &a, Tracer &tr, float *r, const EmaPair &ema, float *rsum_part)
 {
     unsigned char *ws = a.ws;
     const Layout &L = a.lay;
     DevScalars *sc = reinterpret_cast<DevScalars *>(ws + L.scalars);
-    auto *keys = reinterpret_cast<uint64_t *>(ws + L.sp_keys);
-    auto *rank = reinterpret_cast<int32_t *>(ws + L.sp_rank);
-    auto *sorted = reinterpret_cast<uint64_t *>(ws + L.sp_sorted);
-    auto *tilecnt = reinterpret_cast<int32_t *>(ws + L.sp_tilecnt);
-    auto *perm = reinterpret_cast<int32_t *>(ws + L.sp_perm);
-    auto *segidx = reinterpret_cast<int32_t *>(ws + L.sp_segidx);
-    auto *uniq = reinterpret_cast<int32_t *>(ws + L.sp_uniq);
-    auto *segoff = reinterpret_cast<int32_t *>(ws + L.sp_segoff);
     auto *slot = reinterpret_cast<int32_t *>(ws + L.sp_slot);
-    auto *single = reinterpret_cast<int32_t *>(ws + L.sp_single);
-    if (a.N > 0) {
-        const int T = (int)((a.N + kSortTile - 1) / kSortTile);
-        const int64_t npad = (int64_t)T * kSortTile;
-        if (a.ids64)
-            launch_k(k_sp_tile_sort<int64_t>, dim3(T), dim3(kSortThreads), 0, a.stream, tr.pdl(),
-                     static_cast<const int64_t *>(a.ids), a.N, a.V, keys, rank, tilecnt, sc);
-        else
-            launch_k(k_sp_tile_sort<int32_t>, dim3(T), dim3(kSortThreads), 0, a.stream, tr.pdl(),
-                     static_cast<const int32_t *>(a.ids), a.N, a.V, keys, rank, tilecnt, sc);
+    auto *rng = reinterpret_cast<int32_t *>(ws + L.sp_rng);
+    const int64_t len = scan_len(a.V);
+    const int nr = scan_ranges(a.V);
+    const int nb = (int)((a.N + kCountKeys - 1) / kCountKeys);
+    if (nb > 0) {
+        launch_k(k_sp_count<IdT>, dim3(nb), dim3(kSpThreads), 0, a.stream, tr.pdl(),
+                 static_cast<const IdT *>(a.ids), a.N, a.V, slot, reinterpret_cast<int32_t *>(ws + L.sp_arr), rng,
+                 (unsigned)len, nr, sc);
         tr.mark();
-        if (T > 1) {
-            launch_k(k_sp_rank, dim3(T, T), dim3(kSortThreads), 0, a.stream, tr.pdl(), keys, rank);
-            tr.mark();
-        }
-        const int nsc = (int)((npad + kThreads - 1) / kThreads);
-        launch_k(k_sp_scatter, dim3(nsc), dim3(kThreads), 0, a.stream, tr.pdl(), keys, rank, npad, a.V, sorted,
-                 tilecnt);
-        tr.mark();
-        launch_k(k_sp_segments, dim3(T), dim3(kSortThreads), 0, a.stream, tr.pdl(), sorted, a.N, a.V,
-                 tilecnt, uniq, segoff, perm, segidx, slot, single, sc);
-        tr.mark();
-    } else {
-        // no ids: zero distinct ids and zero valid occurrences
-        cudaMemsetAsync(&sc->n_unique, 0, 2 * sizeof(int32_t), a.stream);
-        tr.launched = false;  // the next kernel follows the memset in plain stream order
     }
+    launch_k(k_sp_scan, dim3(nr), dim3(kSpThreads), 0, a.stream, tr.pdl(), slot, a.V, len, rng,
+             reinterpret_cast<int32_t *>(ws + L.sp_uniq), reinterpret_cast<int32_t *>(ws + L.sp_segoff),
+             reinterpret_cast<int32_t *>(ws + L.sp_long), rng + kScanCounters - 1, sc, r, ema, rsum_part);
+    tr.mark();
+}
+
+// Every occurrence to its place in (id, occurrence) order; bounds of the nw
+// workers of the segment sums.
+template <typename IdT>
+void launch_place_order(const SparseArgs &a, Tracer &tr, int nw)
+{
+    unsigned char *ws = a.ws;
+    const Layout &L = a.lay;
+    DevScalars *sc = reinterpret_cast<DevScalars *>(ws + L.scalars);
+    auto *segidx = reinterpret_cast<int32_t *>(ws + L.sp_segidx);
+    auto *segoff = reinterpret_cast<int32_t *>(ws + L.sp_segoff);
+    auto *placed = reinterpret_cast<int32_t *>(ws + L.sp_placed);
+    const int nb = (int)((a.N + kSpThreads - 1) / kSpThreads);
+    if (nb == 0)
+        return;  // no occurrence: the segment sums and the carry see n_valid = 0
+    launch_k(k_sp_place<IdT>, dim3(nb), dim3(kSpThreads), 0, a.stream, tr.pdl(), static_cast<const IdT *>(a.ids), a.N,
+             reinterpret_cast<int32_t *>(ws + L.sp_slot), segoff, reinterpret_cast<int32_t *>(ws + L.sp_arr), placed,
+             segidx, reinterpret_cast<int32_t *>(ws + L.sp_single));
+    tr.mark();
+    const int64_t nbig64 = a.N / (kLongRun + 1) * ((a.N + kWinBits - 1) / kWinBits);
+    const int nbig = (int)(nbig64 < kGridCtas ? nbig64 : kGridCtas);
+    launch_k(k_sp_order, dim3(nbig + (int)((a.N + kOrderThreads - 1) / kOrderThreads)), dim3(kOrderThreads), 0, a.stream, tr.pdl(), placed, segidx, segoff,
+             reinterpret_cast<int32_t *>(ws + L.sp_long),
+             reinterpret_cast<int32_t *>(ws + L.sp_rng) + kScanCounters - 1, sc, a.N, nbig,
+             reinterpret_cast<int32_t *>(ws + L.sp_perm), reinterpret_cast<int32_t *>(ws + L.sp_bounds), nw);
+    tr.mark();
 }
 
 // Distinct ids, their counts and U to caller buffers.
 __global__ void k_sp_export(const int32_t *__restrict__ uniq, const int32_t *__restrict__ segoff,
                             const DevScalars *__restrict__ sc, int64_t N, int32_t *__restrict__ uniq_out,
-                            int32_t *__restrict__ counts_out, int32_t *__restrict__ n_unique_out)
+                            int32_t *__restrict__ counts_out, int32_t *__restrict__ n_unique_out,
+                            int32_t *__restrict__ counters, int ncounters)
 {
     grid_dep_wait();
+    if (blockIdx.x == 0)
+        for (int q = threadIdx.x; q < ncounters; q += blockDim.x)
+            counters[q] = 0;
     const int U = sc->n_unique;
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < N;
          u += (int64_t)gridDim.x * blockDim.x) {
@@ -925,23 +960,30 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     Tracer tr{a.trace, a.n_trace, 0, a.stream};
 
     tr.mark();
-    launch_sort_dedup(a, tr);
     const int G = kSparseCtas;
     const int nw = G / NS;
     const StepConsts kc = make_consts(a.beta2, a.one_minus_beta2, a.V, a.D, a.inv_bc);
+    if (a.ids64) {
+        launch_count_scan<int64_t>(a, tr, a.r, kc.ema, rsum_part);
+        launch_place_order<int64_t>(a, tr, nw);
+    } else {
+        launch_count_scan<int32_t>(a, tr, a.r, kc.ema, rsum_part);
+        launch_place_order<int32_t>(a, tr, nw);
+    }
     launch_k(k_sp_segsum<VEC>, dim3(G), dim3(kThreads), 0, a.stream, tr.pdl(), a.rows, perm, segidx, sc, S,
-             rowpart, carry, colpart, bounds, D, NS, a.r, slot, a.V, kc.ema, rsum_part);
+             rowpart, carry, colpart, bounds, D, NS, reinterpret_cast<int32_t *>(ws + L.sp_rng), kScanCounters);
     tr.mark();
     launch_k(k_sp_carry<VEC>, dim3(G), dim3(kThreads), 0, a.stream, tr.pdl(), segidx, segoff, bounds, sc,
              carry, S, rowpart, colpart, D, NS, nw);
     tr.mark();
     // the touched rows' r and the column pass in one launch; the per-CTA
-    // sums of r follow the segment-sum CTAs' sums of the decayed rows
+    // sums of r follow the scan CTAs' sums of the decayed rows
+    const int nr = scan_ranges(a.V);
     const int64_t ub = (a.N + kStateThreads - 1) / kStateThreads;
-    const int GU = (int)(ub < kRsumParts - G ? ub : kRsumParts - G);
+    const int GU = (int)(ub < kRsumParts - nr ? ub : kRsumParts - nr);
     // (segment-sum CTA b writes only the columns of its slice b % NS)
-    launch_state(colpart, G, rsum_part, G + GU, a.c, csum_part, sc, a.V, D, kc, a.stream, tr.pdl(), a.r, slot, rowpart,
-                 NS, GU, uniq, G, NS, kThreads * VEC);
+    launch_state(colpart, G, rsum_part, nr + GU, a.c, csum_part, sc, a.V, D, kc, a.stream, tr.pdl(), a.r, slot,
+                 rowpart, NS, GU, uniq, nr, NS, kThreads * VEC);
     tr.mark();
     // one launch per column panel (one unless D is wider than a CTA's row)
     const int np = a.map.npanels, pw = a.map.pw;
@@ -991,7 +1033,10 @@ cudaError_t launch_sparse_unique(const SparseArgs &a, int32_t *uniq_out, int32_t
                                  int32_t *n_unique_out)
 {
     Tracer tr{nullptr, 0, 0, a.stream};
-    launch_sort_dedup(a, tr);
+    if (a.ids64)
+        launch_count_scan<int64_t>(a, tr, nullptr, EmaPair{}, nullptr);
+    else
+        launch_count_scan<int32_t>(a, tr, nullptr, EmaPair{}, nullptr);
     const DevScalars *sc = reinterpret_cast<const DevScalars *>(a.ws + a.lay.scalars);
     const int32_t *uniq = reinterpret_cast<const int32_t *>(a.ws + a.lay.sp_uniq);
     const int32_t *segoff = reinterpret_cast<const int32_t *>(a.ws + a.lay.sp_segoff);
@@ -1001,7 +1046,7 @@ cudaError_t launch_sparse_unique(const SparseArgs &a, int32_t *uniq_out, int32_t
     if (nb > 4 * kGridCtas)
         nb = 4 * kGridCtas;
     launch_k(k_sp_export, dim3((int)nb), dim3(kThreads), 0, a.stream, tr.pdl(), uniq, segoff, sc, a.N,
-             uniq_out, counts_out, n_unique_out);
+             uniq_out, counts_out, n_unique_out, reinterpret_cast<int32_t *>(a.ws + a.lay.sp_rng), kScanCounters);
     // the touched-row map must be all-zero again before the next step
     int32_t *slot = reinterpret_cast<int32_t *>(a.ws + a.lay.sp_slot);
     cudaMemsetAsync(slot, 0, sizeof(int32_t) * (size_t)a.V, a.stream);

@@ -1,0 +1,55 @@
+"""Edges of the sparse step's counting dedup: runs as long as a thread orders
+(128) and longer, occurrences on both sides of a bitmap window (65536), and
+tables that fill one id range, its neighbours and more than one scan tile."""
+import pytest
+import torch
+
+from paper_2607_01455_gb300.ember import Ember
+from parity import Opt
+from test_sparse_gpu import check_dedup, gated_sparse_step
+
+pytestmark = pytest.mark.gpu
+
+
+def ids_of(V, counts, N, device, seed):
+    """N shuffled ids: counts[i] times id i * (V - 1) / len, the rest uniform."""
+    g = torch.Generator(device=device).manual_seed(seed)
+    k = len(counts)
+    parts = [torch.full((c,), i * (V - 1) // max(1, k - 1), device=device, dtype=torch.int64)
+             for i, c in enumerate(counts)]
+    ids = torch.cat(parts + [torch.randint(0, V, (N - sum(counts),), generator=g, device=device)])
+    return ids[torch.randperm(N, generator=g, device=device)]
+
+
+@pytest.mark.parametrize("V,N,counts", [
+    (300, 1100, (127, 128, 129)), (256, 129, (129,)), (257, 600, (300, 130)), (77824, 3000, (130, 1, 2)),
+    (77825, 5000, (1000, 1000, 1000)), (400000, 2000, (129, 500)),
+    (1000, 65536, (65536,)), (1000, 65537, (65537,)), (50000, 270000, (140000, 300, 90000)),
+])
+@pytest.mark.parametrize("idtype", [torch.int64, torch.int32])
+def test_dedup_edges(cuda_device, V, N, counts, idtype):
+    D = 8
+    emb = Ember(V, D, wdtype="bf16", max_sparse_N=N, device=cuda_device)
+    ids = ids_of(V, counts, N, cuda_device, V + N).to(idtype)
+    check_dedup(emb, ids)
+    W = torch.zeros(V, D, device=cuda_device, dtype=torch.bfloat16)
+    for t in (1, 2):
+        rows = torch.randn(N, D, device=cuda_device, generator=torch.Generator(device=cuda_device).manual_seed(t)) * 1e-4
+        gated_sparse_step(emb, W, ids, rows, 1e-3, t, Opt())
+
+
+def test_order_within_runs_is_deterministic(cuda_device):
+    """Occurrences arrive in any order; the sums are those of increasing
+    occurrence, so repeated steps give the same bits."""
+    V, D, N = 5000, 64, 200000
+    ids = ids_of(V, (120000, 400, 129, 128), N, cuda_device, 1)
+    rows = torch.randn(N, D, device=cuda_device) * 1e-4
+    outs = []
+    for _ in range(4):
+        emb = Ember(V, D, wdtype="f32", max_sparse_N=N, device=cuda_device)
+        W = torch.zeros(V, D, device=cuda_device)
+        emb.step_sparse(W, ids, rows, 1e-3, 1)
+        outs.append((W, emb.state))
+    for W, st in outs[1:]:
+        assert torch.equal(W.view(torch.int32), outs[0][0].view(torch.int32))
+        assert torch.equal(st.view(torch.int32), outs[0][1].view(torch.int32))
