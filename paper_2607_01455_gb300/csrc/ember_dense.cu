@@ -11,24 +11,16 @@
 //           and the sum of its new r values, written to the workspace.
 //   state   O(D * CTAs) work: per column the exact fixed-point total of the
 //           per-CTA partial sums (ember_device.cuh), the column EMA
-//           c_j <- beta2 c_j + (1-beta2) mean_i g^2; then mean(rhat),
-//           mean(chat) and s = sqrt(mean rhat * mean chat) (the
-//           geometric-mean normaliser).
-//   apply   reads G and W, writes W:
+//           c_j <- beta2 c_j + (1-beta2) mean_i g^2, and the sum of the new c
+//           per 32 columns.
+//   apply   every CTA forms s = sqrt(mean rhat * mean chat) (the
+//           geometric-mean normaliser) from the sums of r and c, then reads
+//           G and W, writes W:
 //           W_ij <- W_ij - lr g_ij / (sqrt(rhat_i) sqrt(chat_j / s) + eps),
 //           the factored preconditioner applied as a row scale times a
 //           column scale, never stored (Section 2.3).
 //
-// By default the three parts run as ONE cooperative launch (k_dense_fused):
-// every CTA reduces its rows, a grid barrier, the CTAs share the column
-// groups, a second grid barrier, then every CTA forms s itself (the same
-// arithmetic in every CTA) and updates its rows.  The barriers replace two
-// kernel boundaries, which is what small and mid-size tables pay for most.
-// The three-kernel form (k_reduce_dense, k_state_dense, k_apply_dense) runs
-// the same device code on the same CTA grid and gives the same bits; it
-// serves the steps that need more than one launch anyway (column panels,
-// the LM-head step, row shards, a gradient in host memory), traced steps,
-// and devices where the cooperative grid does not fit.
+// A small table runs all three parts in one cluster launch (k_dense_cluster).
 //
 // Bandwidth: 4VD bytes (reduce) + 4VD + 2 w VD bytes (apply), w = bytes per
 // weight.  The apply walks each CTA's rows in the reverse order of the
@@ -272,7 +264,7 @@ __device__ __forceinline__ void reduce_rows(const float *__restrict__ G, float *
 template <int VEC, int CPT, int R, bool BF16>
 __device__ __forceinline__ void apply_rows(void *__restrict__ W, const float *__restrict__ G,
                                            const float *__restrict__ r, const float *__restrict__ c,
-                                           float inv_s_full, int64_t V, int D, int ld, int tpr, float inv_bc,
+                                           float inv_s, int64_t V, int D, int ld, int tpr, float inv_bc,
                                            float eps, float lr_signed, int variant, RowSpan span, int cta)
 {
     using F = typename Vec<VEC>::F;
@@ -288,7 +280,6 @@ __device__ __forceinline__ void apply_rows(void *__restrict__ W, const float *__
     const int64_t step = (int64_t)rg * R;
     const int64_t nblocks = (row1 - row0 + step - 1) / step;
 
-    const float inv_s = (variant == EMBER_VARIANT_FULL) ? inv_s_full : 1.f;
     for (int j = tid; j < D; j += kThreads)
         cs[j] = (variant == EMBER_VARIANT_ROW) ? 1.f : sqrtf(__ldcg(c + j) * inv_bc * inv_s);
     __syncthreads();
@@ -358,9 +349,9 @@ struct ColSource {
 
 constexpr int kStateWarps = kStateThreads / 32;
 // partial rows per warp held in registers by the column pass (the dense
-// step's 304 and the sparse step's 456 rows fit; more, as the LM-head step
-// has, take two passes through L2)
-constexpr int kRegParts = 64;
+// step's 304 rows, the sparse step's 456 and those of an LM head of up to
+// 131072 rows fit; more take two passes through L2)
+constexpr int kRegParts = 32;
 static_assert(kRegParts * kStateWarps >= kGridCtas, "the dense step's partial rows fit the register path");
 
 __device__ __forceinline__ void column_group(const ColSource &src, int group, float *__restrict__ c,
@@ -485,88 +476,6 @@ __device__ __forceinline__ void column_group(const ColSource &src, int group, fl
     __syncthreads();  // the shared buffers are reused by the next group
 }
 
-// Exact fixed-point total of n fp32 values load(0) .. load(n-1) (>= 0), by a
-// whole CTA of kStateThreads threads; every thread gets the result.  The
-// loader reads global memory through L2 (the values were written by other
-// CTAs) or another CTA's shared memory in a cluster.
-template <int NT = kStateThreads, typename Load>
-__device__ float block_fx_total(Load load, int n)
-{
-    constexpr int kNW = NT / 32;  // warps
-    __shared__ unsigned ek[kNW];
-    __shared__ unsigned long long ss[kNW];
-    const int lane = threadIdx.x & 31;
-    const int w = threadIdx.x >> 5;
-    // each thread's first value is loaded once and kept for the second pass
-    const float first = ((int)threadIdx.x < n) ? load(threadIdx.x) : 0.f;
-    unsigned e = fx_key(first);
-    for (int b = threadIdx.x + NT; b < n; b += NT)
-        e = max(e, fx_key(load(b)));
-    e = __reduce_max_sync(0xffffffffu, e);
-    if (lane == 0)
-        ek[w] = e;
-    __syncthreads();
-    unsigned E = 0;
-#pragma unroll
-    for (int q = 0; q < kNW; ++q)
-        E = max(E, ek[q]);
-    unsigned long long s = fx_of(first, E);  // 0 for a zero
-    for (int b = threadIdx.x + NT; b < n; b += NT)
-        s += fx_of(load(b), E);
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1)
-        s += shfl_xor_u64(s, o);
-    if (lane == 0)
-        ss[w] = s;
-    __syncthreads();
-    unsigned long long S = 0;
-#pragma unroll
-    for (int q = 0; q < kNW; ++q)
-        S += ss[q];
-    __syncthreads();
-    return fx_value(S, E);
-}
-
-// The normaliser from the total of r (r_total, over the whole table) and the
-// per-group sums of the new c (load(q), q < ngroups), by a whole CTA of NT
-// threads; every thread gets it.  The group sums are added in a fixed order
-// (thread t takes groups t, t + NT, ... in order, then a fixed butterfly,
-// then the warps in order), so every CTA that runs this forms the same bits,
-// and for up to 256 groups CTAs of 256 and 512 threads form the same sums
-// (each thread holds at most one group; the extra warps add zeros).
-struct Norm {
-    float s, rbar, cbar, inv_s;
-};
-template <int NT = kStateThreads, typename Load>
-__device__ Norm normaliser(float r_total, Load load, int ngroups, const StepConsts &kc)
-{
-    constexpr int kNW = NT / 32;  // warps
-    __shared__ float part[kNW];
-    const int lane = threadIdx.x & 31;
-    const int w = threadIdx.x >> 5;
-    float csum = 0.f;
-    for (int q = threadIdx.x; q < ngroups; q += NT)
-        csum += load(q);
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1)
-        csum += __shfl_xor_sync(0xffffffffu, csum, o);
-    if (lane == 0)
-        part[w] = csum;
-    __syncthreads();
-    csum = 0.f;
-    for (int q = 0; q < kNW; ++q)
-        csum += part[q];
-    __syncthreads();
-    Norm n;
-    n.rbar = (r_total * kc.inv_bc) * kc.inv_V;
-    n.cbar = (csum * kc.inv_bc) * kc.inv_D;
-    // the square roots taken apart: their product stays in range where
-    // rbar * cbar would underflow
-    n.s = sqrtf(n.rbar) * sqrtf(n.cbar);
-    n.inv_s = (n.s > 0.f) ? 1.f / n.s : 0.f;
-    return n;
-}
-
 // ---------------------------------------------------------------------------
 // Kernels of the three-launch form.
 // ---------------------------------------------------------------------------
@@ -584,14 +493,11 @@ k_reduce_dense(const float *__restrict__ G, float *__restrict__ r, float *__rest
                                     nullptr);
 }
 
-// Column EMA and normaliser.  The first ngroups CTAs each own one group of
+// Column EMA.  The first ngroups CTAs each own one group of
 // 32 columns (column_group).  For the sparse and LM-head steps and a dense
 // step in column panels the remaining CTAs also do the row pass: r for every
-// row (rows outside a sparse batch see a zero gradient row, touched rows take
-// their sum of g^2 per column slice from `rowpart`) and the sum of the new r
-// per CTA.  The last CTA to finish forms mean(rhat), mean(chat) and s; the
-// sum of r over the table is the exact fixed-point total of the nrsum per-CTA
-// sums, or, in a row-sharded step, comes with the exchanged totals.
+// row (touched rows of a sparse batch only) from the sums of g^2 per column
+// slice in `rowpart`, and the sum of the new r per CTA.
 struct RowPass {
     float *r;               // r[V], updated
     int32_t *slot;          // sparse step: touched-row map, cleared here
@@ -603,15 +509,14 @@ struct RowPass {
 };
 
 __global__ void __launch_bounds__(kStateThreads)
-k_state_dense(ColSource src, float *__restrict__ rsum_part, int nrsum, float *__restrict__ c,
-              float *__restrict__ csum_part, DevScalars *sc, int64_t V, int D, StepConsts kc, RowPass rowp)
+k_state_dense(ColSource src, float *__restrict__ rsum_part, float *__restrict__ c,
+              float *__restrict__ csum_part, const DevScalars *sc, int64_t V, int D, StepConsts kc, RowPass rowp)
 {
     constexpr int kW = kStateWarps;
     const int lane = threadIdx.x & 31;
     const int w = threadIdx.x >> 5;
     const int ngroups = (int)gridDim.x - rowp.nrow_ctas;
     __shared__ float part[kW];
-    __shared__ bool am_last;
     // GB300 runs fp64 at a small fraction of its fp32 rate: everything here
     // is fp32 (the EMAs with float-pair coefficients, sums of at most a few
     // thousand values per CTA in fixed trees, the normaliser) or integer
@@ -670,36 +575,13 @@ k_state_dense(ColSource src, float *__restrict__ rsum_part, int nrsum, float *__
             rsum_part[rowp.rsum_base + rb] = t;
         }
     }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned t = atomicAdd(&sc->ticket, 1u);
-        am_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!am_last)
-        return;
-    __threadfence();
-    // this thread's first group sum of c, loaded together with the sums of r
-    const float c_first = ((int)threadIdx.x < ngroups) ? __ldcg(csum_part + threadIdx.x) : 0.f;
-    const float r_total = (src.sums != nullptr)
-                              ? fx_value(src.sums[D], src.scales[D])
-                              : block_fx_total([&](int b) { return __ldcg(rsum_part + b); }, nrsum);
-    const Norm n = normaliser(
-        r_total, [&](int q) { return q == (int)threadIdx.x ? c_first : __ldcg(csum_part + q); }, ngroups, kc);
-    if (threadIdx.x == 0) {
-        sc->s = n.s;
-        sc->rbar = n.rbar;
-        sc->cbar = n.cbar;
-        sc->inv_s = n.inv_s;
-        sc->ticket = 0u;
-    }
 }
 
 template <int VEC, int CPT, int R, bool BF16>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__restrict__ r,
-              const float *__restrict__ c, const DevScalars *__restrict__ sc, int64_t V, int D, int ld, int tpr,
-              float inv_bc, float eps, float lr_signed, int variant, RowSpan span)
+              const float *__restrict__ c, NormSource norm, int64_t V, int D, int ld, int tpr, StepConsts kc,
+              float eps, float lr_signed, int variant, RowSpan span)
 {
     // While the state pass finishes: pull this thread's first rows of G and
     // W (the last iteration block, walked first) towards L2.
@@ -728,10 +610,11 @@ k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__
             }
         }
     }
-    grid_dep_wait();  // c, s (state pass) and r (reduce pass)
+    grid_dep_wait();  // c and its sums (state pass), r and its sums (reduce pass)
     grid_dep_launch();
-    apply_rows<VEC, CPT, R, BF16>(W, G, r, c, __ldcg(&sc->inv_s), V, D, ld, tpr, inv_bc, eps, lr_signed, variant,
-                                  span, blockIdx.x);
+    const float inv_s = variant == EMBER_VARIANT_FULL ? step_inv_s<kThreads>(norm, kc) : 1.f;
+    apply_rows<VEC, CPT, R, BF16>(W, G, r, c, inv_s, V, D, ld, tpr, kc.inv_bc, eps, lr_signed, variant, span,
+                                  blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -773,7 +656,6 @@ struct SmallArgs {
     void *W;
     const float *G;
     float *r, *c;
-    DevScalars *sc;
     int64_t V;
     int D, tpr, nits;
     StepConsts kc;
@@ -922,21 +804,14 @@ k_dense_cluster(SmallArgs a)
     }
     const float r_total = block_fx_total<kThreads>([&](int b) { return ld_dsmem(&rsum_own, b); }, (int)nb);
     cluster_arrive();  // done reading the other CTAs' shared memory
-    const Norm n = normaliser<kThreads>(r_total, [&](int q) { return csum_sh[q]; }, ngroups, a.kc);
-    if (cta == 0) {
+    const float norm = normaliser<kThreads>(r_total, [&](int q) { return csum_sh[q]; }, ngroups, a.kc);
+    if (cta == 0)
         for (int j = tid; j < D; j += kThreads)
             a.c[j] = cnew[j];
-        if (tid == 0) {
-            a.sc->s = n.s;
-            a.sc->rbar = n.rbar;
-            a.sc->cbar = n.cbar;
-            a.sc->inv_s = n.inv_s;
-        }
-    }
 
     // the update, as apply_rows forms it, from the kept G and W
     const float inv_bc = a.kc.inv_bc;
-    const float inv_s = (a.variant == EMBER_VARIANT_FULL) ? n.inv_s : 1.f;
+    const float inv_s = (a.variant == EMBER_VARIANT_FULL) ? norm : 1.f;
     float *cs = cnew;  // the column scales replace the new c (already written out)
     __syncthreads();
     for (int j = tid; j < D; j += kThreads)
@@ -1277,18 +1152,19 @@ cudaError_t launch_dense_t(const DenseArgs &a)
         }
         const ColSource src{nullptr, 0, sh.sums, sh.scales};
         e = launch_k(k_state_dense, dim3((D + kStateCols - 1) / kStateCols), dim3(kStateThreads), 0, a.stream,
-                     false, src, rsum_part, 0, a.c, csum_part, sc, a.V, D, kc,
+                     false, src, rsum_part, a.c, csum_part, sc, a.V, D, kc,
                      RowPass{nullptr, nullptr, nullptr, 0, 0, nullptr, 0});
         if (e != cudaSuccess || ncta == 0)
             return e != cudaSuccess ? e : cudaGetLastError();
+        const NormSource norm{rsum_part, 0, csum_part, (D + kStateCols - 1) / kStateCols, sh.sums, sh.scales, D};
         const size_t cs_bytes = (size_t)D * sizeof(float);
         if (a.wbf16)
             e = launch_k(k_apply_dense<VEC, CPT, R3, true>, dim3(ncta), dim3(kThreads), cs_bytes, a.stream, pdl,
-                         a.W, a.G, a.r, a.c, sc, a.V, D, ld, a.map.tpr, kc.inv_bc, a.eps, a.lr_signed,
+                         a.W, a.G, a.r, a.c, norm, a.V, D, ld, a.map.tpr, kc, a.eps, a.lr_signed,
                          a.variant, span);
         else
             e = launch_k(k_apply_dense<VEC, CPT, R3, false>, dim3(ncta), dim3(kThreads), cs_bytes, a.stream, pdl,
-                         a.W, a.G, a.r, a.c, sc, a.V, D, ld, a.map.tpr, kc.inv_bc, a.eps, a.lr_signed,
+                         a.W, a.G, a.r, a.c, norm, a.V, D, ld, a.map.tpr, kc, a.eps, a.lr_signed,
                          a.variant, span);
         return e != cudaSuccess ? e : cudaGetLastError();
     }
@@ -1319,7 +1195,7 @@ cudaError_t launch_dense_t(const DenseArgs &a)
             return e;
         if (a.trace)
             cudaEventRecord(a.trace[1], a.stream);
-        e = launch_state(colpart, nparts, rsum_part, nparts, a.c, csum_part, sc, a.V, D, kc, a.stream, pdl, nullptr, nullptr, nullptr, 0, 0);
+        e = launch_state(colpart, nparts, rsum_part, a.c, csum_part, sc, a.V, D, kc, a.stream, pdl, nullptr, nullptr, nullptr, 0, 0);
         if (e != cudaSuccess)
             return e;
         if (a.trace) {
@@ -1340,7 +1216,7 @@ cudaError_t launch_dense_t(const DenseArgs &a)
                 e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
             if (e != cudaSuccess)
                 return e;
-            SmallArgs sa{a.W, a.G, a.r, a.c, sc, a.V, D, a.map.tpr, nits, kc, a.eps, a.lr_signed, a.variant};
+            SmallArgs sa{a.W, a.G, a.r, a.c, a.V, D, a.map.tpr, nits, kc, a.eps, a.lr_signed, a.variant};
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(nparts);
             cfg.blockDim = dim3(kThreads);
@@ -1357,6 +1233,7 @@ cudaError_t launch_dense_t(const DenseArgs &a)
             return e != cudaSuccess ? e : cudaGetLastError();
         }
     }
+    int nrsum = nparts;  // per-CTA sums of r that the update adds up
     if (a.lm) {
         // G comes from the LM-head kernel, which also leaves the sums of g^2
         // per 128-row block (columns) and per 256-column block (rows); the
@@ -1374,7 +1251,8 @@ cudaError_t launch_dense_t(const DenseArgs &a)
         // the state grid made the step slower (measured 0.1-0.3 ms)
         const int64_t vb = (a.V + kStateThreads - 1) / kStateThreads;
         const int nrow_ctas = (int)(vb < kMaxRowCtas ? vb : kMaxRowCtas);
-        e = launch_state(lm_col, lmhead_row_blocks(a.V), rsum_part, nrow_ctas, a.c, csum_part, sc, a.V, D,
+        nrsum = nrow_ctas;
+        e = launch_state(lm_col, lmhead_row_blocks(a.V), rsum_part, a.c, csum_part, sc, a.V, D,
                          kc, a.stream, false, a.r, nullptr, lm_row,
                          lmhead_col_blocks(a.D), nrow_ctas);
         if (e != cudaSuccess)
@@ -1403,11 +1281,12 @@ cudaError_t launch_dense_t(const DenseArgs &a)
         if (a.trace)
             cudaEventRecord(a.trace[1], a.stream);
         if (np == 1) {
-            e = launch_state(colpart, nparts, rsum_part, nparts, a.c, csum_part, sc, a.V, D, kc, a.stream, pdl, nullptr, nullptr, nullptr, 0, 0);
+            e = launch_state(colpart, nparts, rsum_part, a.c, csum_part, sc, a.V, D, kc, a.stream, pdl, nullptr, nullptr, nullptr, 0, 0);
         } else {
             const int64_t vb = (a.V + kStateThreads - 1) / kStateThreads;
             const int nrow_ctas = (int)(vb < kMaxRowCtas ? vb : kMaxRowCtas);
-            e = launch_state(colpart, nparts, rsum_part, nrow_ctas, a.c, csum_part, sc, a.V, D, kc, a.stream, pdl, a.r, nullptr, rowpart, np, nrow_ctas);
+            nrsum = nrow_ctas;
+            e = launch_state(colpart, nparts, rsum_part, a.c, csum_part, sc, a.V, D, kc, a.stream, pdl, a.r, nullptr, rowpart, np, nrow_ctas);
         }
         if (e != cudaSuccess)
             return e;
@@ -1418,17 +1297,18 @@ cudaError_t launch_dense_t(const DenseArgs &a)
     if (a.trace)
         cudaEventRecord(a.trace[2], a.stream);
     const size_t cs_bytes = (size_t)pw * sizeof(float);
+    const NormSource norm{rsum_part, nrsum, csum_part, (D + kStateCols - 1) / kStateCols, nullptr, nullptr, D};
     for (int q = np - 1; q >= 0; --q) {
         const int64_t c0 = (int64_t)q * pw;
         void *Wq = static_cast<unsigned char *>(a.W) + c0 * (a.wbf16 ? 2 : 4);
         if (a.wbf16)
             e = launch_k(k_apply_dense<VEC, CPT, R3, true>, dim3(nparts), dim3(kThreads), cs_bytes,
-                         a.stream, pdl, Wq, Gd + c0, a.r, a.c + c0, sc, a.V, cols(q), ld, a.map.tpr,
-                         kc.inv_bc, a.eps, a.lr_signed, a.variant, span);
+                         a.stream, pdl, Wq, Gd + c0, a.r, a.c + c0, norm, a.V, cols(q), ld, a.map.tpr,
+                         kc, a.eps, a.lr_signed, a.variant, span);
         else
             e = launch_k(k_apply_dense<VEC, CPT, R3, false>, dim3(nparts), dim3(kThreads), cs_bytes,
-                         a.stream, pdl, Wq, Gd + c0, a.r, a.c + c0, sc, a.V, cols(q), ld, a.map.tpr,
-                         kc.inv_bc, a.eps, a.lr_signed, a.variant, span);
+                         a.stream, pdl, Wq, Gd + c0, a.r, a.c + c0, norm, a.V, cols(q), ld, a.map.tpr,
+                         kc, a.eps, a.lr_signed, a.variant, span);
         if (e != cudaSuccess)
             return e;
     }
@@ -1439,8 +1319,8 @@ cudaError_t launch_dense_t(const DenseArgs &a)
 
 }  // namespace
 
-cudaError_t launch_state(const float *colpart, int nparts, float *rsum_part, int nrsum, float *c,
-                         float *csum_part, DevScalars *sc, int64_t V, int D, const StepConsts &kc,
+cudaError_t launch_state(const float *colpart, int nparts, float *rsum_part, float *c,
+                         float *csum_part, const DevScalars *sc, int64_t V, int D, const StepConsts &kc,
                          cudaStream_t stream, bool pdl, float *r_rows, int32_t *slot, const float *rowpart,
                          int nslices, int nrow_ctas, const int32_t *uniq, int rsum_base, int pstride, int pcols)
 {
@@ -1448,7 +1328,7 @@ cudaError_t launch_state(const float *colpart, int nparts, float *rsum_part, int
     RowPass rp{r_rows, slot, rowpart, nslices, nrow_ctas, uniq, rsum_base};
     const ColSource src{colpart, nparts, nullptr, nullptr, pstride, pcols};
     return launch_k(k_state_dense, dim3(ngroups + nrow_ctas), dim3(kStateThreads), 0, stream, pdl, src,
-                    rsum_part, nrsum, c, csum_part, sc, V, D, kc, rp);
+                    rsum_part, c, csum_part, sc, V, D, kc, rp);
 }
 
 bool choose_colmap(int64_t D, bool vec4_ok, ColMap *m)

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ember_internal.h"
+
 namespace ember {
 namespace dev {
 
@@ -301,6 +303,101 @@ __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long x,
     const unsigned lo = __shfl_xor_sync(0xffffffffu, (unsigned)x, m);
     const unsigned hi = __shfl_xor_sync(0xffffffffu, (unsigned)(x >> 32), m);
     return ((unsigned long long)hi << 32) | lo;
+}
+
+// Exact fixed-point total of n fp32 values load(0) .. load(n-1) (>= 0), by a
+// whole CTA of NT threads; every thread gets the result.  The
+// loader reads global memory through L2 (the values were written by other
+// CTAs) or another CTA's shared memory in a cluster.
+template <int NT, typename Load>
+__device__ float block_fx_total(Load load, int n)
+{
+    constexpr int kNW = NT / 32;  // warps
+    __shared__ unsigned ek[kNW];
+    __shared__ unsigned long long ss[kNW];
+    const int lane = threadIdx.x & 31;
+    const int w = threadIdx.x >> 5;
+    // each thread's first value is loaded once and kept for the second pass
+    const float first = ((int)threadIdx.x < n) ? load(threadIdx.x) : 0.f;
+    unsigned e = fx_key(first);
+    for (int b = threadIdx.x + NT; b < n; b += NT)
+        e = max(e, fx_key(load(b)));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0)
+        ek[w] = e;
+    __syncthreads();
+    unsigned E = 0;
+#pragma unroll
+    for (int q = 0; q < kNW; ++q)
+        E = max(E, ek[q]);
+    unsigned long long s = fx_of(first, E);  // 0 for a zero
+    for (int b = threadIdx.x + NT; b < n; b += NT)
+        s += fx_of(load(b), E);
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1)
+        s += shfl_xor_u64(s, o);
+    if (lane == 0)
+        ss[w] = s;
+    __syncthreads();
+    unsigned long long S = 0;
+#pragma unroll
+    for (int q = 0; q < kNW; ++q)
+        S += ss[q];
+    __syncthreads();
+    return fx_value(S, E);
+}
+
+// The normaliser from the total of r (r_total, over the whole table) and the
+// per-group sums of the new c (load(q), q < ngroups), by a whole CTA of NT
+// threads; every thread gets it.  The group sums are added in a fixed order
+// (thread t takes groups t, t + NT, ... in order, then a fixed butterfly,
+// then the warps in order), so every CTA of NT threads forms the same bits.
+// Returns 1 / s, or 0 when s is 0.
+template <int NT, typename Load>
+__device__ float normaliser(float r_total, Load load, int ngroups, const StepConsts &kc)
+{
+    constexpr int kNW = NT / 32;  // warps
+    __shared__ float part[kNW];
+    const int lane = threadIdx.x & 31;
+    const int w = threadIdx.x >> 5;
+    float csum = 0.f;
+    for (int q = threadIdx.x; q < ngroups; q += NT)
+        csum += load(q);
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1)
+        csum += __shfl_xor_sync(0xffffffffu, csum, o);
+    if (lane == 0)
+        part[w] = csum;
+    __syncthreads();
+    csum = 0.f;
+    for (int q = 0; q < kNW; ++q)
+        csum += part[q];
+    __syncthreads();
+    const float rbar = (r_total * kc.inv_bc) * kc.inv_V;
+    const float cbar = (csum * kc.inv_bc) * kc.inv_D;
+    // the square roots taken apart: their product stays in range where
+    // rbar * cbar would underflow
+    const float s = sqrtf(rbar) * sqrtf(cbar);
+    return (s > 0.f) ? 1.f / s : 0.f;
+}
+
+// 1 / s of a step by a CTA of the update: the sum of r over the table is the
+// exact fixed-point total of the nrsum per-CTA sums, or, in a row-sharded
+// step, comes with the exchanged totals.  Every CTA of the update forms it
+// itself: one trip to L2 for all the values, against the 4 us that a last
+// CTA of the state pass took to learn that the others were done (a ticket),
+// form it and hand it over through a kernel boundary.
+template <int NT>
+__device__ float step_inv_s(const NormSource &n, const StepConsts &kc)
+{
+    const int t = threadIdx.x;
+    // this thread's first group sum of c, loaded together with the sums of r
+    const float c_first = (t < n.ngroups) ? __ldcg(n.csum_part + t) : 0.f;
+    const float r_total = (n.sums != nullptr)
+                              ? fx_value(n.sums[n.D], n.scales[n.D])
+                              : block_fx_total<NT>([&](int b) { return __ldcg(n.rsum_part + b); }, n.nrsum);
+    return normaliser<NT>(
+        r_total, [&](int q) { return q == t ? c_first : __ldcg(n.csum_part + q); }, n.ngroups, kc);
 }
 
 }  // namespace dev

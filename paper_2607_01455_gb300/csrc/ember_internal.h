@@ -24,13 +24,13 @@ constexpr int kSparseCtasPerSm = 3;
 constexpr int kSparseCtas = kSms * kSparseCtasPerSm;
 constexpr int kPartRows = kSparseCtas > kGridCtas ? kSparseCtas : kGridCtas;
 
-// The state pass reduces 32 columns per CTA of kStateThreads threads (16
+// The state pass reduces 32 columns per CTA of kStateThreads threads (32
 // warps, so that each warp adds few per-CTA partial rows).  Its row pass runs
 // up to kMaxRowCtas CTAs: about one row per thread for the LM-head step (whose
 // rows each sum ceil(D/256) slices) and for a dense step in column panels
 // (one slice per panel), and one touched row per thread for the sparse step.
 constexpr int kStateCols = 32;
-constexpr int kStateThreads = 512;
+constexpr int kStateThreads = 1024;
 constexpr int kMaxRowCtas = 1024;
 constexpr int kRsumParts = kMaxRowCtas > kGridCtas ? kMaxRowCtas : kGridCtas;
 
@@ -38,14 +38,8 @@ constexpr int kRsumParts = kMaxRowCtas > kGridCtas ? kMaxRowCtas : kGridCtas;
 constexpr unsigned kFlagIdRange = 1u << 0;
 constexpr unsigned kFlagTimeout = 1u << 1;
 
-// Scalars that live in the workspace.  `ticket` counts finished CTAs of the
-// state pass and is returned to zero by the last one.
+// Scalars that live in the workspace.
 struct DevScalars {
-    double s;          // geometric-mean normaliser sqrt(mean rhat * mean chat)
-    double rbar;       // mean over rows of rhat
-    double cbar;       // mean over columns of chat
-    float inv_s;       // 1/s in fp32, 0 when s == 0
-    unsigned ticket;
     unsigned flags;    // sticky device error bits (kFlag*)
     int32_t n_unique;  // sparse step: number of distinct valid ids
     int32_t n_valid;   // sparse step: number of ids inside [0, V)
@@ -260,18 +254,28 @@ inline StepConsts make_consts(double beta2, double one_minus_beta2, int64_t V, i
     return k;
 }
 
-// Column EMA and normaliser; with nrow_ctas > 0 the same launch also runs a
+// What 1/s is formed from, after the state pass (see step_inv_s).
+struct NormSource {
+    const float *rsum_part;          // nrsum per-CTA sums of the new r
+    int nrsum;
+    const float *csum_part;          // ngroups sums of the new c
+    int ngroups;
+    const unsigned long long *sums;  // nullptr, or a row-sharded step's totals ...
+    const unsigned char *scales;     // ... and their scale exponents, the sum of r at index D
+    int D;
+};
+
+// Column EMA; with nrow_ctas > 0 the same launch also runs a
 // row pass: r from per-slice sums of g^2, taken from rowpart[u][nslices] for
 // the touched rows of the sparse step, or, with slot == nullptr, from
 // rowpart[nslices][V] for every row.
 // Column totals are exact fixed-point sums of the nparts partial rows
-// (ember_device.cuh); the normaliser's sum of r likewise over the nrsum
-// per-CTA sums in rsum_part.
+// (ember_device.cuh).
 // For the sparse step (slot set) the row pass covers only the U touched rows
 // uniq[0..U) (the segment-sum kernel decays the others) and writes its
 // per-CTA sums of r from rsum_part[rsum_base] on.
-cudaError_t launch_state(const float *colpart, int nparts, float *rsum_part, int nrsum, float *c,
-                         float *csum_part, DevScalars *sc, int64_t V, int D, const StepConsts &k,
+cudaError_t launch_state(const float *colpart, int nparts, float *rsum_part, float *c,
+                         float *csum_part, const DevScalars *sc, int64_t V, int D, const StepConsts &k,
                          cudaStream_t stream, bool pdl, float *r_rows, int32_t *slot, const float *rowpart,
                          int nslices, int nrow_ctas, const int32_t *uniq = nullptr, int rsum_base = 0,
                          int pstride = 1, int pcols = 0);

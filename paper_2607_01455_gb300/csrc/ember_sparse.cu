@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(kThreads, apply_ctas_per_sm(CPT))
 k_sp_apply(void *__restrict__ W, const float *__restrict__ S, const float *__restrict__ rows,
            const int32_t *__restrict__ uniq, const int32_t *__restrict__ single,
            const float *__restrict__ r, const float *__restrict__ c,
-           const DevScalars *__restrict__ sc, int D, int ld, int tpr, float inv_bc, float eps,
+           const DevScalars *__restrict__ sc, NormSource norm, int D, int ld, int tpr, StepConsts kc, float eps,
            float lr_signed, int variant)
 {
     using F = typename Vec<VEC>::F;
@@ -758,10 +758,11 @@ k_sp_apply(void *__restrict__ W, const float *__restrict__ S, const float *__res
     const int rg = kThreads / tpr;
     const int g = tid / tpr;
     const int l = tid - g * tpr;
-    grid_dep_wait();  // s, c, r and the summed rows
+    grid_dep_wait();  // c, r, their sums and the summed rows
     grid_dep_launch();
     const int U = sc->n_unique;
-    const float inv_s = (variant == EMBER_VARIANT_FULL) ? sc->inv_s : 1.f;
+    const float inv_bc = kc.inv_bc;
+    const float inv_s = (variant == EMBER_VARIANT_FULL) ? step_inv_s<kThreads>(norm, kc) : 1.f;
     for (int j = tid; j < D; j += kThreads)
         cs[j] = (variant == EMBER_VARIANT_ROW) ? 1.f : sqrtf(c[j] * inv_bc * inv_s);
     __syncthreads();
@@ -976,13 +977,15 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     launch_k(k_sp_carry<VEC>, dim3(G), dim3(kThreads), 0, a.stream, tr.pdl(), segidx, segoff, bounds, sc,
              carry, S, rowpart, colpart, D, NS, nw);
     tr.mark();
-    // the touched rows' r and the column pass in one launch; the per-CTA
+    // the touched rows' r and the column pass in one launch (a row per thread
+    // for up to one CTA per SM: more would only wait for a place); the per-CTA
     // sums of r follow the scan CTAs' sums of the decayed rows
     const int nr = scan_ranges(a.V);
     const int64_t ub = (a.N + kStateThreads - 1) / kStateThreads;
-    const int GU = (int)(ub < kRsumParts - nr ? ub : kRsumParts - nr);
+    const int GU = (int)(ub < kSms ? ub : kSms);
+    const NormSource norm{rsum_part, nr + GU, csum_part, (D + kStateCols - 1) / kStateCols, nullptr, nullptr, D};
     // (segment-sum CTA b writes only the columns of its slice b % NS)
-    launch_state(colpart, G, rsum_part, nr + GU, a.c, csum_part, sc, a.V, D, kc, a.stream, tr.pdl(), a.r, slot,
+    launch_state(colpart, G, rsum_part, a.c, csum_part, sc, a.V, D, kc, a.stream, tr.pdl(), a.r, slot,
                  rowpart, NS, GU, uniq, nr, NS, kThreads * VEC);
     tr.mark();
     // one launch per column panel (one unless D is wider than a CTA's row)
@@ -996,11 +999,11 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
         const float *rq = a.rows ? a.rows + c0 : nullptr;
         if (a.wbf16)
             launch_k(k_sp_apply<VEC, CPT, R, true>, dim3(GA), dim3(kThreads), cs_bytes, a.stream, tr.pdl(), Wq,
-                     S + c0, rq, uniq, single, a.r, a.c + c0, sc, dq, (int)a.D, a.map.tpr, (float)a.inv_bc, a.eps,
+                     S + c0, rq, uniq, single, a.r, a.c + c0, sc, norm, dq, (int)a.D, a.map.tpr, kc, a.eps,
                      a.lr_signed, a.variant);
         else
             launch_k(k_sp_apply<VEC, CPT, R, false>, dim3(GA), dim3(kThreads), cs_bytes, a.stream, tr.pdl(), Wq,
-                     S + c0, rq, uniq, single, a.r, a.c + c0, sc, dq, (int)a.D, a.map.tpr, (float)a.inv_bc, a.eps,
+                     S + c0, rq, uniq, single, a.r, a.c + c0, sc, norm, dq, (int)a.D, a.map.tpr, kc, a.eps,
                      a.lr_signed, a.variant);
     }
     tr.mark();
