@@ -131,6 +131,13 @@ __device__ __forceinline__ void reduce_rows(const float *__restrict__ G, float *
             acc[c][e] = 0.f;
     float rsum = 0.f;
 
+    // The update reads G again from the last rows back.  Everything before
+    // the last kKeepBytes of the table (spread over the CTAs) is loaded
+    // evict-first, so that it does not push those out of L2: the 32000 x 4096
+    // fp32 step takes 333 us instead of 341, 151936 x 896 258.5 instead of
+    // 261.4 (100 MB kept: 333.5 and 259.3).
+    const uint64_t pol_pass = policy_evict_first(), pol_keep = policy_evict_normal();
+    const int64_t keep0 = row1 - kKeepBytes / (int64_t)sizeof(float) / ld / span.nparts;
     const int rows_per_it = rg * R;                 // rows of one iteration
     const int its_per_buf = kRowBuf / rows_per_it;  // >= 1: rg * R <= 128
     int64_t buf_base = row0;
@@ -138,6 +145,7 @@ __device__ __forceinline__ void reduce_rows(const float *__restrict__ G, float *
     int it = 0;    // iteration index (the slot of the kept G)
     for (int64_t base = row0; base < row1; base += rows_per_it, ++it) {
         F v[R][CPT];
+        const uint64_t pol = base >= keep0 ? pol_keep : pol_pass;
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const int64_t i = base + (int64_t)g * R + k;
@@ -151,8 +159,8 @@ __device__ __forceinline__ void reduce_rows(const float *__restrict__ G, float *
                     if (in)
                         *reinterpret_cast<F *>(G_stage + idx) = v[k][c];
                 } else {
-                    v[k][c] = in ? load_g<VEC>(G + (i - span.row_base) * ld + (int64_t)col * VEC)
-                                 : zero_vec<VEC>();
+                    const float *src = G + (i - span.row_base) * ld + (int64_t)col * VEC;
+                    v[k][c] = !in ? zero_vec<VEC>() : KEEP ? load_g<VEC>(src) : load_g_hint<VEC>(src, pol);
                 }
                 if constexpr (KEEP)  // this thread's slot of the iteration, read back by the update
                     keep[((it * R + k) * CPT + c) * kThreads + tid] = v[k][c];
@@ -250,79 +258,6 @@ __device__ __forceinline__ void reduce_rows(const float *__restrict__ G, float *
         for (int q = 0; q < kWarps; ++q)
             s += rsum_sh[q];
         *rsum_out = s;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Apply: the update of the CTA's rows, walked from the last iteration block
-// to the first.  The column scales live in shared memory (D floats): cs[j] =
-// sqrt(chat_j / s) (FULL), sqrt(chat_j) (COL) or 1 (ROW).  D columns from row
-// stride ld, as in the reduce: W, G and c point at the first column of the
-// panel.  r and c are read through L2 (they may have been written earlier in
-// the same launch).
-// ---------------------------------------------------------------------------
-template <int VEC, int CPT, int R, bool BF16>
-__device__ __forceinline__ void apply_rows(void *__restrict__ W, const float *__restrict__ G,
-                                           const float *__restrict__ r, const float *__restrict__ c,
-                                           float inv_s, int64_t V, int D, int ld, int tpr, float inv_bc,
-                                           float eps, float lr_signed, int variant, RowSpan span, int cta)
-{
-    using F = typename Vec<VEC>::F;
-    using WT = typename WRaw<BF16, VEC>::T;
-    extern __shared__ float cs[];  // D column scales
-    const int DV = D / VEC;
-    const int tid = threadIdx.x;
-    const int rg = kThreads / tpr;
-    const int g = tid / tpr;
-    const int l = tid - g * tpr;
-    const int64_t row0 = (int64_t)(span.cta_base + cta) * V / span.nparts;
-    const int64_t row1 = (int64_t)(span.cta_base + cta + 1) * V / span.nparts;
-    const int64_t step = (int64_t)rg * R;
-    const int64_t nblocks = (row1 - row0 + step - 1) / step;
-
-    for (int j = tid; j < D; j += kThreads)
-        cs[j] = (variant == EMBER_VARIANT_ROW) ? 1.f : sqrtf(__ldcg(c + j) * inv_bc * inv_s);
-    __syncthreads();
-
-    for (int64_t b = nblocks - 1; b >= 0; --b) {
-        const int64_t base = row0 + b * step;
-        F gv[R][CPT];
-        WT wr[R][CPT];
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int64_t i = base + (int64_t)g * R + k;
-#pragma unroll
-            for (int cc = 0; cc < CPT; ++cc) {
-                const int col = l + cc * tpr;
-                if (i < row1 && col < DV) {
-                    const int64_t idx = (i - span.row_base) * ld + (int64_t)col * VEC;
-                    gv[k][cc] = load_g<VEC>(G + idx);
-                    wr[k][cc] = load_w<BF16, VEC>(W, idx);
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int64_t i = base + (int64_t)g * R + k;
-            if (i >= row1)
-                continue;
-            const float rs = (variant == EMBER_VARIANT_COL) ? 1.f : sqrtf(__ldcg(r + i) * inv_bc);
-#pragma unroll
-            for (int cc = 0; cc < CPT; ++cc) {
-                const int col = l + cc * tpr;
-                if (col >= DV)
-                    continue;
-                float w[VEC];
-                unpack_w(wr[k][cc], w);
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) {
-                    const float den = fmaf(rs, cs[col * VEC + e], eps);
-                    const float u = update_ratio(comp(gv[k][cc], e), den);
-                    w[e] = fmaf(lr_signed, u, w[e]);
-                }
-                store_w<BF16, VEC>(W, (i - span.row_base) * ld + (int64_t)col * VEC, w);
-            }
-        }
     }
 }
 
@@ -577,35 +512,71 @@ k_state_dense(ColSource src, float *__restrict__ rsum_part, float *__restrict__ 
     }
 }
 
-template <int VEC, int CPT, int R, bool BF16>
+// ---------------------------------------------------------------------------
+// Apply: the update of the CTA's rows, walked from the last to the first (the
+// reduce pass read the last ones last, and they are still in L2).  A warp
+// takes units of R row blocks x one column segment of 32 K accesses (or
+// 32 / lpr whole rows of fewer than 32 accesses); the CTA's warps take them
+// in turn.  Bound by HBM: 6.5-7 TB/s on tables far larger than L2.  Letting
+// warps claim units from counters, their own range's or another's, balanced
+// the CTAs' ends (they differ by 15 %) but cost more in claims than it
+// gained: 361 against 339 us on 32000 x 4096 fp32.
+//   The column scales live in shared memory: cs[j] = sqrt(chat_j / s) (FULL),
+// sqrt(chat_j) (COL) or 1 (ROW).  D columns from row stride ld: W, G and c
+// point at the first column of the panel.
+//   RAG: a row does not start on a 16-byte boundary.  The accesses stay
+// aligned: m = (the row's first element) mod 4 elements before the row are
+// skipped, the row's first and last access may be partial (element by
+// element), and four copies of the column scales, each shifted by one m, keep
+// their reads aligned too.  `mis` is the panel's first column mod 4.
+// ---------------------------------------------------------------------------
+template <int VEC, int K, int R, bool BF16, bool RAG>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__restrict__ r,
-              const float *__restrict__ c, NormSource norm, int64_t V, int D, int ld, int tpr, StepConsts kc,
-              float eps, float lr_signed, int variant, RowSpan span)
+              const float *__restrict__ c, NormSource norm, int64_t V, int D, int ld, int lpr, int nseg, int mis,
+              StepConsts kc, float eps, float lr_signed, int variant, RowSpan span)
 {
-    // While the state pass finishes: pull this thread's first rows of G and
-    // W (the last iteration block, walked first) towards L2.
-    {
-        const int rg = kThreads / tpr;
-        const int g = threadIdx.x / tpr;
-        const int l = threadIdx.x - g * tpr;
-        const int DV = D / VEC;
-        const int64_t row0 = (int64_t)(span.cta_base + blockIdx.x) * V / span.nparts;
-        const int64_t row1 = (int64_t)(span.cta_base + blockIdx.x + 1) * V / span.nparts;
-        const int64_t step = (int64_t)rg * R;
-        const int64_t nblocks = (row1 - row0 + step - 1) / step;
-        if (nblocks > 0) {
-            const int64_t base = row0 + (nblocks - 1) * step;
-            for (int k = 0; k < R; ++k) {
-                const int64_t i = base + (int64_t)g * R + k;
-                for (int cc = 0; cc < CPT; ++cc) {
-                    const int col = l + cc * tpr;
-                    if (i < row1 && col < DV) {
-                        const int64_t idx = (i - span.row_base) * ld + (int64_t)col * VEC;
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(G + idx));
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char *>(W) +
-                                                                       idx * (BF16 ? 2 : 4)));
-                    }
+    static_assert(!RAG || VEC == 4, "shifted rows use 16-byte accesses");
+    using F = typename Vec<VEC>::F;
+    using WT = typename WRaw<BF16, VEC>::T;
+    extern __shared__ __align__(16) float cs[];  // D column scales (RAG: four shifted copies)
+    constexpr int kWarps = kThreads / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int l = lane & (lpr - 1);     // position within the row's accesses
+    const int rpa = 32 / lpr;           // rows per warp-wide access
+    const int rows_per_unit = R * rpa;
+    const int DV = RAG ? (D + 6) / 4 : D / VEC;
+    const int csw = (D + 3) / 4 * 4 + 4;  // RAG: floats of one copy of the scales
+    const int64_t row0 = (int64_t)(span.cta_base + blockIdx.x) * V / span.nparts;
+    const int64_t row1 = (int64_t)(span.cta_base + blockIdx.x + 1) * V / span.nparts;
+    const int nunits = (int)((row1 - row0 + rows_per_unit - 1) / rows_per_unit) * nseg;
+    // element offset of access cc of row i from W and G; m: elements of the
+    // access before the row's first (RAG)
+    auto offset = [&](int64_t i, int v, int &m) {
+        const int64_t at = (i - span.row_base) * ld;
+        if constexpr (RAG) {
+            m = (int)((at + mis) & 3);
+            return at - m + 4 * (int64_t)v;
+        } else {
+            m = 0;
+            return at + (int64_t)v * VEC;
+        }
+    };
+    auto whole = [&](int v, int m) { return !RAG || (4 * v >= m && 4 * v - m + 4 <= D); };
+
+    // While the state pass finishes: pull this warp's first unit towards L2.
+    if (warp < nunits) {
+        const int rb = warp / nseg, seg = warp - rb * nseg;
+        const int64_t base = row1 - (int64_t)(rb + 1) * rows_per_unit;
+        for (int k = 0; k < R; ++k) {
+            const int64_t i = base + k * rpa + lane / lpr;
+            for (int cc = 0; cc < K; ++cc) {
+                const int v = (seg * K + cc) * lpr + l;
+                int m;
+                const int64_t o = offset(i, v, m);
+                if (i >= row0 && v < DV && whole(v, m)) {
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(G + o));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char *>(W) + o * (BF16 ? 2 : 4)));
                 }
             }
         }
@@ -613,8 +584,172 @@ k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__
     grid_dep_wait();  // c and its sums (state pass), r and its sums (reduce pass)
     grid_dep_launch();
     const float inv_s = variant == EMBER_VARIANT_FULL ? step_inv_s<kThreads>(norm, kc) : 1.f;
-    apply_rows<VEC, CPT, R, BF16>(W, G, r, c, inv_s, V, D, ld, tpr, kc.inv_bc, eps, lr_signed, variant, span,
-                                  blockIdx.x);
+    for (int j = tid; j < D; j += kThreads) {
+        const float x = (variant == EMBER_VARIANT_ROW) ? 1.f : sqrtf(__ldcg(c + j) * kc.inv_bc * inv_s);
+        if constexpr (RAG) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                cs[m * csw + m + j] = x;
+        } else {
+            cs[j] = x;
+        }
+    }
+    __syncthreads();
+
+    for (int idx = warp; idx < nunits; idx += kWarps) {
+        const int rb = idx / nseg, seg = idx - rb * nseg;
+        const int64_t base = row1 - (int64_t)(rb + 1) * rows_per_unit;
+        F gv[R][K];
+        WT wr[R][K];
+        float rv[R];
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const int64_t i = base + k * rpa + lane / lpr;
+            rv[k] = (i >= row0) ? __ldcg(r + i) : 0.f;
+#pragma unroll
+            for (int cc = 0; cc < K; ++cc) {
+                const int v = (seg * K + cc) * lpr + l;
+                int m;
+                const int64_t o = offset(i, v, m);
+                if (i >= row0 && v < DV) {
+                    if (whole(v, m)) {
+                        gv[k][cc] = load_g<VEC>(G + o);
+                        wr[k][cc] = load_w<BF16, VEC>(W, o);
+                    } else if constexpr (RAG) {
+                        float g4[4], w4[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int col = 4 * v - m + e;
+                            const bool in = col >= 0 && col < D;
+                            g4[e] = in ? __ldg(G + o + e) : 0.f;
+                            w4[e] = 0.f;
+                            if (in) {
+                                float one[1];
+                                unpack_w(load_w<BF16, 1>(W, o + e), one);
+                                w4[e] = one[0];
+                            }
+                        }
+                        gv[k][cc] = make_float4(g4[0], g4[1], g4[2], g4[3]);
+                        wr[k][cc] = pack_w<BF16>(w4);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const int64_t i = base + k * rpa + lane / lpr;
+            const float rs = (variant == EMBER_VARIANT_COL) ? 1.f : sqrtf(rv[k] * kc.inv_bc);
+#pragma unroll
+            for (int cc = 0; cc < K; ++cc) {
+                const int v = (seg * K + cc) * lpr + l;
+                int m;
+                const int64_t o = offset(i, v, m);
+                if (i < row0 || v >= DV)
+                    continue;
+                float w[VEC];
+                unpack_w(wr[k][cc], w);
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) {
+                    const float den = fmaf(rs, cs[(RAG ? m * csw : 0) + v * VEC + e], eps);
+                    const float u = update_ratio(comp(gv[k][cc], e), den);
+                    w[e] = fmaf(lr_signed, u, w[e]);
+                }
+                if (whole(v, m)) {
+                    store_w<BF16, VEC>(W, o, w);
+                } else if constexpr (RAG) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int col = 4 * v - m + e;
+                        const float one[1] = {w[e]};
+                        if (col >= 0 && col < D)
+                            store_w<BF16, 1>(W, o + e, one);
+                    }
+                }
+            }
+        }
+    }
+}
+
+// How a warp of the update covers rows of pw columns: K accesses per lane
+// and unit, R row blocks per unit with R K about 8 (the accesses in flight),
+// segments of 32 K accesses chosen equal so that few lanes are idle.
+struct ApplyMap {
+    int lpr, nseg, k;
+};
+ApplyMap apply_map(int pw, int vec, bool rag)
+{
+    const int dv = rag ? (pw + 6) / 4 : pw / vec;
+    ApplyMap m{32, 1, 1};
+    if (dv < 32) {
+        for (m.lpr = 1; m.lpr < dv; m.lpr *= 2)
+            ;
+        return m;
+    }
+    m.nseg = (dv + 255) / 256;
+    m.k = (dv + 32 * m.nseg - 1) / (32 * m.nseg);
+    if (rag || vec == 1)  // fewer instantiations of the slower forms
+        while (m.k & (m.k - 1))
+            ++m.k;
+    return m;
+}
+
+struct ApplyArgs {
+    void *W;
+    const float *G;
+    const float *r, *c;
+    NormSource norm;
+    int64_t V;
+    int D, ld, mis;
+    StepConsts kc;
+    float eps, lr_signed;
+    int variant;
+    RowSpan span;
+    int ncta;
+    cudaStream_t stream;
+    bool pdl;
+};
+
+template <int VEC, int K, int R, bool RAG>
+cudaError_t launch_apply_t(const ApplyArgs &a, const ApplyMap &m, bool bf16)
+{
+    const size_t smem = sizeof(float) * (RAG ? 4 * (size_t)((a.D + 3) / 4 * 4 + 4) : (size_t)a.D);
+    auto *k = bf16 ? k_apply_dense<VEC, K, R, true, RAG> : k_apply_dense<VEC, K, R, false, RAG>;
+    return launch_k(k, dim3(a.ncta), dim3(kThreads), smem, a.stream, a.pdl, a.W, a.G, a.r, a.c, a.norm, a.V, a.D, a.ld,
+                    m.lpr, m.nseg, a.mis, a.kc, a.eps, a.lr_signed, a.variant, a.span);
+}
+
+// vec 4: every row starts on a 16-byte boundary of G (and as many elements
+// of W); rag: only W and G themselves do; otherwise 4-byte accesses.
+cudaError_t launch_apply(const ApplyArgs &a, int vec, bool rag, bool bf16)
+{
+    const ApplyMap m = apply_map(a.D, vec, rag);
+    if (rag) {
+        switch (m.k) {
+        case 1: return launch_apply_t<4, 1, 8, true>(a, m, bf16);
+        case 2: return launch_apply_t<4, 2, 4, true>(a, m, bf16);
+        case 4: return launch_apply_t<4, 4, 2, true>(a, m, bf16);
+        case 8: return launch_apply_t<4, 8, 1, true>(a, m, bf16);
+        }
+    } else if (vec == 4) {
+        switch (m.k) {
+        case 1: return launch_apply_t<4, 1, 8, false>(a, m, bf16);
+        case 2: return launch_apply_t<4, 2, 4, false>(a, m, bf16);
+        case 3: return launch_apply_t<4, 3, 2, false>(a, m, bf16);
+        case 4: return launch_apply_t<4, 4, 2, false>(a, m, bf16);
+        case 5: return launch_apply_t<4, 5, 1, false>(a, m, bf16);
+        case 6: return launch_apply_t<4, 6, 1, false>(a, m, bf16);
+        case 7: return launch_apply_t<4, 7, 1, false>(a, m, bf16);
+        case 8: return launch_apply_t<4, 8, 1, false>(a, m, bf16);
+        }
+    } else {
+        switch (m.k) {
+        case 1: return launch_apply_t<1, 1, 8, false>(a, m, bf16);
+        case 2: return launch_apply_t<1, 2, 4, false>(a, m, bf16);
+        case 4: return launch_apply_t<1, 4, 2, false>(a, m, bf16);
+        case 8: return launch_apply_t<1, 8, 1, false>(a, m, bf16);
+        }
+    }
+    return cudaErrorInvalidValue;
 }
 
 // ---------------------------------------------------------------------------
@@ -1100,7 +1235,6 @@ __global__ void k_shard_pack(const float *__restrict__ colpart, const float *__r
 template <int VEC, int CPT, int R1>
 cudaError_t launch_dense_t(const DenseArgs &a)
 {
-    constexpr int R3 = (8 / CPT) < 1 ? 1 : (8 / CPT);
     const int nparts = dense_parts(a.V, a.D);
     const int D = (int)a.D;
     DevScalars *sc = reinterpret_cast<DevScalars *>(a.ws + a.lay.scalars);
@@ -1114,6 +1248,10 @@ cudaError_t launch_dense_t(const DenseArgs &a)
     const int np = a.map.npanels;
     const int pw = a.map.pw;
     const int ld = (int)a.D;
+    // 16-byte accesses at shifted rows: only the arrays need to be aligned
+    auto rag_ok = [](const void *W, const float *G, int wbf16) {
+        return VEC == 1 && (uintptr_t)G % 16 == 0 && (uintptr_t)W % (wbf16 ? 8 : 16) == 0;
+    };
     auto cols = [&](int q) { return (q + 1 < np) ? pw : (int)(a.D - (int64_t)q * pw); };
     const size_t shmem = (rg > 1) ? (size_t)rg * pw * sizeof(float) : 0;  // the row groups' column sums
 
@@ -1157,15 +1295,9 @@ cudaError_t launch_dense_t(const DenseArgs &a)
         if (e != cudaSuccess || ncta == 0)
             return e != cudaSuccess ? e : cudaGetLastError();
         const NormSource norm{rsum_part, 0, csum_part, (D + kStateCols - 1) / kStateCols, sh.sums, sh.scales, D};
-        const size_t cs_bytes = (size_t)D * sizeof(float);
-        if (a.wbf16)
-            e = launch_k(k_apply_dense<VEC, CPT, R3, true>, dim3(ncta), dim3(kThreads), cs_bytes, a.stream, pdl,
-                         a.W, a.G, a.r, a.c, norm, a.V, D, ld, a.map.tpr, kc, a.eps, a.lr_signed,
-                         a.variant, span);
-        else
-            e = launch_k(k_apply_dense<VEC, CPT, R3, false>, dim3(ncta), dim3(kThreads), cs_bytes, a.stream, pdl,
-                         a.W, a.G, a.r, a.c, norm, a.V, D, ld, a.map.tpr, kc, a.eps, a.lr_signed,
-                         a.variant, span);
+        e = launch_apply(ApplyArgs{a.W, a.G, a.r, a.c, norm, a.V, D, ld, 0, kc, a.eps, a.lr_signed, a.variant, span,
+                                   ncta, a.stream, pdl},
+                         VEC, rag_ok(a.W, a.G, a.wbf16), a.wbf16);
         return e != cudaSuccess ? e : cudaGetLastError();
     }
     if (a.variant == EMBER_VARIANT_ROW && !a.lm && np == 1) {
@@ -1286,7 +1418,8 @@ cudaError_t launch_dense_t(const DenseArgs &a)
             const int64_t vb = (a.V + kStateThreads - 1) / kStateThreads;
             const int nrow_ctas = (int)(vb < kMaxRowCtas ? vb : kMaxRowCtas);
             nrsum = nrow_ctas;
-            e = launch_state(colpart, nparts, rsum_part, a.c, csum_part, sc, a.V, D, kc, a.stream, pdl, a.r, nullptr, rowpart, np, nrow_ctas);
+            e = launch_state(colpart, nparts, rsum_part, a.c, csum_part, sc, a.V, D, kc, a.stream, pdl, a.r, nullptr, rowpart, np,
+                             nrow_ctas);
         }
         if (e != cudaSuccess)
             return e;
@@ -1296,19 +1429,14 @@ cudaError_t launch_dense_t(const DenseArgs &a)
     const float *Gd = a.lm ? a.lm->G : a.G_stage ? a.G_stage : a.G;
     if (a.trace)
         cudaEventRecord(a.trace[2], a.stream);
-    const size_t cs_bytes = (size_t)pw * sizeof(float);
     const NormSource norm{rsum_part, nrsum, csum_part, (D + kStateCols - 1) / kStateCols, nullptr, nullptr, D};
+    const bool rag = rag_ok(a.W, Gd, a.wbf16);
     for (int q = np - 1; q >= 0; --q) {
         const int64_t c0 = (int64_t)q * pw;
         void *Wq = static_cast<unsigned char *>(a.W) + c0 * (a.wbf16 ? 2 : 4);
-        if (a.wbf16)
-            e = launch_k(k_apply_dense<VEC, CPT, R3, true>, dim3(nparts), dim3(kThreads), cs_bytes,
-                         a.stream, pdl, Wq, Gd + c0, a.r, a.c + c0, norm, a.V, cols(q), ld, a.map.tpr,
-                         kc, a.eps, a.lr_signed, a.variant, span);
-        else
-            e = launch_k(k_apply_dense<VEC, CPT, R3, false>, dim3(nparts), dim3(kThreads), cs_bytes,
-                         a.stream, pdl, Wq, Gd + c0, a.r, a.c + c0, norm, a.V, cols(q), ld, a.map.tpr,
-                         kc, a.eps, a.lr_signed, a.variant, span);
+        e = launch_apply(ApplyArgs{Wq, Gd + c0, a.r, a.c + c0, norm, a.V, cols(q), ld, (int)(c0 & 3), kc, a.eps,
+                                   a.lr_signed, a.variant, span, nparts, a.stream, pdl},
+                         VEC, rag, a.wbf16);
         if (e != cudaSuccess)
             return e;
     }

@@ -120,6 +120,17 @@ __device__ __forceinline__ void unpack_w(const float4 &f, float (&w)[4])
 }
 __device__ __forceinline__ void unpack_w(const float &f, float (&w)[1]) { w[0] = f; }
 
+// Four weights as a raw vector, from values that its type holds exactly.
+template <bool BF16>
+__device__ __forceinline__ typename WRaw<BF16, 4>::T pack_w(const float (&w)[4])
+{
+    if constexpr (BF16)
+        return make_uint2((__float_as_uint(w[0]) >> 16) | (__float_as_uint(w[1]) & 0xFFFF0000u),
+                          (__float_as_uint(w[2]) >> 16) | (__float_as_uint(w[3]) & 0xFFFF0000u));
+    else
+        return make_float4(w[0], w[1], w[2], w[3]);
+}
+
 template <bool BF16, int VEC>
 __device__ __forceinline__ void store_w(void *W, int64_t idx, const float (&w)[VEC])
 {
@@ -144,6 +155,12 @@ __device__ __forceinline__ uint64_t policy_evict_first()
 {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ uint64_t policy_evict_normal()
+{
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
 __device__ __forceinline__ uint64_t policy_evict_last()

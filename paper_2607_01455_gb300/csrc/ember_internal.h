@@ -34,6 +34,10 @@ constexpr int kStateThreads = 1024;
 constexpr int kMaxRowCtas = 1024;
 constexpr int kRsumParts = kMaxRowCtas > kGridCtas ? kMaxRowCtas : kGridCtas;
 
+// Bytes of G that the reduce pass leaves in L2 for the update: a little over
+// half of the 129 MB (the update's rows of W need the rest).
+constexpr int64_t kKeepBytes = 70 << 20;
+
 // Bits of the sticky device flag.
 constexpr unsigned kFlagIdRange = 1u << 0;
 constexpr unsigned kFlagTimeout = 1u << 1;
@@ -277,8 +281,8 @@ struct NormSource {
 cudaError_t launch_state(const float *colpart, int nparts, float *rsum_part, float *c,
                          float *csum_part, const DevScalars *sc, int64_t V, int D, const StepConsts &k,
                          cudaStream_t stream, bool pdl, float *r_rows, int32_t *slot, const float *rowpart,
-                         int nslices, int nrow_ctas, const int32_t *uniq = nullptr, int rsum_base = 0,
-                         int pstride = 1, int pcols = 0);
+                         int nslices, int nrow_ctas, const int32_t *uniq = nullptr,
+                         int rsum_base = 0, int pstride = 1, int pcols = 0);
 
 struct SparseArgs {
     int64_t V, D, N;
