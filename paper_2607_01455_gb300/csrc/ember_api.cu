@@ -41,8 +41,12 @@ Layout make_layout(int64_t V, int64_t D, int64_t max_sparse_N)
         L.sp_slot = take(sizeof(int32_t) * (size_t)V);
         L.sp_single = take(sizeof(int32_t) * N);
         L.sp_rowpart = take(sizeof(float) * N * nslices);
-        L.sp_carry = take(sizeof(float) * 2 * (size_t)kSparseCtas * (size_t)D);
-        L.sp_bounds = take(sizeof(int32_t) * ((size_t)kSparseCtas + 1));
+        // two pieces of at most D columns per worker; a CTA's workers cover
+        // kThreads accesses of up to 4 columns, or it is one worker
+        const size_t wide = (size_t)(D > 4 * kThreads ? D : 4 * kThreads);
+        L.sp_carry = take(sizeof(float) * 2 * (size_t)kSparseCtas * wide);
+        L.sp_bounds = take(sizeof(int32_t) * ((size_t)kSparseCtas * (kThreads / 32) + 1));
+        L.sp_cuts = take(sizeof(int2) * (size_t)kSparseCtas * (kThreads / 32));
         L.sp_rows = take(sizeof(float) * N * (size_t)D);
     }
     L.lm_colpart = take(sizeof(float) * (size_t)lmhead_row_blocks(V) * (size_t)D);

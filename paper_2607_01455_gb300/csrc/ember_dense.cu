@@ -671,12 +671,16 @@ k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__
 }
 
 // How a warp of the update covers rows of pw columns: K accesses per lane
-// and unit, R row blocks per unit with R K about 8 (the accesses in flight),
-// segments of 32 K accesses chosen equal so that few lanes are idle.
+// and unit, R row blocks per unit, segments of 32 K accesses chosen equal so
+// that few lanes are idle.  R K accesses of G and W are in flight per lane:
+// about 8 with bf16 weights and 4 to 6 with fp32 ones, 65 to 100 KB per SM
+// either way.  More makes the step slower, not only less: 32000 x 4096 fp32
+// takes 326.5 us with 4 (66 KB) and 334 with 8 (131 KB); bf16 50257 x 768
+// takes 88 us with 6 (74 KB), 104 with 3 and 94 with three CTAs per SM.
 struct ApplyMap {
     int lpr, nseg, k;
 };
-ApplyMap apply_map(int pw, int vec, bool rag)
+ApplyMap apply_map(int pw, int vec, bool rag, bool bf16)
 {
     const int dv = rag ? (pw + 6) / 4 : pw / vec;
     ApplyMap m{32, 1, 1};
@@ -685,7 +689,10 @@ ApplyMap apply_map(int pw, int vec, bool rag)
             ;
         return m;
     }
-    m.nseg = (dv + 255) / 256;
+    if (bf16 || rag || vec == 1)
+        m.nseg = (dv + 255) / 256;
+    else
+        m.nseg = dv <= 192 ? 1 : (dv + 127) / 128;
     m.k = (dv + 32 * m.nseg - 1) / (32 * m.nseg);
     if (rag || vec == 1)  // fewer instantiations of the slower forms
         while (m.k & (m.k - 1))
@@ -709,11 +716,11 @@ struct ApplyArgs {
     bool pdl;
 };
 
-template <int VEC, int K, int R, bool RAG>
+template <int VEC, int K, int RB, int RF, bool RAG>  // RB, RF: R with bf16 and with fp32 weights
 cudaError_t launch_apply_t(const ApplyArgs &a, const ApplyMap &m, bool bf16)
 {
     const size_t smem = sizeof(float) * (RAG ? 4 * (size_t)((a.D + 3) / 4 * 4 + 4) : (size_t)a.D);
-    auto *k = bf16 ? k_apply_dense<VEC, K, R, true, RAG> : k_apply_dense<VEC, K, R, false, RAG>;
+    auto *k = bf16 ? k_apply_dense<VEC, K, RB, true, RAG> : k_apply_dense<VEC, K, RF, false, RAG>;
     return launch_k(k, dim3(a.ncta), dim3(kThreads), smem, a.stream, a.pdl, a.W, a.G, a.r, a.c, a.norm, a.V, a.D, a.ld,
                     m.lpr, m.nseg, a.mis, a.kc, a.eps, a.lr_signed, a.variant, a.span);
 }
@@ -722,31 +729,31 @@ cudaError_t launch_apply_t(const ApplyArgs &a, const ApplyMap &m, bool bf16)
 // of W); rag: only W and G themselves do; otherwise 4-byte accesses.
 cudaError_t launch_apply(const ApplyArgs &a, int vec, bool rag, bool bf16)
 {
-    const ApplyMap m = apply_map(a.D, vec, rag);
+    const ApplyMap m = apply_map(a.D, vec, rag, bf16);
     if (rag) {
         switch (m.k) {
-        case 1: return launch_apply_t<4, 1, 8, true>(a, m, bf16);
-        case 2: return launch_apply_t<4, 2, 4, true>(a, m, bf16);
-        case 4: return launch_apply_t<4, 4, 2, true>(a, m, bf16);
-        case 8: return launch_apply_t<4, 8, 1, true>(a, m, bf16);
+        case 1: return launch_apply_t<4, 1, 8, 8, true>(a, m, bf16);
+        case 2: return launch_apply_t<4, 2, 4, 4, true>(a, m, bf16);
+        case 4: return launch_apply_t<4, 4, 2, 2, true>(a, m, bf16);
+        case 8: return launch_apply_t<4, 8, 1, 1, true>(a, m, bf16);
         }
     } else if (vec == 4) {
         switch (m.k) {
-        case 1: return launch_apply_t<4, 1, 8, false>(a, m, bf16);
-        case 2: return launch_apply_t<4, 2, 4, false>(a, m, bf16);
-        case 3: return launch_apply_t<4, 3, 2, false>(a, m, bf16);
-        case 4: return launch_apply_t<4, 4, 2, false>(a, m, bf16);
-        case 5: return launch_apply_t<4, 5, 1, false>(a, m, bf16);
-        case 6: return launch_apply_t<4, 6, 1, false>(a, m, bf16);
-        case 7: return launch_apply_t<4, 7, 1, false>(a, m, bf16);
-        case 8: return launch_apply_t<4, 8, 1, false>(a, m, bf16);
+        case 1: return launch_apply_t<4, 1, 8, 4, false>(a, m, bf16);
+        case 2: return launch_apply_t<4, 2, 4, 2, false>(a, m, bf16);
+        case 3: return launch_apply_t<4, 3, 2, 2, false>(a, m, bf16);
+        case 4: return launch_apply_t<4, 4, 2, 1, false>(a, m, bf16);
+        case 5: return launch_apply_t<4, 5, 1, 1, false>(a, m, bf16);
+        case 6: return launch_apply_t<4, 6, 1, 1, false>(a, m, bf16);
+        case 7: return launch_apply_t<4, 7, 1, 1, false>(a, m, bf16);
+        case 8: return launch_apply_t<4, 8, 1, 1, false>(a, m, bf16);
         }
     } else {
         switch (m.k) {
-        case 1: return launch_apply_t<1, 1, 8, false>(a, m, bf16);
-        case 2: return launch_apply_t<1, 2, 4, false>(a, m, bf16);
-        case 4: return launch_apply_t<1, 4, 2, false>(a, m, bf16);
-        case 8: return launch_apply_t<1, 8, 1, false>(a, m, bf16);
+        case 1: return launch_apply_t<1, 1, 8, 8, false>(a, m, bf16);
+        case 2: return launch_apply_t<1, 2, 4, 4, false>(a, m, bf16);
+        case 4: return launch_apply_t<1, 4, 2, 2, false>(a, m, bf16);
+        case 8: return launch_apply_t<1, 8, 1, 1, false>(a, m, bf16);
         }
     }
     return cudaErrorInvalidValue;

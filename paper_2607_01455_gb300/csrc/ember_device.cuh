@@ -186,6 +186,19 @@ __device__ __forceinline__ typename Vec<VEC>::F load_g_hint(const float *p, uint
     }
 }
 
+// VEC floats from global to shared memory, asynchronously.
+template <int VEC>
+__device__ __forceinline__ void cp_async_hint(void *smem, const float *p, uint64_t pol)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
+    if constexpr (VEC == 4)
+        asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(d), "l"(p), "l"(pol)
+                     : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 4, %2;" ::"r"(d), "l"(p), "l"(pol)
+                     : "memory");
+}
+
 template <bool BF16, int VEC>
 __device__ __forceinline__ typename WRaw<BF16, VEC>::T load_w_hint(const void *W, int64_t idx, uint64_t pol)
 {

@@ -19,8 +19,7 @@ constexpr int kThreads = 256;
 constexpr int kCtasPerSm = 2;
 constexpr int kSms = 152;
 constexpr int kGridCtas = kSms * kCtasPerSm;
-// The sparse step's segment sums run three smaller CTAs per SM.
-constexpr int kSparseCtasPerSm = 3;
+constexpr int kSparseCtasPerSm = 2;  // of the sparse step's segment sums
 constexpr int kSparseCtas = kSms * kSparseCtasPerSm;
 constexpr int kPartRows = kSparseCtas > kGridCtas ? kSparseCtas : kGridCtas;
 
@@ -81,8 +80,9 @@ struct Layout {
     size_t sp_slot;     // int32[V]      1 + distinct-id index of a touched row, else 0
     size_t sp_single;   // int32[N]      occurrence index of an id seen once, else -1
     size_t sp_rowpart;  // float[N * ceil(D / kThreads)]  sum g^2 per (distinct id, slice)
-    size_t sp_carry;    // float[2 * kSparseCtas * D]  partial sums of runs cut by worker ranges
-    size_t sp_bounds;   // int32[kSparseCtas + 1]  first sorted position of each worker range
+    size_t sp_carry;    // float[2 * kSparseCtas * max(D, 1024)]  partial sums of runs cut by worker ranges
+    size_t sp_bounds;   // int32[8 * kSparseCtas + 1]  first sorted position of each worker range
+    size_t sp_cuts;     // int2[8 * kSparseCtas]  run cut by each worker's start, and the worker it ends in
     size_t sp_rows;     // float[N * D]  summed gradient row of each distinct id seen twice or more
     // LM-head step (the gradient formed here on the tensor cores)
     size_t lm_colpart;  // float[ceil(V/128) * D]  sums of g^2 over each 128-row block

@@ -326,6 +326,29 @@ __device__ __forceinline__ int64_t cost_target(int w, int nw, int64_t C)
     return ((int64_t)w * C) / nw;
 }
 
+// Workers in use: of the nw1 rg groups of a slice's CTAs (group g of CTA b is
+// worker g nw1 + b), nw1 times as many groups as have kMinRows occurrences
+// each.  A worker of fewer rows would mostly wait for its indices.  A function of the valid ids, so that skipped ones
+// change nothing.
+constexpr int kMinRows = 16;
+__device__ __forceinline__ int workers_of(int n_valid, int nw1, int rg)
+{
+    const int most = n_valid / (kMinRows * nw1);
+    return nw1 * (most < 1 ? 1 : most < rg ? most : rg);
+}
+
+// Worker whose range holds sorted position p of run u.
+__device__ __forceinline__ int worker_of(int p, int u, int nw, int64_t C)
+{
+    const int64_t c = (int64_t)p + u;
+    int w = (int)((c * nw) / C);
+    while (w + 1 < nw && cost_target(w + 1, nw, C) <= c)
+        ++w;
+    while (w > 0 && cost_target(w, nw, C) > c)
+        --w;
+    return w;
+}
+
 // Each run's occurrences in increasing order, and the workers' bounds.
 // A run of up to kLongRun occurrences: the thread of each position counts the
 // smaller ones in its run (a warp's positions mostly share a run, so the
@@ -339,7 +362,7 @@ __global__ void __launch_bounds__(kOrderThreads)
 k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segidx,
            const int32_t *__restrict__ segoff, const int32_t *__restrict__ longrun,
            const int32_t *__restrict__ nlong, const DevScalars *__restrict__ sc, int64_t N, int nbig,
-           int32_t *__restrict__ perm, int32_t *__restrict__ bounds, int nw)
+           int32_t *__restrict__ perm, int32_t *__restrict__ bounds, int2 *__restrict__ cuts, int nw1, int rg)
 {
     constexpr int kW = kOrderThreads / 32;
     constexpr int kPer = 16;
@@ -366,7 +389,10 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
         }
         // the workers whose target lies above the position before this one
         // and not above this one start here (and those above the last
-        // position at the end)
+        // position at the end); cuts[q]: the run that goes on at the start of
+        // worker q and began in worker q - 1's range, and the worker it ends
+        // in, or (-1, 0)
+        const int nw = workers_of(n_valid, nw1, rg);
         const int64_t C = (int64_t)n_valid + U;
         const int64_t c1 = p + u;
         const int64_t c0 = p > 0 ? p - 1 + before : -1;
@@ -375,6 +401,10 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
             if (!here && p + 1 < n_valid)
                 break;
             bounds[q] = here ? (int)p : n_valid;
+            int2 cut = make_int2(-1, 0);
+            if (here && s < p && q > 0 && cost_target((int)q - 1, nw, C) <= (int64_t)s + u)
+                cut = make_int2(u, worker_of(e - 1, u, nw, C));
+            cuts[q] = cut;
         }
         if (p + 1 == n_valid)
             bounds[nw] = n_valid;
@@ -440,51 +470,108 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
     }
 }
 
-// Worker whose range holds sorted position p of run u.
-__device__ __forceinline__ int worker_of(int p, int u, int nw, int64_t C)
+// How the segment sums cover D columns: NS slices of tpb threads (one access
+// each, equal slices so that few threads are idle), and rg groups of tpb
+// threads per CTA (a narrow row leaves room for several), each group a worker
+// of its own.
+struct SumMap {
+    int NS, tpb, rg;
+};
+SumMap sum_map(int DV)
 {
-    const int64_t c = (int64_t)p + u;
-    int w = (int)((c * nw) / C);
-    while (w + 1 < nw && cost_target(w + 1, nw, C) <= c)
-        ++w;
-    while (w > 0 && cost_target(w, nw, C) > c)
-        --w;
-    return w;
+    SumMap m;
+    m.NS = (DV + kThreads - 1) / kThreads;
+    m.tpb = ((DV + m.NS - 1) / m.NS + 31) / 32 * 32;
+    m.rg = kThreads / m.tpb;
+    return m;
 }
 
-// Sum the occurrences of each run.  CTA b works on column slice b % NS
-// (kThreads vector columns) of the sorted positions of worker b / NS, adding
-// each run's rows in increasing occurrence order with a running sum that
-// crosses the worker's whole range.  A run that starts before the range or
-// ends after it leaves its piece in the carry buffer (slot 0: the range's
-// first run, slot 1: its last run); k_sp_carry adds the pieces in worker
-// order.  Completed runs are written to S with their sum of g^2 per slice.
-template <int VEC>
+// Barrier over the tpb threads of one group (named barriers 1 .. 8), or over
+// the CTA when it is one group.
+__device__ __forceinline__ void group_bar(int g, int rg, int tpb)
+{
+    if (rg == 1)
+        __syncthreads();
+    else
+        asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(tpb) : "memory");
+}
+
+// Column sums of the CTA's groups, added in group order, to (or onto) its
+// partial row.
+template <int VEC, bool ADD>
+__device__ __forceinline__ void combine_groups(const float (&colacc)[VEC], float *comb, float *out, int g, int l,
+                                               int tpb, int rg, int col0, int width)
+{
+#pragma unroll
+    for (int e = 0; e < VEC; ++e)
+        comb[(g * tpb + l) * VEC + e] = colacc[e];
+    __syncthreads();
+    for (int j = threadIdx.x; j < width; j += blockDim.x) {
+        float t = comb[j];
+        for (int q = 1; q < rg; ++q)
+            t += comb[q * tpb * VEC + j];
+        if (ADD)
+            t += out[col0 + j];
+        out[col0 + j] = t;
+    }
+}
+
+// Sum the occurrences of each run.  A group of tpb threads works on column
+// slice sigma of the sorted positions of its worker, adding each run's rows
+// in increasing occurrence order with a running sum that crosses the worker's
+// whole range.  A run that starts before the range or ends after it leaves
+// its piece in the carry buffer (slot 0: the range's first run, slot 1: its
+// last run); k_sp_carry adds the pieces in worker order.  Completed runs are
+// written to S with their sum of g^2 per slice.
+//   Bound by HBM (the occurrence rows are read once).  Each thread copies its
+// own column slice of the rows to come into a ring of kRing rows in shared
+// memory with cp.async, kBatch rows per commit group, so that the copies in
+// flight take no registers and no row waits for the adds of another; a thread
+// reads back only what it copied itself, so the ring needs no barrier.  A
+// ring is 48 KiB (two CTAs: 96 KiB in flight per SM) whatever the width:
+// 32768 rows of 2048 columns (4 KiB slices) take 105.8 us per step with 12
+// rows, 115 with 18 of them per CTA's worth in flight (three CTAs); 262144 rows
+// of 768 columns 219.7 us with 16 rows, 222.0 with 12, 226.7 with 20.
+constexpr int kBatch = 4;
+constexpr int kRingBytes = 48 << 10;
+template <int VEC, int NT>
+constexpr int ring_rows() { return kRingBytes / (4 * VEC * NT) / kBatch * kBatch; }
+template <int VEC, int NT>  // NT: at least the CTA's threads
 __global__ void __launch_bounds__(kThreads, kSparseCtasPerSm)
 k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
             const int32_t *__restrict__ segidx, const DevScalars *__restrict__ sc,
             float *__restrict__ S, float *__restrict__ rowpart, float *__restrict__ carry,
-            float *__restrict__ colpart, const int32_t *__restrict__ bounds, int D, int NS,
+            float *__restrict__ colpart, const int32_t *__restrict__ bounds, int D, SumMap map,
             int32_t *__restrict__ counters, int ncounters)
 {
     using F = typename Vec<VEC>::F;
-    constexpr int R = 8;  // rows in flight per thread
+    constexpr int kRing = ring_rows<VEC, NT>();
+    constexpr int kFin = 8;               // completed runs buffered before their g^2 sums are written
     constexpr int kWarps = kThreads / 32;
-    constexpr int kFin = 128;  // completed runs buffered before their g^2 sums are written
-    constexpr int kIdxWindow = 1024;
-    __shared__ float rp[kFin][kWarps];
-    __shared__ int fin[kFin];
+    constexpr int kIdxWindow = 1024;      // occurrences whose indices the CTA holds
+    __shared__ float rp[kFin][kThreads];
+    __shared__ int fin[kWarps][kFin];
     __shared__ int sperm[kIdxWindow];
     __shared__ int sseg[kIdxWindow];
+    __shared__ float comb[kThreads * VEC];
     const int DV = D / VEC;
+    const int NS = map.NS, tpb = map.tpb, rg = map.rg;
+    const int g = threadIdx.x / tpb;
+    const int l = threadIdx.x - g * tpb;
     const int sigma = blockIdx.x % NS;
-    const int w = blockIdx.x / NS;
-    const int nw = gridDim.x / NS;
-    const int col = sigma * kThreads + threadIdx.x;
+    const int nw1 = (int)(gridDim.x / NS);
+    const int b1 = (int)(blockIdx.x / NS);  // nw1 or more: a CTA left over by the division
+    const int w = g * nw1 + b1;
+    const int col = sigma * tpb + l;
     const bool active = col < DV;
     // threads past the row's end load its last vector (and discard the sums)
     const float *src = rows + (int64_t)(active ? col : DV - 1) * VEC;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int wpg = tpb >> 5;
+    const int window = kIdxWindow / rg;
+    int *const wperm = sperm + g * window, *const wseg = sseg + g * window;
+    extern __shared__ __align__(16) unsigned char sp_ring[];
+    F *const ring = reinterpret_cast<F *>(sp_ring) + threadIdx.x;  // slot q at ring[q * NT]
     grid_dep_wait();  // runs and occurrence order from the dedup kernels
     grid_dep_launch();
     const int n_valid = sc->n_valid;
@@ -497,9 +584,8 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
     const uint64_t pol_rows = policy_evict_first();
     const uint64_t pol_sums = policy_evict_last();
 
-    const bool worker = w < nw && n_valid > 0;
     int p0 = 0, p1 = 0;
-    if (worker) {
+    if (b1 < nw1 && n_valid > 0 && w < workers_of(n_valid, nw1, rg)) {
         p0 = bounds[w];
         p1 = bounds[w + 1];
         if (p0 == p1 && active) {
@@ -510,15 +596,20 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
         }
     }
     int nfin = 0;
-    auto drain = [&]() {  // uniform: all threads call it together
-        __syncthreads();
-        if (threadIdx.x < nfin) {
+    // the buffered runs' sums of g^2 over the group's threads, a warp per run
+    auto drain = [&]() {  // uniform over the group
+        group_bar(g, rg, tpb);
+        for (int q = warp - g * wpg; q < nfin; q += wpg) {
             float t = 0.f;
-            for (int k = 0; k < kWarps; ++k)
-                t += rp[threadIdx.x][k];
-            rowpart[(int64_t)fin[threadIdx.x] * NS + sigma] = t;
+            for (int k = lane; k < tpb; k += 32)
+                t += rp[q][g * tpb + k];
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1)
+                t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0)
+                rowpart[(int64_t)fin[g][q] * NS + sigma] = t;
         }
-        __syncthreads();
+        group_bar(g, rg, tpb);
         nfin = 0;
     };
     if (p0 < p1) {
@@ -554,13 +645,9 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
                         ps += a * a;
                     }
                 }
-#pragma unroll
-                for (int o = 16; o >= 1; o >>= 1)
-                    ps += __shfl_xor_sync(0xffffffffu, ps, o);
-                if (lane == 0)
-                    rp[nfin][warp] = ps;
-                if (threadIdx.x == 0)
-                    fin[nfin] = u;
+                rp[nfin][threadIdx.x] = ps;
+                if (l == 0)
+                    fin[g][nfin] = u;
                 ++nfin;
                 if (nfin == kFin)
                     drain();
@@ -570,92 +657,114 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
             }
         };
         // The range's occurrence and run indices go to shared memory a
-        // window at a time, so each batch of rows costs one trip to HBM.
-        for (int wb = p0; wb < p1; wb += kIdxWindow) {
-            const int we = (wb + kIdxWindow < p1) ? wb + kIdxWindow : p1;
-            __syncthreads();  // the previous window's indices are no longer read
-            for (int p = wb + threadIdx.x; p < we; p += kThreads) {
-                sperm[p - wb] = perm[p];
-                sseg[p - wb] = segidx[p];
+        // window at a time, so that a row costs one trip to HBM.
+        for (int wb = p0; wb < p1; wb += window) {
+            const int n = (wb + window < p1 ? wb + window : p1) - wb;
+            group_bar(g, rg, tpb);  // the previous window's indices are no longer read
+            for (int q = l; q < n; q += tpb) {
+                wperm[q] = perm[wb + q];
+                wseg[q] = segidx[wb + q];
             }
-            __syncthreads();
-            for (int pb = wb; pb < we; pb += R) {
-                // R rows in flight; only the window's last batch is partial
-                const int nb = (we - pb < R) ? we - pb : R;
-                const int *bp = sperm + (pb - wb);
-                F v[R];
-                if (nb == R) {
+            group_bar(g, rg, tpb);
+            // rows b .. b + kBatch - 1 of the window into the kBatch slots
+            // from `slot` on, one commit group
+            auto fetch = [&](int b, F *slot) {
+                if (b + kBatch <= n) {
 #pragma unroll
-                    for (int k = 0; k < R; ++k)
-                        v[k] = load_g_hint<VEC>(src + (int64_t)bp[k] * D, pol_rows);
+                    for (int k = 0; k < kBatch; ++k)
+                        cp_async_hint<VEC>(slot + k * NT, src + (int64_t)wperm[b + k] * D, pol_rows);
                 } else {
+                    for (int k = 0; b + k < n; ++k)
+                        cp_async_hint<VEC>(slot + k * NT, src + (int64_t)wperm[b + k] * D, pol_rows);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            auto add = [&](const F &x, int u) {
+                if (u != cur) {
+                    flush(cur);
+                    acc = zero_vec<VEC>();
+                    cmp = zero_vec<VEC>();
+                    cur = u;
+                    len = 0;
+                }
+                ++len;
 #pragma unroll
-                    for (int k = 0; k < R; ++k)
-                        v[k] = (k < nb) ? load_g_hint<VEC>(src + (int64_t)bp[k] * D, pol_rows) : zero_vec<VEC>();
+                for (int e = 0; e < VEC; ++e) {
+                    const float y = comp(x, e) - comp(cmp, e);
+                    const float t = comp(acc, e) + y;
+                    set_comp(cmp, e, (t - comp(acc, e)) - y);
+                    set_comp(acc, e, t);
+                }
+            };
+            F *slot = ring;
+#pragma unroll 1
+            for (int b = 0; b < kRing; b += kBatch)
+                fetch(b, ring + b * NT);
+            int b = 0;
+#pragma unroll 1
+            for (; b + kBatch <= n; b += kBatch) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(kRing / kBatch - 1) : "memory");
+                F v[kBatch];
+                int u[kBatch];
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) {
+                    v[k] = slot[k * NT];
+                    u[k] = wseg[b + k];
                 }
 #pragma unroll
-                for (int k = 0; k < R; ++k) {
-                    if (k >= nb)
-                        break;
-                    const int u = sseg[pb - wb + k];
-                    if (u != cur) {
-                        flush(cur);
-                        acc = zero_vec<VEC>();
-                        cmp = zero_vec<VEC>();
-                        cur = u;
-                        len = 0;
-                    }
-                    ++len;
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) {
-                        const float y = comp(v[k], e) - comp(cmp, e);
-                        const float t = comp(acc, e) + y;
-                        set_comp(cmp, e, (t - comp(acc, e)) - y);
-                        set_comp(acc, e, t);
-                    }
-                }
+                for (int k = 0; k < kBatch; ++k)
+                    add(v[k], u[k]);
+                fetch(b + kRing, slot);
+                slot = (slot == ring + (kRing - kBatch) * NT) ? ring : slot + kBatch * NT;
             }
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            for (int k = 0; b + k < n; ++k)
+                add(slot[k * NT], wseg[b + k]);
         }
         flush(cur);
     }
     if (nfin > 0)
         drain();
-    float *out = colpart + (int64_t)blockIdx.x * D;
-    for (int j = threadIdx.x; j < D; j += kThreads)
-        out[j] = 0.f;
-    __syncthreads();
-    if (active && worker)
-#pragma unroll
-        for (int e = 0; e < VEC; ++e)
-            out[col * VEC + e] = colacc[e];
+    // this CTA's partial row: its own slice's column sums (the column pass
+    // reads no other columns of it)
+    const int col0 = sigma * tpb * VEC;
+    combine_groups<VEC, false>(colacc, comb, colpart + (int64_t)blockIdx.x * D, g, l, tpb, rg, col0,
+                               col0 + tpb * VEC < D ? tpb * VEC : D - col0);
 
     // the dedup's range counts and list length start the next step at zero
     if (blockIdx.x == 0)
-        for (int q = threadIdx.x; q < ncounters; q += kThreads)
+        for (int q = threadIdx.x; q < ncounters; q += blockDim.x)
             counters[q] = 0;
 }
 
-// Runs cut by worker boundaries.  CTA b handles boundary bd = b / NS + 1
-// (position first(bd)) on slice b % NS: if the run holding that position
-// started inside the previous worker's range, this CTA adds the run's
-// pieces -- the previous worker's last piece, then the first pieces of the
-// following workers up to the one holding the run's end -- in worker order.
+// Runs cut by worker boundaries.  Group g of CTA b handles the boundary
+// before worker bd = g nw1 + b / NS + 1 on slice b % NS: if a run that
+// started inside the previous worker's range goes on there, this group adds
+// the run's pieces -- the previous worker's last piece, then the first pieces
+// of the following workers up to the one holding the run's end -- in worker
+// order.
 template <int VEC>
 __global__ void __launch_bounds__(kThreads, kSparseCtasPerSm)
-k_sp_carry(const int32_t *__restrict__ segidx, const int32_t *__restrict__ segoff,
-           const int32_t *__restrict__ bounds, const DevScalars *__restrict__ sc,
-           const float *__restrict__ carry, float *__restrict__ S, float *__restrict__ rowpart,
-           float *__restrict__ colpart, int D, int NS, int nw)
+k_sp_carry(const int2 *__restrict__ cuts, const DevScalars *__restrict__ sc, const float *__restrict__ carry, float *__restrict__ S, float *__restrict__ rowpart,
+           float *__restrict__ colpart, int D, SumMap map)
 {
     using F = typename Vec<VEC>::F;
     constexpr int kWarps = kThreads / 32;
+    constexpr int kManyPieces = 24;
     __shared__ float red[kWarps];
+    __shared__ float comb[kThreads * VEC];
+    __shared__ int3 shared_cut[kWarps];
     const int DV = D / VEC;
+    const int NS = map.NS, tpb = map.tpb, rg = map.rg;
+    const int g = threadIdx.x / tpb;
+    const int l = threadIdx.x - g * tpb;
     const int sigma = blockIdx.x % NS;
-    const int bd = blockIdx.x / NS + 1;
-    const int col = sigma * kThreads + threadIdx.x;
+    const int nw1 = (int)(gridDim.x / NS);
+    const int bd = g * nw1 + (int)(blockIdx.x / NS) + 1;
+    const int col = sigma * tpb + l;
     const bool active = col < DV;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int wpg = tpb >> 5;
     grid_dep_wait();  // carry pieces from k_sp_segsum
     grid_dep_launch();
     const int n_valid = sc->n_valid;
@@ -663,47 +772,41 @@ k_sp_carry(const int32_t *__restrict__ segidx, const int32_t *__restrict__ segof
 #pragma unroll
     for (int e = 0; e < VEC; ++e)
         colacc[e] = 0.f;
-    bool mine = false;
-    int u = 0, w0 = 0, w1 = 0;
-    if (bd < nw && n_valid > 0) {
-        const int p = bounds[bd];
-        if (p < n_valid) {
-            u = segidx[p];
-            const int s0 = segoff[u], s1 = segoff[u + 1];
-            w0 = bd - 1;
-            mine = s0 < p && s0 >= bounds[w0];
-            const int64_t C = (int64_t)n_valid + sc->n_unique;
-            w1 = worker_of(s1 - 1, u, nw, C);
-        }
-    }
-    if (mine) {
-        float ps = 0.f;
-        if (active) {
-            const int64_t off = (int64_t)col * VEC;
-            F acc = load_g<VEC>(carry + ((int64_t)2 * w0 + 1) * D + off);
-            F cmp = zero_vec<VEC>();  // compensated (Kahan) sum, as in k_sp_segsum
-            constexpr int kB = 8;
-            for (int qb = w0 + 1; qb <= w1; qb += kB) {
-                F v[kB];
+    const int2 cut = ((int)(blockIdx.x / NS) < nw1 && n_valid > 0 && bd < workers_of(n_valid, nw1, rg)) ? cuts[bd] : make_int2(-1, 0);
+    const bool mine = cut.x >= 0;
+    // pieces q0 .. q1 of the run that began in worker w (piece 0: its last
+    // piece; piece q: the first piece of worker w + q, zero where that range is
+    // empty), compensated as in k_sp_segsum
+    const int64_t off = (int64_t)(active ? col : DV - 1) * VEC;
+    auto sum_pieces = [&](int w, int q0, int q1) {
+        F acc = zero_vec<VEC>();
+        F cmp = zero_vec<VEC>();
+        constexpr int kB = 12;
+        for (int qb = q0; qb <= q1; qb += kB) {
+            F v[kB];
 #pragma unroll
-                for (int k = 0; k < kB; ++k) {
-                    // workers with an empty range wrote zero pieces
-                    const int q = qb + k;
-                    v[k] = (q <= w1) ? load_g<VEC>(carry + ((int64_t)2 * q) * D + off) : zero_vec<VEC>();
-                }
-#pragma unroll
-                for (int k = 0; k < kB; ++k)
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) {
-                        const float y = comp(v[k], e) - comp(cmp, e);
-                        const float t = comp(acc, e) + y;
-                        set_comp(cmp, e, (t - comp(acc, e)) - y);
-                        set_comp(acc, e, t);
-                    }
+            for (int k = 0; k < kB; ++k) {
+                const int q = qb + k;
+                v[k] = (q <= q1) ? load_g<VEC>(carry + ((int64_t)2 * (w + q) + (q == 0)) * D + off) : zero_vec<VEC>();
             }
 #pragma unroll
-            for (int e = 0; e < VEC; ++e)
-                set_comp(acc, e, comp(acc, e) - comp(cmp, e));
+            for (int k = 0; k < kB; ++k)
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) {
+                    const float y = comp(v[k], e) - comp(cmp, e);
+                    const float t = comp(acc, e) + y;
+                    set_comp(cmp, e, (t - comp(acc, e)) - y);
+                    set_comp(acc, e, t);
+                }
+        }
+#pragma unroll
+        for (int e = 0; e < VEC; ++e)
+            set_comp(acc, e, comp(acc, e) - comp(cmp, e));
+        return acc;
+    };
+    auto finish = [&](const F &acc, int u) {  // by a whole group
+        float ps = 0.f;
+        if (active) {
             *reinterpret_cast<F *>(S + (int64_t)u * D + off) = acc;
 #pragma unroll
             for (int e = 0; e < VEC; ++e) {
@@ -717,22 +820,55 @@ k_sp_carry(const int32_t *__restrict__ segidx, const int32_t *__restrict__ segof
             ps += __shfl_xor_sync(0xffffffffu, ps, o);
         if (lane == 0)
             red[warp] = ps;
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        group_bar(g, rg, tpb);
+        if (l == 0) {
             float t = 0.f;
-            for (int k = 0; k < kWarps; ++k)
-                t += red[k];
+            for (int k = 0; k < wpg; ++k)
+                t += red[g * wpg + k];
             rowpart[(int64_t)u * NS + sigma] = t;
         }
-    }
-    // CTA b of this kernel and CTA b of k_sp_segsum share worker bd - 1 and
-    // slice sigma: add this run's column sums to that CTA's partial row
-    // (its value plus this one, in that order)
-    if (active && mine) {
-        float *out = colpart + (int64_t)blockIdx.x * D;
+        group_bar(g, rg, tpb);
+    };
+    // a run of many pieces is added by all the CTA's groups, a stretch each
+    const bool many = rg > 1 && mine && cut.y - (bd - 1) >= kManyPieces;
+    if (l == 0)
+        shared_cut[g] = many ? make_int3(cut.x, bd - 1, cut.y) : make_int3(-1, 0, 0);
+    if (mine && !many)  // uniform over the group
+        finish(sum_pieces(bd - 1, 0, cut.y - (bd - 1)), cut.x);
+    if (__syncthreads_or(many))
+        for (int q = 0; q < rg; ++q) {
+            const int3 run = shared_cut[q];
+            if (run.x < 0)
+                continue;
+            const int n = run.z - run.y + 1, per = (n + rg - 1) / rg;
+            const F part = sum_pieces(run.y, g * per, (g + 1) * per < n ? (g + 1) * per - 1 : n - 1);
 #pragma unroll
-        for (int e = 0; e < VEC; ++e)
-            out[col * VEC + e] += colacc[e];
+            for (int e = 0; e < VEC; ++e)
+                comb[(g * tpb + l) * VEC + e] = comp(part, e);
+            __syncthreads();
+            if (g == q) {
+                F acc = zero_vec<VEC>(), cmp = zero_vec<VEC>();
+                for (int k = 0; k < rg; ++k)
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) {
+                        const float y = comb[(k * tpb + l) * VEC + e] - comp(cmp, e);
+                        const float t = comp(acc, e) + y;
+                        set_comp(cmp, e, (t - comp(acc, e)) - y);
+                        set_comp(acc, e, t);
+                    }
+#pragma unroll
+                for (int e = 0; e < VEC; ++e)
+                    set_comp(acc, e, comp(acc, e) - comp(cmp, e));
+                finish(acc, run.x);
+            }
+            __syncthreads();
+        }
+    // CTA b of this kernel and CTA b of k_sp_segsum share the workers bd - 1
+    // and slice sigma: add these runs' column sums to that CTA's partial row
+    if (__syncthreads_or(mine)) {
+        const int col0 = sigma * tpb * VEC;
+        combine_groups<VEC, true>(colacc, comb, colpart + (int64_t)blockIdx.x * D, g, l, tpb, rg, col0,
+                                  col0 + tpb * VEC < D ? tpb * VEC : D - col0);
     }
 }
 
@@ -886,10 +1022,10 @@ void launch_count_scan(const SparseArgs &a, Tracer &tr, float *r, const EmaPair 
     tr.mark();
 }
 
-// Every occurrence to its place in (id, occurrence) order; bounds of the nw
-// workers of the segment sums.
+// Every occurrence to its place in (id, occurrence) order; bounds of the
+// workers of the segment sums (rg groups in each of nw1 CTAs per slice).
 template <typename IdT>
-void launch_place_order(const SparseArgs &a, Tracer &tr, int nw)
+void launch_place_order(const SparseArgs &a, Tracer &tr, int nw1, int rg)
 {
     unsigned char *ws = a.ws;
     const Layout &L = a.lay;
@@ -909,7 +1045,8 @@ void launch_place_order(const SparseArgs &a, Tracer &tr, int nw)
     launch_k(k_sp_order, dim3(nbig + (int)((a.N + kOrderThreads - 1) / kOrderThreads)), dim3(kOrderThreads), 0, a.stream, tr.pdl(), placed, segidx, segoff,
              reinterpret_cast<int32_t *>(ws + L.sp_long),
              reinterpret_cast<int32_t *>(ws + L.sp_rng) + kScanCounters - 1, sc, a.N, nbig,
-             reinterpret_cast<int32_t *>(ws + L.sp_perm), reinterpret_cast<int32_t *>(ws + L.sp_bounds), nw);
+             reinterpret_cast<int32_t *>(ws + L.sp_perm), reinterpret_cast<int32_t *>(ws + L.sp_bounds),
+             reinterpret_cast<int2 *>(ws + L.sp_cuts), nw1, rg);
     tr.mark();
 }
 
@@ -945,37 +1082,45 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     auto *perm = reinterpret_cast<int32_t *>(ws + L.sp_perm);
     auto *segidx = reinterpret_cast<int32_t *>(ws + L.sp_segidx);
     auto *uniq = reinterpret_cast<int32_t *>(ws + L.sp_uniq);
-    auto *segoff = reinterpret_cast<int32_t *>(ws + L.sp_segoff);
     auto *slot = reinterpret_cast<int32_t *>(ws + L.sp_slot);
     auto *single = reinterpret_cast<int32_t *>(ws + L.sp_single);
     auto *rowpart = reinterpret_cast<float *>(ws + L.sp_rowpart);
     auto *carry = reinterpret_cast<float *>(ws + L.sp_carry);
     auto *bounds = reinterpret_cast<int32_t *>(ws + L.sp_bounds);
+    auto *cuts = reinterpret_cast<int2 *>(ws + L.sp_cuts);
     auto *S = reinterpret_cast<float *>(ws + L.sp_rows);
     auto *colpart = reinterpret_cast<float *>(ws + L.colpart);
     auto *rsum_part = reinterpret_cast<float *>(ws + L.rsum_part);
     auto *csum_part = reinterpret_cast<float *>(ws + L.csum_part);
     const int D = (int)a.D;
     const int DV = D / VEC;
-    const int NS = (DV + kThreads - 1) / kThreads;
+    const SumMap map = sum_map(DV);
+    const int NS = map.NS;
+    const dim3 sum_threads(map.rg * map.tpb);
     Tracer tr{a.trace, a.n_trace, 0, a.stream};
 
     tr.mark();
     const int G = kSparseCtas;
-    const int nw = G / NS;
     const StepConsts kc = make_consts(a.beta2, a.one_minus_beta2, a.V, a.D, a.inv_bc);
     if (a.ids64) {
         launch_count_scan<int64_t>(a, tr, a.r, kc.ema, rsum_part);
-        launch_place_order<int64_t>(a, tr, nw);
+        launch_place_order<int64_t>(a, tr, G / NS, map.rg);
     } else {
         launch_count_scan<int32_t>(a, tr, a.r, kc.ema, rsum_part);
-        launch_place_order<int32_t>(a, tr, nw);
+        launch_place_order<int32_t>(a, tr, G / NS, map.rg);
     }
-    launch_k(k_sp_segsum<VEC>, dim3(G), dim3(kThreads), 0, a.stream, tr.pdl(), a.rows, perm, segidx, sc, S,
-             rowpart, carry, colpart, bounds, D, NS, reinterpret_cast<int32_t *>(ws + L.sp_rng), kScanCounters);
+    auto *segsum = sum_threads.x > 192   ? k_sp_segsum<VEC, 256>
+                   : sum_threads.x > 128 ? k_sp_segsum<VEC, 192>
+                                         : k_sp_segsum<VEC, 128>;
+    // the ring and the static arrays together pass 48 KiB
+    const cudaError_t e = cudaFuncSetAttribute(segsum, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    if (e != cudaSuccess)
+        return e;
+    launch_k(segsum, dim3(G), sum_threads, kRingBytes, a.stream, tr.pdl(), a.rows, perm, segidx, sc, S, rowpart, carry,
+             colpart, bounds, D, map, reinterpret_cast<int32_t *>(ws + L.sp_rng), kScanCounters);
     tr.mark();
-    launch_k(k_sp_carry<VEC>, dim3(G), dim3(kThreads), 0, a.stream, tr.pdl(), segidx, segoff, bounds, sc,
-             carry, S, rowpart, colpart, D, NS, nw);
+    launch_k(k_sp_carry<VEC>, dim3(G), sum_threads, 0, a.stream, tr.pdl(), cuts, sc, carry, S, rowpart,
+             colpart, D, map);
     tr.mark();
     // the touched rows' r and the column pass in one launch (a row per thread
     // for up to one CTA per SM: more would only wait for a place); the per-CTA
@@ -986,7 +1131,7 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     const NormSource norm{rsum_part, nr + GU, csum_part, (D + kStateCols - 1) / kStateCols, nullptr, nullptr, D};
     // (segment-sum CTA b writes only the columns of its slice b % NS)
     launch_state(colpart, G, rsum_part, a.c, csum_part, sc, a.V, D, kc, a.stream, tr.pdl(), a.r, slot,
-                 rowpart, NS, GU, uniq, nr, NS, kThreads * VEC);
+                 rowpart, NS, GU, uniq, nr, NS, map.tpb * VEC);
     tr.mark();
     // one launch per column panel (one unless D is wider than a CTA's row)
     const int np = a.map.npanels, pw = a.map.pw;
