@@ -61,6 +61,8 @@ constexpr int kScanCtas = kGridCtas;
 constexpr int kScanMin = 256;
 constexpr int kScanCounters = 2 * kScanCtas + 1;  // two per range, then the number of long runs
 constexpr int kLongRun = 128;
+// Batches of up to kSmallN occurrences are deduped by comparing all pairs.
+constexpr int kSmallN = 4096;
 
 // Workspace layout (byte offsets, each 256-byte aligned).
 struct Layout {

@@ -20,7 +20,8 @@
 //             puts every occurrence at its run's start plus its arrival
 //             number; k_sp_order sorts each run by occurrence, so that
 //             arrival order (the only thing that varies from run to run)
-//             leaves no trace.
+//             leaves no trace.  A small batch takes one kernel instead,
+//             k_sp_dedup_small.
 //   segsum    k_sp_segsum, k_sp_carry: the summed gradient row of every
 //             distinct id, adding its occurrences in increasing occurrence
 //             order (compensated fp32 sums); per (id, column slice) sums of
@@ -40,6 +41,8 @@
 // launch and waits (griddepcontrol.wait) before it reads earlier results.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "ember_device.cuh"
 #include "ember_internal.h"
@@ -467,6 +470,135 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
             at += __shfl_sync(0xffffffffu, x, 31);
         }
         __syncthreads();  // the bitmap is cleared for the next pair
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Dedup of a small batch (N <= kSmallN) in one launch: a warp per occurrence
+// compares its id with every other one in shared memory, which gives the
+// occurrence's sorted position at once.  Runs are numbered by their first
+// position (uniq holds -1 elsewhere, and n_unique is the number of
+// positions), so nothing has to be scanned.  N^2 comparisons: 1 us for 1024
+// occurrences; the four kernels above, a few trips to L2 and a launch each,
+// take 13.7 us.  The CTAs from `nkey` on decay r on the rows outside the
+// batch, kScanTile-sized ranges as in k_sp_scan, from a bitmap of the ids.
+// ---------------------------------------------------------------------------
+template <typename IdT>
+__global__ void __launch_bounds__(kSpThreads)
+k_sp_dedup_small(const IdT *__restrict__ ids, int N, int64_t V, int32_t *__restrict__ perm,
+                 int32_t *__restrict__ segidx, int32_t *__restrict__ uniq, int32_t *__restrict__ single,
+                 int32_t *__restrict__ bounds, int2 *__restrict__ cuts, int nw1, int rg, DevScalars *sc, int nkey,
+                 int64_t len, float *__restrict__ r, EmaPair ema, float *__restrict__ rsum_part)
+{
+    constexpr int kW = kSpThreads / 32;
+    constexpr int kNone = 0x7fffffff;  // a skipped id: V < 2^31, so every valid one is below
+    constexpr int kBitWords = 2048;
+    __shared__ __align__(16) int sid[kSmallN];
+    __shared__ unsigned bits[kBitWords];
+    __shared__ float wr[kW];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int npad = (N + 127) / 128 * 128;
+    grid_dep_wait();  // first kernel of a step: returns at once
+    grid_dep_launch();
+    bool bad = false;
+    for (int q = tid; q < npad; q += kSpThreads) {
+        int x = kNone;
+        if (q < N) {
+            const int64_t id = (int64_t)ids[q];
+            if (id >= 0 && id < V)
+                x = (int)id;
+            else
+                bad = true;
+        }
+        sid[q] = x;
+    }
+    if (bad && blockIdx.x == 0)
+        atomicOr(&sc->flags, kFlagIdRange);
+    __syncthreads();
+    if ((int)blockIdx.x < nkey) {
+        const int k = (int)blockIdx.x * kW + w;
+        if (k >= N)
+            return;
+        const int x = sid[k];
+        int less = 0, before = 0, same = 0, valid = 0;
+        for (int q = lane * 4; q < npad; q += 128) {
+            const int4 v = *reinterpret_cast<const int4 *>(sid + q);
+            const int y[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                less += y[e] < x;
+                same += y[e] == x;
+                before += y[e] == x && q + e < k;
+                valid += y[e] != kNone;
+            }
+        }
+        less = __reduce_add_sync(0xffffffffu, less);
+        same = __reduce_add_sync(0xffffffffu, same);
+        before = __reduce_add_sync(0xffffffffu, before);
+        valid = __reduce_add_sync(0xffffffffu, valid);
+        if (k == 0 && lane == 0)
+            sc->n_unique = sc->n_valid = valid;
+        if (x == kNone)
+            return;
+        const int p = less + before;
+        if (lane == 0) {
+            perm[p] = k;
+            segidx[p] = less;
+            uniq[p] = before == 0 ? x : -1;
+            single[p] = same == 1 ? k : -1;
+        }
+        // the workers that start here (equal shares of the positions), and
+        // the run each start cuts, as in k_sp_order
+        const int nw = workers_of(valid, nw1, rg);
+        for (int q = (p * nw + valid - 1) / valid + lane; q < nw && q * valid / nw == p; q += 32) {
+            bounds[q] = p;
+            int2 cut = make_int2(-1, 0);
+            if (before > 0 && q > 0 && (q - 1) * valid / nw <= less) {
+                int to = (less + same - 1) * nw / valid;  // the worker whose range holds the run's last position
+                while (to + 1 < nw && (to + 1) * valid / nw <= less + same - 1)
+                    ++to;
+                cut = make_int2(less, to);
+            }
+            cuts[q] = cut;
+        }
+        if (p + 1 == valid && lane == 0)
+            bounds[nw] = valid;
+        return;
+    }
+    const int64_t b = (int)blockIdx.x - nkey;
+    const int64_t i1 = (b + 1) * len < V ? (b + 1) * len : V;
+    float rsum = 0.f;
+    for (int64_t c0 = b * len; c0 < i1; c0 += 32 * kBitWords) {
+        const int n = (int)(i1 - c0 < 32 * kBitWords ? i1 - c0 : 32 * kBitWords);
+        for (int q = tid; q < (n + 31) / 32; q += kSpThreads)
+            bits[q] = 0u;
+        __syncthreads();
+        for (int q = tid; q < N; q += kSpThreads) {
+            const int64_t o = sid[q] - c0;
+            if (o >= 0 && o < n)
+                atomicOr(&bits[o >> 5], 1u << (o & 31));
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int q = tid; q < n; q += kSpThreads)
+            if (!(bits[q >> 5] >> (q & 31) & 1u)) {
+                const float rn = ema_pair(ema, r[c0 + q], 0.f);
+                r[c0 + q] = rn;
+                rsum += rn;
+            }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1)
+        rsum += __shfl_xor_sync(0xffffffffu, rsum, o);
+    if (lane == 0)
+        wr[w] = rsum;
+    __syncthreads();
+    if (tid == 0) {
+        float t = 0.f;
+        for (int q = 0; q < kW; ++q)
+            t += wr[q];
+        rsum_part[b] = t;
     }
 }
 
@@ -1102,7 +1234,20 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     tr.mark();
     const int G = kSparseCtas;
     const StepConsts kc = make_consts(a.beta2, a.one_minus_beta2, a.V, a.D, a.inv_bc);
-    if (a.ids64) {
+    if (a.N > 0 && a.N <= kSmallN) {
+        const int nkey = (int)((a.N + kSpThreads / 32 - 1) / (kSpThreads / 32));
+        auto go = [&](auto *ids) {
+            using IdT = std::remove_const_t<std::remove_pointer_t<decltype(ids)>>;
+            launch_k(k_sp_dedup_small<IdT>, dim3(nkey + scan_ranges(a.V)), dim3(kSpThreads), 0, a.stream, tr.pdl(), ids,
+                     (int)a.N, a.V, perm, segidx, uniq, single, bounds, cuts, G / NS, map.rg, sc, nkey, scan_len(a.V),
+                     a.r, kc.ema, rsum_part);
+        };
+        if (a.ids64)
+            go(static_cast<const int64_t *>(a.ids));
+        else
+            go(static_cast<const int32_t *>(a.ids));
+        tr.mark();
+    } else if (a.ids64) {
         launch_count_scan<int64_t>(a, tr, a.r, kc.ema, rsum_part);
         launch_place_order<int64_t>(a, tr, G / NS, map.rg);
     } else {
