@@ -1018,8 +1018,8 @@ __device__ __forceinline__ void cp_async8(void *smem, const void *gmem)
                  "l"(gmem)
                  : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 template <int VEC, int CPT, int R, bool BF16, bool ASYNC>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
@@ -1511,9 +1511,9 @@ cudaError_t launch_dense_step(const DenseArgs &a)
         const bool half = reduce_rows_per_thread(a.V, a.D, a.map) == 8;
         switch (a.map.cpt) {
         case 1: return half ? launch_dense_t<1, 1, 8>(a) : launch_dense_t<1, 1, 16>(a);
-        case 2: return launch_dense_t<1, 2, 8>(a);
-        case 4: return launch_dense_t<1, 4, 4>(a);
-        case 8: return launch_dense_t<1, 8, 2>(a);
+        case 2: return launch_dense_t<1, 2, 16>(a);
+        case 4: return launch_dense_t<1, 4, 8>(a);
+        case 8: return launch_dense_t<1, 8, 4>(a);
         }
     }
     return cudaErrorInvalidValue;

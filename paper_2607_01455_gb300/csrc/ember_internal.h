@@ -200,7 +200,7 @@ inline int dense_parts(int64_t V, int64_t D)
 }
 
 // Rows a thread of the reduce pass takes per iteration (its rows in flight):
-// 16 / cpt, halved for rows of one access per thread when a CTA's rows fit
+// 16 / cpt (32 / cpt with 4-byte accesses of several per row), halved for rows of one access per thread when a CTA's rows fit
 // in half an iteration, so that on a small table every thread reduces (and,
 // in the one-launch step, updates) half as many rows.  A function of (V, D)
 // and the column map only, like the grid: every form of the step forms the
@@ -209,7 +209,7 @@ inline int reduce_rows_per_thread(int64_t V, int64_t D, const ColMap &m)
 {
     const int r = (16 / m.cpt) < 1 ? 1 : 16 / m.cpt;
     if (m.cpt != 1)
-        return r;
+        return m.vec == 1 ? 2 * r : r;
     const int nparts = dense_parts(V, D);
     const int64_t rows = (V + nparts - 1) / nparts;
     return rows <= (int64_t)(kThreads / m.tpr) * (r / 2) ? r / 2 : r;

@@ -329,13 +329,17 @@ __device__ __forceinline__ int64_t cost_target(int w, int nw, int64_t C)
     return ((int64_t)w * C) / nw;
 }
 
-// Workers in use: of the nw1 rg groups of a slice's CTAs (group g of CTA b is
-// worker g nw1 + b), nw1 times as many groups as have kMinRows occurrences
-// each.  A worker of fewer rows would mostly wait for its indices.  A function of the valid ids, so that skipped ones
-// change nothing.
-constexpr int kMinRows = 16;
+// Workers in use, of the nw1 rg groups of a slice's CTAs (group g of CTA b is
+// worker g nw1 + b): nw1 times as many groups as have kMinRows occurrences
+// each, or, of a small batch, as many workers as have kFewRows (a batch of
+// rows in flight).  More workers would cut frequent ids into more pieces, for
+// the carry to add up one after another.  A function of the valid ids, so
+// that skipped ones change nothing.
+constexpr int kMinRows = 16, kFewRows = 8;
 __device__ __forceinline__ int workers_of(int n_valid, int nw1, int rg)
 {
+    if (n_valid < kFewRows * nw1)
+        return n_valid < kFewRows ? 1 : n_valid / kFewRows;
     const int most = n_valid / (kMinRows * nw1);
     return nw1 * (most < 1 ? 1 : most < rg ? most : rg);
 }
