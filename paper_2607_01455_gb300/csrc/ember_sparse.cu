@@ -37,8 +37,8 @@
 //   apply     k_sp_apply: the update of the touched rows only (once per
 //             column panel for tables wider than a CTA holds).
 //
-// Every kernel after the first is launched with programmatic dependent
-// launch and waits (griddepcontrol.wait) before it reads earlier results.
+// Every kernel is launched with programmatic dependent launch (but see
+// small_first_pdl) and waits (griddepcontrol.wait) before it reads anything.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -90,6 +90,14 @@ k_sp_count(const IdT *__restrict__ ids, int64_t N, int64_t V, int32_t *__restric
     __shared__ int cnt[2 * kScanCtas];
     const int tid = threadIdx.x, lane = tid & 31;
     const int64_t k0 = (int64_t)blockIdx.x * kCountKeys + tid;
+    for (int q = tid; q < kTab; q += kSpThreads) {
+        tag[q] = -1;
+        num[q] = 0;
+    }
+    for (int q = tid; q < 2 * nrange; q += kSpThreads)
+        cnt[q] = 0;
+    grid_dep_wait();  // whatever ran before on the stream
+    grid_dep_launch();
     int id[kPer];
     bool bad = false;
 #pragma unroll
@@ -104,14 +112,6 @@ k_sp_count(const IdT *__restrict__ ids, int64_t N, int64_t V, int32_t *__restric
                 bad = true;  // skipped
         }
     }
-    for (int q = tid; q < kTab; q += kSpThreads) {
-        tag[q] = -1;
-        num[q] = 0;
-    }
-    for (int q = tid; q < 2 * nrange; q += kSpThreads)
-        cnt[q] = 0;
-    grid_dep_wait();  // first kernel of a step: returns at once
-    grid_dep_launch();
     __syncthreads();
     if (__any_sync(0xffffffffu, bad) && lane == 0)
         atomicOr(&sc->flags, kFlagIdRange);
@@ -502,7 +502,7 @@ k_sp_dedup_small(const IdT *__restrict__ ids, int N, int64_t V, int32_t *__restr
     __shared__ float wr[kW];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int npad = (N + 127) / 128 * 128;
-    grid_dep_wait();  // first kernel of a step: returns at once
+    grid_dep_wait();  // whatever ran before on the stream
     grid_dep_launch();
     bool bad = false;
     for (int q = tid; q < npad; q += kSpThreads) {
@@ -1105,21 +1105,14 @@ struct Tracer {
     const cudaEvent_t *ev;
     int n, next;
     cudaStream_t s;
-    bool launched = false;  // a kernel of this step is already on the stream
     void mark()
     {
         if (ev && next < n)
             cudaEventRecord(ev[next], s);
         ++next;
     }
-    // programmatic dependent launch for every kernel after the first,
-    // unless events are recorded between the kernels
-    bool pdl()
-    {
-        const bool p = launched && ev == nullptr;
-        launched = true;
-        return p;
-    }
+    // programmatic dependent launch, unless events are recorded between the kernels
+    bool pdl() const { return ev == nullptr; }
 };
 
 // Ids per range of k_sp_count and k_sp_scan, and the number of ranges: a
@@ -1208,6 +1201,14 @@ __global__ void k_sp_export(const int32_t *__restrict__ uniq, const int32_t *__r
         *n_unique_out = U;
 }
 
+// Whether the one dedup kernel of a small batch may be launched while the
+// kernel before it on the stream is still running.  With few CTAs it gains
+// its launch latency, 128 ids over 67019 x 480: 22.7 us per step against 24.0.
+// With many, its waiting CTAs cost the kernel before it more: 1024 ids over
+// 50257 x 768 take 28.6 us with it and 26.6 without, 1384 over 5656 x 96 31.6
+// and 27.9.
+bool small_first_pdl(int64_t N) { return N <= 256; }
+
 template <int VEC, int CPT>
 cudaError_t launch_sparse_t(const SparseArgs &a)
 {
@@ -1242,7 +1243,8 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
         const int nkey = (int)((a.N + kSpThreads / 32 - 1) / (kSpThreads / 32));
         auto go = [&](auto *ids) {
             using IdT = std::remove_const_t<std::remove_pointer_t<decltype(ids)>>;
-            launch_k(k_sp_dedup_small<IdT>, dim3(nkey + scan_ranges(a.V)), dim3(kSpThreads), 0, a.stream, tr.pdl(), ids,
+            launch_k(k_sp_dedup_small<IdT>, dim3(nkey + scan_ranges(a.V)), dim3(kSpThreads), 0, a.stream,
+                     tr.pdl() && small_first_pdl(a.N), ids,
                      (int)a.N, a.V, perm, segidx, uniq, single, bounds, cuts, G / NS, map.rg, sc, nkey, scan_len(a.V),
                      a.r, kc.ema, rsum_part);
         };
