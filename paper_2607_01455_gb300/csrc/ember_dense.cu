@@ -12,7 +12,7 @@
 //   state   O(D * CTAs) work: per column the exact fixed-point total of the
 //           per-CTA partial sums (ember_device.cuh), the column EMA
 //           c_j <- beta2 c_j + (1-beta2) mean_i g^2, and the sum of the new c
-//           per 32 columns.
+//           per 8 columns.
 //   apply   every CTA forms s = sqrt(mean rhat * mean chat) (the
 //           geometric-mean normaliser) from the sums of r and c, then reads
 //           G and W, writes W:
@@ -262,14 +262,18 @@ __device__ __forceinline__ void reduce_rows(const float *__restrict__ G, float *
 }
 
 // ---------------------------------------------------------------------------
-// Column pass of one group of kStateCols = 32 columns, by a whole CTA of
-// kStateThreads threads: lane l of every warp owns column j0 + l.
-// Source: the partial rows colpart[b * D + j], b < nparts (warp w reads rows
-// w, w + 8, ...; the column's total is their exact fixed-point sum at the
-// largest key among them), or, with `sums` set, the totals already formed
-// elsewhere (the all-reduce of a row-sharded step) at scales[j].
+// Column pass of one group of kStateCols = 8 columns (one 32-byte sector of
+// each partial row), by a whole CTA of kStateThreads threads: lane l of warp w
+// owns column j0 + (l & 7) and reads every 32nd partial row from 4 w + l / 8
+// on; the column's total is their exact fixed-point sum at the largest key
+// among them.  Or, with `sums` set, the totals already formed elsewhere (the
+// all-reduce of a row-sharded step) at scales[j].
 // Writes c_j <- beta2 c_j + (1 - beta2) total_j / V and csum_part[group] =
 // the fp32 sum of the group's new c (a fixed butterfly).
+//   Bound by latency: one trip to L2 for the partials, two barriers, and the
+// 64-bit arithmetic of a thread's rows.  Groups of 8 columns spread that
+// arithmetic over four times as many SMs as groups of 32 (whose CTAs of 1024
+// threads spent most of 4.8 us on it).
 // ---------------------------------------------------------------------------
 struct ColSource {
     const float *colpart;                 // [nparts][D]
@@ -283,33 +287,81 @@ struct ColSource {
 };
 
 constexpr int kStateWarps = kStateThreads / 32;
-// partial rows per warp held in registers by the column pass (the dense
-// step's 304 rows, the sparse step's 456 and those of an LM head of up to
-// 131072 rows fit; more take two passes through L2)
+// partial rows per thread held in registers by the column pass (the dense and
+// sparse steps' 304 rows and those of an LM head of up to 131072 rows fit;
+// more take two passes through L2), out of kStateSub threads per column
 constexpr int kRegParts = 32;
-static_assert(kRegParts * kStateWarps >= kGridCtas, "the dense step's partial rows fit the register path");
+constexpr int kStateSub = kStateThreads / kStateCols;
+static_assert(kRegParts * kStateSub >= kPartRows, "the dense and sparse steps' partial rows fit the register path");
+
+// Sum over the kStateCols lanes of a column group (a fixed butterfly).
+__device__ __forceinline__ float group_sum(float x)
+{
+#pragma unroll
+    for (int o = kStateCols / 2; o >= 1; o >>= 1)
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
 
 __device__ __forceinline__ void column_group(const ColSource &src, int group, float *__restrict__ c,
                                              float *__restrict__ csum_part, int D, const StepConsts &kc)
 {
-    __shared__ unsigned emax_sh[kStateWarps][32];
-    __shared__ unsigned long long ssum_sh[kStateWarps][32];
+    __shared__ unsigned emax_sh[kStateWarps][kStateCols];
+    __shared__ unsigned long long ssum_sh[kStateWarps][kStateCols];
     const int lane = threadIdx.x & 31;
     const int w = threadIdx.x >> 5;
-    const int j = group * kStateCols + lane;
+    const int jl = lane & (kStateCols - 1);
+    const int sub = threadIdx.x / kStateCols;  // this thread's first partial row
+    const int j = group * kStateCols + jl;
     const float c_old = (w == 0 && j < D) ? __ldcg(c + j) : 0.f;  // loaded with the partials
     // the partial rows of this group's slice: b = sigma + p pstride, p < np
     // (the other rows are zero in these columns and add nothing)
     const int sigma = (src.pstride > 1) ? (group * kStateCols) / src.pcols : 0;
     const int np = (src.nparts - sigma + src.pstride - 1) / src.pstride;
+    auto load = [&](int p) {
+        return (p < np && j < D) ? __ldcg(src.colpart + (int64_t)(sigma + p * src.pstride) * D + j) : 0.f;
+    };
+    // largest key and sum over the lanes of a warp that share a column, then
+    // over the warps through shared memory
+    auto max_all = [&](unsigned e) {
+#pragma unroll
+        for (int o = 16; o >= kStateCols; o >>= 1)
+            e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+        if (lane < kStateCols)
+            emax_sh[w][lane] = e;
+        __syncthreads();
+        unsigned E = 0;
+#pragma unroll
+        for (int q = 0; q < kStateWarps; ++q)
+            E = max(E, emax_sh[q][jl]);
+        return E;
+    };
+    auto sum_all = [&](unsigned long long s) {  // valid in warp 0
+#pragma unroll
+        for (int o = 16; o >= kStateCols; o >>= 1)
+            s += shfl_xor_u64(s, o);
+        if (lane < kStateCols)
+            ssum_sh[w][lane] = s;
+        __syncthreads();
+        unsigned long long S = 0;
+        if (w == 0)
+#pragma unroll
+            for (int q = 0; q < kStateWarps; ++q)
+                S += ssum_sh[q][jl];
+        return S;
+    };
     unsigned long long S = 0;
     unsigned E = 0;
-    if (src.sums == nullptr && np <= kRegParts * kStateWarps) {
-        // up to kRegParts partial rows per warp: one trip to L2, the values
-        // kept in registers for both the largest key and the sum
-        // (in chunks of 8, the chunks past this warp's last row skipped)
+    if (src.sums != nullptr) {
+        if (w == 0 && j < D) {
+            S = src.sums[j];
+            E = src.scales[j];
+        }
+    } else if (np <= kRegParts * kStateSub) {
+        // one trip to L2, the values kept in registers for both the largest
+        // key and the sum (in chunks, those past the last row skipped)
         constexpr int kChunk = 8;
-        const int kv = (np - w + kStateWarps - 1) / kStateWarps;  // this warp's rows
+        const int kv = (np - sub + kStateSub - 1) / kStateSub;  // this thread's rows
         float v[kRegParts];
         unsigned e = 0;
 #pragma unroll
@@ -317,10 +369,8 @@ __device__ __forceinline__ void column_group(const ColSource &src, int group, fl
             if (k0 >= kv)
                 break;
 #pragma unroll
-            for (int k = k0; k < k0 + kChunk; ++k) {
-                const int p = w + k * kStateWarps;
-                v[k] = (p < np && j < D) ? __ldcg(src.colpart + (int64_t)(sigma + p * src.pstride) * D + j) : 0.f;
-            }
+            for (int k = k0; k < k0 + kChunk; ++k)
+                v[k] = load(sub + k * kStateSub);
         }
 #pragma unroll
         for (int k0 = 0; k0 < kRegParts; k0 += kChunk) {
@@ -330,11 +380,7 @@ __device__ __forceinline__ void column_group(const ColSource &src, int group, fl
             for (int k = k0; k < k0 + kChunk; ++k)
                 e = max(e, fx_key(v[k]));
         }
-        emax_sh[w][lane] = e;
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < kStateWarps; ++q)
-            E = max(E, emax_sh[q][lane]);
+        E = max_all(e);
         unsigned long long s = 0;
 #pragma unroll
         for (int k0 = 0; k0 < kRegParts; k0 += kChunk) {
@@ -344,71 +390,46 @@ __device__ __forceinline__ void column_group(const ColSource &src, int group, fl
             for (int k = k0; k < k0 + kChunk; ++k)
                 s += fx_of(v[k], E);
         }
-        ssum_sh[w][lane] = s;
-        __syncthreads();
-        if (w == 0)
-#pragma unroll
-            for (int q = 0; q < kStateWarps; ++q)
-                S += ssum_sh[q][lane];
-    } else if (src.sums == nullptr) {
+        S = sum_all(s);
+    } else {
         constexpr int kBatch = 16;
         // pass 1: the largest key of the column (loads batched for latency)
         unsigned e = 0;
-        if (j < D)
-            for (int p0 = w; p0 < np; p0 += kBatch * kStateWarps) {
-                float v[kBatch];
+        for (int p0 = sub; p0 < np; p0 += kBatch * kStateSub) {
+            float v[kBatch];
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k) {
-                    const int p = p0 + k * kStateWarps;
-                    v[k] = (p < np) ? __ldcg(src.colpart + (int64_t)(sigma + p * src.pstride) * D + j) : 0.f;
-                }
+            for (int k = 0; k < kBatch; ++k)
+                v[k] = load(p0 + k * kStateSub);
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k)
-                    e = max(e, fx_key(v[k]));
-            }
-        emax_sh[w][lane] = e;
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < kStateWarps; ++q)
-            E = max(E, emax_sh[q][lane]);
+            for (int k = 0; k < kBatch; ++k)
+                e = max(e, fx_key(v[k]));
+        }
+        E = max_all(e);
         // pass 2: the exact total (the partials are still in L2)
         unsigned long long s = 0;
-        if (j < D)
-            for (int p0 = w; p0 < np; p0 += kBatch * kStateWarps) {
-                float v[kBatch];
+        for (int p0 = sub; p0 < np; p0 += kBatch * kStateSub) {
+            float v[kBatch];
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k) {
-                    const int p = p0 + k * kStateWarps;
-                    v[k] = (p < np) ? __ldcg(src.colpart + (int64_t)(sigma + p * src.pstride) * D + j) : 0.f;
-                }
+            for (int k = 0; k < kBatch; ++k)
+                v[k] = load(p0 + k * kStateSub);
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k)
-                    s += fx_of(v[k], E);
-            }
-        ssum_sh[w][lane] = s;
-        __syncthreads();
-        if (w == 0)
-#pragma unroll
-            for (int q = 0; q < kStateWarps; ++q)
-                S += ssum_sh[q][lane];
-    } else if (w == 0 && j < D) {
-        S = src.sums[j];
-        E = src.scales[j];
+            for (int k = 0; k < kBatch; ++k)
+                s += fx_of(v[k], E);
+        }
+        S = sum_all(s);
     }
     if (w == 0) {
         float cn = 0.f;
         if (j < D) {
             const float m = fx_value(S, E) * kc.inv_V;
             cn = ema_pair(kc.ema, c_old, m);
-            c[j] = cn;
+            if (lane < kStateCols)
+                c[j] = cn;
         }
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1)
-            cn += __shfl_xor_sync(0xffffffffu, cn, o);
+        cn = group_sum(cn);
         if (lane == 0)
             csum_part[group] = cn;
     }
-    __syncthreads();  // the shared buffers are reused
 }
 
 // ---------------------------------------------------------------------------
@@ -429,7 +450,7 @@ k_reduce_dense(const float *__restrict__ G, float *__restrict__ r, float *__rest
 }
 
 // Column EMA.  The first ngroups CTAs each own one group of
-// 32 columns (column_group).  For the sparse and LM-head steps and a dense
+// kStateCols columns (column_group).  For the sparse and LM-head steps and a dense
 // step in column panels the remaining CTAs also do the row pass: r for every
 // row (touched rows of a sparse batch only) from the sums of g^2 per column
 // slice in `rowpart`, and the sum of the new r per CTA.
@@ -923,8 +944,8 @@ k_dense_cluster(SmallArgs a)
     // the column pass for every column, as column_group forms it
     const int lane = tid & 31, w = tid >> 5;
     const int ngroups = (D + kStateCols - 1) / kStateCols;
-    for (int q = w; q < ngroups; q += kThreads / 32) {
-        const int j = q * kStateCols + lane;
+    for (int q = w; q < (D + 31) / 32; q += kThreads / 32) {
+        const int j = q * 32 + lane;
         float v[kMaxClusterCtas];
         unsigned E = 0;
 #pragma unroll
@@ -942,11 +963,9 @@ k_dense_cluster(SmallArgs a)
             cn = ema_pair(a.kc.ema, cold[j], m);
             cnew[j] = cn;
         }
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1)
-            cn += __shfl_xor_sync(0xffffffffu, cn, o);
-        if (lane == 0)
-            csum_sh[q] = cn;
+        cn = group_sum(cn);
+        if (lane % kStateCols == 0 && j < D)
+            csum_sh[j / kStateCols] = cn;
     }
     const float r_total = block_fx_total<kThreads>([&](int b) { return ld_dsmem(&rsum_own, b); }, (int)nb);
     cluster_arrive();  // done reading the other CTAs' shared memory

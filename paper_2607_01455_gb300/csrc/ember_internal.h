@@ -23,13 +23,13 @@ constexpr int kSparseCtasPerSm = 2;  // of the sparse step's segment sums
 constexpr int kSparseCtas = kSms * kSparseCtasPerSm;
 constexpr int kPartRows = kSparseCtas > kGridCtas ? kSparseCtas : kGridCtas;
 
-// The state pass reduces 32 columns per CTA of kStateThreads threads (32
-// warps, so that each warp adds few per-CTA partial rows).  Its row pass runs
+// The state pass reduces kStateCols columns per CTA of kStateThreads threads
+// (32 threads per column, so that each adds few per-CTA partial rows).  Its row pass runs
 // up to kMaxRowCtas CTAs: about one row per thread for the LM-head step (whose
 // rows each sum ceil(D/256) slices) and for a dense step in column panels
 // (one slice per panel), and one touched row per thread for the sparse step.
-constexpr int kStateCols = 32;
-constexpr int kStateThreads = 1024;
+constexpr int kStateCols = 8;
+constexpr int kStateThreads = 256;
 constexpr int kMaxRowCtas = 1024;
 constexpr int kRsumParts = kMaxRowCtas > kGridCtas ? kMaxRowCtas : kGridCtas;
 
@@ -68,7 +68,7 @@ constexpr int kSmallN = 4096;
 struct Layout {
     size_t scalars;     // DevScalars
     size_t rsum_part;   // float[kRsumParts]            sum of new r per CTA
-    size_t csum_part;   // float[ceil(D/32)]            sum of new c per 32-column group
+    size_t csum_part;   // float[ceil(D/8)]             sum of new c per 8-column group
     size_t colpart;     // float[kPartRows * D]     column sums of g^2 per CTA
     // sparse step (present when max_sparse_N > 0), N = max_sparse_N
     size_t sp_arr;      // int32[N]      arrival number of each occurrence within its id
