@@ -72,24 +72,25 @@ __device__ __forceinline__ int warp_scan(int x, int lane)
 // ---------------------------------------------------------------------------
 
 // slot[id] <- how often the id occurs; arr[k] <- how many of its occurrences
-// arrived before occurrence k (any order: k_sp_order undoes it).  A CTA adds
-// up the equal ids of its kCountKeys occurrences in a hash table in shared
-// memory first and makes one global atomic per id: a frequent id's atomics
-// queue on one address at about 3 ns each (one per warp took 27 us on 262144
-// Zipf ids).  An id that finds its table entry taken goes to the map
-// directly.  rng[2 q], rng[2 q + 1]: distinct ids and occurrences in the ids
+// arrived before occurrence k (any order: k_sp_order undoes it).  A warp's
+// equal ids make one global atomic (one occurrence per thread), or, with
+// TABLE, those of the CTA's kCountKeys occurrences, added up in a hash table in
+// shared memory first: a frequent id's atomics queue on one address at about
+// 3 ns each.  An id that finds its table entry taken goes to the map directly.
+// rng[2 q], rng[2 q + 1]: distinct ids and occurrences in the ids
 // [q len, (q + 1) len).
-template <typename IdT>
+template <typename IdT, bool TABLE>
 __global__ void __launch_bounds__(kSpThreads)
 k_sp_count(const IdT *__restrict__ ids, int64_t N, int64_t V, int32_t *__restrict__ slot,
            int32_t *__restrict__ arr, int32_t *__restrict__ rng, unsigned len, int nrange, DevScalars *sc)
 {
-    constexpr int kTab = kCountKeys;  // a power of two
-    constexpr int kPer = kCountKeys / kSpThreads;
+    constexpr int kTab = TABLE ? kCountKeys : kSpThreads;  // a power of two
+    constexpr int kPer = TABLE ? kCountKeys / kSpThreads : 1;
     __shared__ int tag[kTab], num[kTab];
     __shared__ int cnt[2 * kScanCtas];
     const int tid = threadIdx.x, lane = tid & 31;
-    const int64_t k0 = (int64_t)blockIdx.x * kCountKeys + tid;
+    const int64_t k0 = (int64_t)blockIdx.x * (kPer * kSpThreads) + tid;
+    if constexpr (TABLE)
     for (int q = tid; q < kTab; q += kSpThreads) {
         tag[q] = -1;
         num[q] = 0;
@@ -128,7 +129,11 @@ k_sp_count(const IdT *__restrict__ ids, int64_t N, int64_t V, int32_t *__restric
         const int lead = __ffs(peers) - 1;
         const int n = __popc(peers);
         int h = -1, m = 0;
-        if (id[e] >= 0 && lane == lead) {
+        if (!TABLE && id[e] >= 0 && lane == lead) {
+            m = atomicAdd(&slot[id[e]], n);
+            count_in(id[e], n, m);
+        }
+        if (TABLE && id[e] >= 0 && lane == lead) {
             h = (int)(((unsigned)id[e] * 2654435761u) >> 16) & (kTab - 1);  // Fibonacci hashing
             const int old = atomicCAS(&tag[h], -1, id[e]);
             if (old == -1 || old == id[e]) {
@@ -143,7 +148,7 @@ k_sp_count(const IdT *__restrict__ ids, int64_t N, int64_t V, int32_t *__restric
         mine[e] = __shfl_sync(0xffffffffu, m, lead) + __popc(peers & ((1u << lane) - 1u));
     }
     __syncthreads();
-    {
+    if constexpr (TABLE) {
         // the table's ids to the map, all of a thread's atomics in one trip
         constexpr int kE = kTab / kSpThreads;
         int n[kE], x[kE], before[kE];
@@ -161,8 +166,8 @@ k_sp_count(const IdT *__restrict__ ids, int64_t N, int64_t V, int32_t *__restric
                 num[tid + e * kSpThreads] = before[e];
                 count_in(x[e], n[e], before[e]);
             }
+        __syncthreads();
     }
-    __syncthreads();
 #pragma unroll
     for (int e = 0; e < kPer; ++e) {
         const int64_t k = k0 + e * kSpThreads;
@@ -687,6 +692,7 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
     constexpr int kIdxWindow = 1024;      // occurrences whose indices the CTA holds
     __shared__ float rp[kFin][kThreads];
     __shared__ int fin[kWarps][kFin];
+    __shared__ int edge[kWarps][4];
     __shared__ int sperm[kIdxWindow];
     __shared__ int sseg[kIdxWindow];
     __shared__ float comb[kThreads * VEC];
@@ -710,6 +716,8 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
     F *const ring = reinterpret_cast<F *>(sp_ring) + threadIdx.x;  // slot q at ring[q * NT]
     grid_dep_wait();  // runs and occurrence order from the dedup kernels
     grid_dep_launch();
+    // (the bounds are loaded with n_valid, before it says whether they count)
+    const int q0 = bounds[w], q1 = bounds[w + 1];
     const int n_valid = sc->n_valid;
     float colacc[VEC];
 #pragma unroll
@@ -722,8 +730,8 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
 
     int p0 = 0, p1 = 0;
     if (b1 < nw1 && n_valid > 0 && w < workers_of(n_valid, nw1, rg)) {
-        p0 = bounds[w];
-        p1 = bounds[w + 1];
+        p0 = q0;
+        p1 = q1;
         if (p0 == p1 && active) {
             // an empty range holds no piece of the run that spans it
             const F z = zero_vec<VEC>();
@@ -750,12 +758,15 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
     };
     if (p0 < p1) {
         // Only the range's first run can have started before it and only
-        // its last run can continue after it; decide both once, here.
-        const int u_first = segidx[p0];
-        const int u_last = segidx[p1 - 1];
-        const bool first_cut = p0 > 0 && segidx[p0 - 1] == u_first;
-        const bool last_cut = p1 < n_valid && segidx[p1] == u_last;
-        int cur = u_first;
+        // its last run can continue after it; both are decided once, from the
+        // run indices at the range's edges, loaded with the first window's.
+        if (l < 4) {
+            const int at = l == 0 ? p0 - 1 : l == 1 ? p0 : l == 2 ? p1 - 1 : p1;
+            edge[g][l] = at >= 0 && at < n_valid ? segidx[at] : -1;
+        }
+        int u_first = -1, u_last = -1;
+        bool first_cut = false, last_cut = false;
+        int cur = -1;
         int len = 0;  // occurrences of `cur` seen in this range
         // Per-id sums in occurrence order, compensated (Kahan): `acc` is the
         // running sum, `cmp` the part of it that rounding added, so the sum
@@ -802,6 +813,12 @@ k_sp_segsum(const float *__restrict__ rows, const int32_t *__restrict__ perm,
                 wseg[q] = segidx[wb + q];
             }
             group_bar(g, rg, tpb);
+            if (wb == p0) {
+                u_first = cur = edge[g][1];
+                u_last = edge[g][2];
+                first_cut = edge[g][0] == u_first;
+                last_cut = edge[g][3] == u_last;
+            }
             // rows b .. b + kBatch - 1 of the window into the kBatch slots
             // from `slot` on, one commit group
             auto fetch = [&](int b, F *slot) {
@@ -908,7 +925,8 @@ k_sp_carry(const int2 *__restrict__ cuts, const DevScalars *__restrict__ sc, con
 #pragma unroll
     for (int e = 0; e < VEC; ++e)
         colacc[e] = 0.f;
-    const int2 cut = ((int)(blockIdx.x / NS) < nw1 && n_valid > 0 && bd < workers_of(n_valid, nw1, rg)) ? cuts[bd] : make_int2(-1, 0);
+    const bool in_use = (int)(blockIdx.x / NS) < nw1 && n_valid > 0 && bd < workers_of(n_valid, nw1, rg);
+    const int2 cut = in_use ? cuts[bd] : make_int2(-1, 0);
     const bool mine = cut.x >= 0;
     // pieces q0 .. q1 of the run that began in worker w (piece 0: its last
     // piece; piece q: the first piece of worker w + q, zero where that range is
@@ -1019,8 +1037,8 @@ __global__ void __launch_bounds__(kThreads, apply_ctas_per_sm(CPT))
 k_sp_apply(void *__restrict__ W, const float *__restrict__ S, const float *__restrict__ rows,
            const int32_t *__restrict__ uniq, const int32_t *__restrict__ single,
            const float *__restrict__ r, const float *__restrict__ c,
-           const DevScalars *__restrict__ sc, NormSource norm, int D, int ld, int tpr, StepConsts kc, float eps,
-           float lr_signed, int variant)
+           const DevScalars *__restrict__ sc, NormSource norm, int D, int ld, int tpr, StepConsts kc,
+           float eps, float lr_signed, int variant)
 {
     using F = typename Vec<VEC>::F;
     using WT = typename WRaw<BF16, VEC>::T;
@@ -1115,6 +1133,12 @@ struct Tracer {
     bool pdl() const { return ev == nullptr; }
 };
 
+// Fewest occurrences that are counted through the hash table: below, at most
+// 3.3 ns of atomics queue on one address per 32 occurrences of one id, and
+// the direct form's one trip to L2 ends sooner (32768 Zipf ids: 5.6 us
+// against 7.2; 262144: 27.8 against 14.4).
+constexpr int64_t kTableMinN = 65536;
+
 // Ids per range of k_sp_count and k_sp_scan, and the number of ranges: a
 // function of V alone.
 int64_t scan_len(int64_t V)
@@ -1138,9 +1162,10 @@ void launch_count_scan(const SparseArgs &a, Tracer &tr, float *r, const EmaPair 
     auto *rng = reinterpret_cast<int32_t *>(ws + L.sp_rng);
     const int64_t len = scan_len(a.V);
     const int nr = scan_ranges(a.V);
-    const int nb = (int)((a.N + kCountKeys - 1) / kCountKeys);
-    if (nb > 0) {
-        launch_k(k_sp_count<IdT>, dim3(nb), dim3(kSpThreads), 0, a.stream, tr.pdl(),
+    if (a.N > 0) {
+        const bool table = a.N >= kTableMinN;
+        const int keys = table ? kCountKeys : kSpThreads;
+        launch_k(table ? k_sp_count<IdT, true> : k_sp_count<IdT, false>, dim3((int)((a.N + keys - 1) / keys)), dim3(kSpThreads), 0, a.stream, tr.pdl(),
                  static_cast<const IdT *>(a.ids), a.N, a.V, slot, reinterpret_cast<int32_t *>(ws + L.sp_arr), rng,
                  (unsigned)len, nr, sc);
         tr.mark();
