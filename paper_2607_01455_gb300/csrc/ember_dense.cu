@@ -145,6 +145,19 @@ __device__ __forceinline__ void reduce_rows(const float *__restrict__ G, float *
     int it = 0;    // iteration index (the slot of the kept G)
     for (int64_t base = row0; base < row1; base += rows_per_it, ++it) {
         F v[R][CPT];
+        // the old r of the row this thread finishes, when this iteration ends
+        // with that: loaded with the rows, not after the barrier that follows
+        // (0.7 to 1 us off 50257 x 768 and 151936 x 896; with 4-byte accesses or
+        // eight per row it is not worth its instructions: 30011 x 1003 83.8 us
+        // against 79.5)
+        constexpr bool kEarly = VEC == 4 && CPT <= 4;
+        static_assert(kRowBuf <= kThreads, "a thread finishes one row of the buffer");
+        float r_old = 0.f;
+        if constexpr (kEarly) {
+            const bool last = nbuf + 1 == its_per_buf || base + rows_per_it >= row1;
+            if (last && rowpart == nullptr && tid < (nbuf + 1) * rows_per_it && buf_base + tid < row1)
+                r_old = r[buf_base + tid];
+        }
         const uint64_t pol = base >= keep0 ? pol_keep : pol_pass;
 #pragma unroll
         for (int k = 0; k < R; ++k) {
@@ -218,7 +231,7 @@ __device__ __forceinline__ void reduce_rows(const float *__restrict__ G, float *
                         rowpart[i] = sum;
                         continue;
                     }
-                    const float rn = ema_pair(kc.ema, r[i], sum * kc.inv_D);
+                    const float rn = ema_pair(kc.ema, kEarly ? r_old : r[i], sum * kc.inv_D);
                     r[i] = rn;
                     if (keep_r)  // the one-launch step's update reads it back here
                         keep_r[i - row0] = rn;
@@ -1111,7 +1124,17 @@ k_rowonly_dense(void *__restrict__ W, const float *__restrict__ G, float *__rest
             acc[c][e] = 0.f;
     float rsum = 0.f;
     const int rows_per_it = rg * R;
+    // the old r of the row that this thread finishes, an iteration ahead: a
+    // trip to L2 between the two barriers of every iteration otherwise (50304 x
+    // 2048: 132 us per step against 151)
+    auto old_r = [&](int64_t base) {
+        const int64_t i = base + (int64_t)g * R + l;
+        return (l < R && i < row1) ? r[i] : 0.f;
+    };
+    float r_next = old_r(row0);
     for (int64_t base = row0; base < row1; base += rows_per_it) {
+        const float r_old = r_next;
+        r_next = old_r(base + rows_per_it);
         F v[R][CPT];
         WT wr[R][CPT];
         if constexpr (ASYNC) {
@@ -1167,7 +1190,7 @@ k_rowonly_dense(void *__restrict__ W, const float *__restrict__ G, float *__rest
                 float sum = 0.f;
                 for (int q = 0; q < wpg; ++q)
                     sum += red[g * wpg + q][l];
-                const float rn = ema_pair(kc.ema, r[i], sum * kc.inv_D);
+                const float rn = ema_pair(kc.ema, r_old, sum * kc.inv_D);
                 r[i] = rn;
                 rsum += rn;
                 rsv = sqrtf(rn * kc.inv_bc);
