@@ -1398,7 +1398,9 @@ cudaError_t launch_dense_t(const DenseArgs &a)
             // a small table: the whole step in one cluster launch, the kept
             // G and W in shared memory
             auto *k = a.wbf16 ? k_dense_cluster<CPT, R1, true> : k_dense_cluster<CPT, R1, false>;
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            e = cudaSuccess;
+            if (sm > (size_t)40 << 10)  // with the static arrays up to 48 KiB need no leave
+                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
             if (e == cudaSuccess && nparts > 8)
                 e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
             if (e != cudaSuccess)

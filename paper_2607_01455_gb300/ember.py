@@ -118,11 +118,18 @@ def _addr(x):
 
 def _stream(s):
     if s is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(s, int):
         return s
     return s.cuda_stream
+
+
+def _current_stream():
+    """Handle of torch's current stream on the current device.  Asked of torch
+    directly: a torch.cuda.Stream object made for its handle alone takes longer
+    than the rest of a call's marshalling."""
+    import torch
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _check(status, where):
