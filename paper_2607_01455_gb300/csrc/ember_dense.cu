@@ -569,7 +569,7 @@ k_state_dense(ColSource src, float *__restrict__ rsum_part, float *__restrict__ 
 template <int VEC, int K, int R, bool BF16, bool RAG>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__restrict__ r,
-              const float *__restrict__ c, NormSource norm, int64_t V, int D, int ld, int lpr, int nseg, int mis,
+              const float *__restrict__ c, NormSource norm, int64_t V, int D, int ld, int lpr_arg, int nseg, int mis,
               StepConsts kc, float eps, float lr_signed, int variant, RowSpan span)
 {
     static_assert(!RAG || VEC == 4, "shifted rows use 16-byte accesses");
@@ -578,6 +578,7 @@ k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__
     extern __shared__ __align__(16) float cs[];  // D column scales (RAG: four shifted copies)
     constexpr int kWarps = kThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int lpr = K > 1 ? 32 : lpr_arg;  // a constant, so that the accesses' offsets are immediates
     const int l = lane & (lpr - 1);     // position within the row's accesses
     const int rpa = 32 / lpr;           // rows per warp-wide access
     const int rows_per_unit = R * rpa;
@@ -632,8 +633,10 @@ k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__
     }
     __syncthreads();
 
+    // unit idx is row block rb and segment seg, kept without a division per unit
+    const int drb = kWarps / nseg, dseg = kWarps - drb * nseg;
+    int rb = warp / nseg, seg = warp - rb * nseg;
     for (int idx = warp; idx < nunits; idx += kWarps) {
-        const int rb = idx / nseg, seg = idx - rb * nseg;
         const int64_t base = row1 - (int64_t)(rb + 1) * rows_per_unit;
         F gv[R][K];
         WT wr[R][K];
@@ -702,6 +705,12 @@ k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__
                     }
                 }
             }
+        }
+        rb += drb;
+        seg += dseg;
+        if (seg >= nseg) {
+            seg -= nseg;
+            ++rb;
         }
     }
 }
