@@ -139,11 +139,11 @@ size_t ember_state_numel(const ember_handle *h);
  * carry at most max_sparse_N ids (0 if only dense steps are used).  Returns
  * 0 for a NULL handle or a negative max_sparse_N.  The workspace holds
  * per-block partial sums (among them the LM-head step's per-tile sums of
- * g^2, V*D*4*(1/128 + 1/256) bytes, always reserved), the sort buffers of
+ * g^2, V*D*4*(1/128 + 1/256) bytes, always reserved), the dedup buffers of
  * the sparse step, the summed gradient rows of the sparse step (up to
  * max_sparse_N x D fp32), a V-entry map of touched rows and a few scalars.
- * It is not optimizer state, but the steps leave the touched-row map zeroed
- * for the next one: the caller must not write to the workspace after binding
+ * It is not optimizer state, but the steps leave the touched-row map and the
+ * dedup's counters zeroed for the next one: the caller must not write to the workspace after binding
  * it, nor touch it while a step is in flight. */
 size_t ember_workspace_bytes(const ember_handle *h, int64_t max_sparse_N);
 
@@ -166,8 +166,9 @@ ember_status ember_bind_workspace(ember_handle *h, void *workspace, size_t bytes
  * covers in a few passes) runs as one launch of a thread-block cluster of
  * up to 16 CTAs that keeps G and W in shared memory and reads G from HBM
  * once; every other table runs as three launches (reduce, column
- * statistics and normaliser, update), chained with programmatic dependent
- * launch.  Both forms run the same arithmetic on the same CTA row
+ * statistics, update).  Every launch is a programmatic dependent one and
+ * waits for the work before it on the stream before it reads anything.
+ * Both forms run the same arithmetic on the same CTA row
  * ranges and give the same bits.  Graph capture works for both. */
 ember_status ember_step_dense(ember_handle *h, void *W, const float *G, float *state,
                               float lr, int64_t t, void *stream);
