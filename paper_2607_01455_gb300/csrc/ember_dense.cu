@@ -1135,15 +1135,19 @@ k_rowonly_dense(void *__restrict__ W, const float *__restrict__ G, float *__rest
     const int rows_per_it = rg * R;
     // the old r of the row that this thread finishes, an iteration ahead: a
     // trip to L2 between the two barriers of every iteration otherwise (50304 x
-    // 2048: 132 us per step against 151)
+    // 2048: 132 us per step against 151).  Not with eight accesses per row,
+    // whose 128 registers have no room for it (128256 x 8192: 1226 us without,
+    // 1251 with it).
+    constexpr bool kAhead = CPT <= 4;
     auto old_r = [&](int64_t base) {
         const int64_t i = base + (int64_t)g * R + l;
         return (l < R && i < row1) ? r[i] : 0.f;
     };
-    float r_next = old_r(row0);
+    float r_next = kAhead ? old_r(row0) : 0.f;
     for (int64_t base = row0; base < row1; base += rows_per_it) {
         const float r_old = r_next;
-        r_next = old_r(base + rows_per_it);
+        if (kAhead)
+            r_next = old_r(base + rows_per_it);
         F v[R][CPT];
         WT wr[R][CPT];
         if constexpr (ASYNC) {
@@ -1199,7 +1203,7 @@ k_rowonly_dense(void *__restrict__ W, const float *__restrict__ G, float *__rest
                 float sum = 0.f;
                 for (int q = 0; q < wpg; ++q)
                     sum += red[g * wpg + q][l];
-                const float rn = ema_pair(kc.ema, r_old, sum * kc.inv_D);
+                const float rn = ema_pair(kc.ema, kAhead ? r_old : r[i], sum * kc.inv_D);
                 r[i] = rn;
                 rsum += rn;
                 rsv = sqrtf(rn * kc.inv_bc);
@@ -1321,7 +1325,7 @@ cudaError_t launch_dense_t(const DenseArgs &a)
     // follows the previous one; without, every kernel uses programmatic
     // dependent launch, the first one too: it waits for the work before the
     // step on the stream only when it runs.  That takes 1.5 to 2 us off a step
-    // (4096 x 256 bf16 14.4 -> 12.6 us, 1024 x 64 fp32 9.4 -> 7.8).
+    // (1024 x 64 fp32 9.4 -> 7.8 us, 50257 x 768 bf16 88.3 -> 86.7).
     const bool pdl = (a.trace == nullptr);
     cudaError_t e;
     RowSpan span{0, nparts, 0};
