@@ -1261,6 +1261,15 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     const dim3 sum_threads(map.rg * map.tpb);
     Tracer tr{a.trace, a.n_trace, 0, a.stream};
 
+    auto *segsum = sum_threads.x > 192   ? k_sp_segsum<VEC, 256>
+                   : sum_threads.x > 128 ? k_sp_segsum<VEC, 192>
+                                         : k_sp_segsum<VEC, 128>;
+    // the ring and the static arrays together pass 48 KiB; asked for before the
+    // first launch, which leaves counts that only a whole step clears
+    const cudaError_t e = cudaFuncSetAttribute(segsum, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    if (e != cudaSuccess)
+        return e;
+
     tr.mark();
     const int G = kSparseCtas;
     const StepConsts kc = make_consts(a.beta2, a.one_minus_beta2, a.V, a.D, a.inv_bc);
@@ -1285,13 +1294,6 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
         launch_count_scan<int32_t>(a, tr, a.r, kc.ema, rsum_part);
         launch_place_order<int32_t>(a, tr, G / NS, map.rg);
     }
-    auto *segsum = sum_threads.x > 192   ? k_sp_segsum<VEC, 256>
-                   : sum_threads.x > 128 ? k_sp_segsum<VEC, 192>
-                                         : k_sp_segsum<VEC, 128>;
-    // the ring and the static arrays together pass 48 KiB
-    const cudaError_t e = cudaFuncSetAttribute(segsum, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
-    if (e != cudaSuccess)
-        return e;
     launch_k(segsum, dim3(G), sum_threads, kRingBytes, a.stream, tr.pdl(), a.rows, perm, segidx, sc, S, rowpart, carry,
              colpart, bounds, D, map, reinterpret_cast<int32_t *>(ws + L.sp_rng), kScanCounters);
     tr.mark();
