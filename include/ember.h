@@ -306,7 +306,10 @@ ember_status ember_shard_update(ember_handle *h, int shard, int nshards, void *W
  * rows[k] over the k with ids[k] == u, summed in increasing k: every row of
  * r decays by beta2, the column statistics divide by V, and rows of W whose
  * id does not occur are left bit-identical.  An id outside [0, V) is
- * skipped and sets EMBER_ERR_ID_OUT_OF_RANGE in the device flag. */
+ * skipped and sets EMBER_ERR_ID_OUT_OF_RANGE in the device flag.
+ *   A kernel launch that fails partway ends the call with EMBER_ERR_CUDA:
+ * nothing more is launched, the step is incomplete (r and c may already be
+ * updated), and the workspace is made ready for the next step. */
 ember_status ember_step_sparse(ember_handle *h, void *W, const void *ids,
                                ember_idtype idtype, int64_t N, const float *rows,
                                float *state, float lr, int64_t t, void *stream);

@@ -174,6 +174,7 @@ ember_status ember_bind_workspace(ember_handle *h, void *workspace, size_t bytes
     h->ws = (unsigned char *)workspace;
     h->ws_bytes = bytes;
     h->ws_max_N = max_sparse_N;
+    h->sp_unclean = false;
     return EMBER_OK;
 }
 
@@ -530,6 +531,7 @@ ember_status ember_step_sparse(ember_handle *h, void *W, const void *ids, ember_
     a.stream = (cudaStream_t)stream;
     a.trace = h->n_trace > 0 ? h->trace : nullptr;
     a.n_trace = h->n_trace;
+    a.unclean = &h->sp_unclean;
     const bool vec4 = (h->D % 4 == 0) && is_aligned(W, 4 * wsz) && (N == 0 || is_aligned(rows, 16));
     if (!choose_colmap(h->D, vec4, &a.map))
         return EMBER_ERR_UNSUPPORTED;
@@ -560,6 +562,7 @@ ember_status ember_sparse_unique(ember_handle *h, const void *ids, ember_idtype 
     a.ws = h->ws;
     a.lay = make_layout(h->V, h->D, h->ws_max_N);
     a.stream = (cudaStream_t)stream;
+    a.unclean = &h->sp_unclean;
     return launch_sparse_unique(a, uniq, counts, n_unique) == cudaSuccess ? EMBER_OK : EMBER_ERR_CUDA;
 }
 

@@ -305,6 +305,7 @@ struct SparseArgs {
     cudaStream_t stream;
     const cudaEvent_t *trace;  // nullptr, or events to record at kernel boundaries
     int n_trace;
+    bool *unclean;  // the handle's: set when a failed call left the map or the counters nonzero
 };
 
 cudaError_t launch_sparse_step(const SparseArgs &a);
@@ -348,4 +349,5 @@ struct ember_handle {
     cudaEvent_t trace[ember::kMaxTraceEvents];
     int n_trace;
     uint64_t wait_ns;  // limit of the bounded waits inside kernels (ember_set_wait_limit_ns)
+    bool sp_unclean;   // the sparse step's map and counters must be cleared before their next use
 };

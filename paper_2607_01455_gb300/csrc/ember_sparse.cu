@@ -1119,19 +1119,68 @@ k_sp_apply(void *__restrict__ W, const float *__restrict__ S, const float *__res
     }
 }
 
-struct Tracer {
+// The launches of one step or dedup on its stream, in order, with the trace
+// events between them.  After a launch that fails nothing more is launched:
+// the kernels after it would read what it has not written (k_sp_place, for
+// one, would take the counts left in the map for run numbers).
+struct Launches {
     const cudaEvent_t *ev;
     int n, next;
     cudaStream_t s;
+    cudaError_t err = cudaSuccess;  // of the first launch that failed
+    template <typename K, typename... Args>
+    void launch(K kernel, dim3 grid, dim3 block, size_t smem, bool early, Args &&...args)
+    {
+        if (err == cudaSuccess)
+            err = launch_k(kernel, grid, block, smem, s, early, static_cast<Args &&>(args)...);
+    }
     void mark()
     {
-        if (ev && next < n)
+        if (err == cudaSuccess && ev && next < n)
             cudaEventRecord(ev[next], s);
         ++next;
     }
     // programmatic dependent launch, unless events are recorded between the kernels
     bool pdl() const { return ev == nullptr; }
 };
+
+// The map and the counters back to zero, as every step expects them.
+cudaError_t clear_dedup(const SparseArgs &a)
+{
+    const cudaError_t e = cudaMemsetAsync(a.ws + a.lay.sp_slot, 0, sizeof(int32_t) * (size_t)a.V, a.stream);
+    return e != cudaSuccess ? e
+                            : cudaMemsetAsync(a.ws + a.lay.sp_rng, 0, sizeof(int32_t) * kScanCounters, a.stream);
+}
+
+// Before the first launch: what an earlier call could not clear.  A clear that
+// is only captured leaves the next call to clear again.
+cudaError_t begin(const SparseArgs &a)
+{
+    if (!*a.unclean)
+        return cudaSuccess;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(a.stream, &capture);
+    if (e == cudaSuccess)
+        e = clear_dedup(a);
+    if (e == cudaSuccess && capture == cudaStreamCaptureStatusNone)
+        *a.unclean = false;
+    return e;
+}
+
+// After the last launch.  A failed one leaves counts, run numbers or range
+// counters behind, which the kernels launched next would add to and take
+// positions from: they are cleared behind the kernels that did run, or, where
+// that fails too, before the next step.
+cudaError_t finish(const SparseArgs &a, const Launches &la)
+{
+    if (la.err == cudaSuccess)
+        return cudaGetLastError();
+    cudaGetLastError();  // reported here, not by the next call
+    if (clear_dedup(a) != cudaSuccess)
+        *a.unclean = true;
+    cudaGetLastError();
+    return la.err;
+}
 
 // Fewest occurrences that are counted through the hash table: below, at most
 // 3.3 ns of atomics queue on one address per 32 occurrences of one id, and
@@ -1153,7 +1202,7 @@ int scan_ranges(int64_t V) { return (int)((V + scan_len(V) - 1) / scan_len(V)); 
 // Count the ids and number the distinct ones; with r also decay the rows
 // outside the batch (their sums to rsum_part[0 .. scan_ranges)).
 template <typename IdT>
-void launch_count_scan(const SparseArgs &a, Tracer &tr, float *r, const EmaPair &ema, float *rsum_part)
+void launch_count_scan(const SparseArgs &a, Launches &la, float *r, const EmaPair &ema, float *rsum_part)
 {
     unsigned char *ws = a.ws;
     const Layout &L = a.lay;
@@ -1165,21 +1214,22 @@ void launch_count_scan(const SparseArgs &a, Tracer &tr, float *r, const EmaPair 
     if (a.N > 0) {
         const bool table = a.N >= kTableMinN;
         const int keys = table ? kCountKeys : kSpThreads;
-        launch_k(table ? k_sp_count<IdT, true> : k_sp_count<IdT, false>, dim3((int)((a.N + keys - 1) / keys)), dim3(kSpThreads), 0, a.stream, tr.pdl(),
+        la.launch(table ? k_sp_count<IdT, true> : k_sp_count<IdT, false>, dim3((int)((a.N + keys - 1) / keys)),
+                  dim3(kSpThreads), 0, la.pdl(),
                  static_cast<const IdT *>(a.ids), a.N, a.V, slot, reinterpret_cast<int32_t *>(ws + L.sp_arr), rng,
                  (unsigned)len, nr, sc);
-        tr.mark();
+        la.mark();
     }
-    launch_k(k_sp_scan, dim3(nr), dim3(kSpThreads), 0, a.stream, tr.pdl(), slot, a.V, len, rng,
+    la.launch(k_sp_scan, dim3(nr), dim3(kSpThreads), 0, la.pdl(), slot, a.V, len, rng,
              reinterpret_cast<int32_t *>(ws + L.sp_uniq), reinterpret_cast<int32_t *>(ws + L.sp_segoff),
              reinterpret_cast<int32_t *>(ws + L.sp_long), rng + kScanCounters - 1, sc, r, ema, rsum_part);
-    tr.mark();
+    la.mark();
 }
 
 // Every occurrence to its place in (id, occurrence) order; bounds of the
 // workers of the segment sums (rg groups in each of nw1 CTAs per slice).
 template <typename IdT>
-void launch_place_order(const SparseArgs &a, Tracer &tr, int nw1, int rg)
+void launch_place_order(const SparseArgs &a, Launches &la, int nw1, int rg)
 {
     unsigned char *ws = a.ws;
     const Layout &L = a.lay;
@@ -1190,18 +1240,19 @@ void launch_place_order(const SparseArgs &a, Tracer &tr, int nw1, int rg)
     const int nb = (int)((a.N + kSpThreads - 1) / kSpThreads);
     if (nb == 0)
         return;  // no occurrence: the segment sums and the carry see n_valid = 0
-    launch_k(k_sp_place<IdT>, dim3(nb), dim3(kSpThreads), 0, a.stream, tr.pdl(), static_cast<const IdT *>(a.ids), a.N,
+    la.launch(k_sp_place<IdT>, dim3(nb), dim3(kSpThreads), 0, la.pdl(), static_cast<const IdT *>(a.ids), a.N,
              reinterpret_cast<int32_t *>(ws + L.sp_slot), segoff, reinterpret_cast<int32_t *>(ws + L.sp_arr), placed,
              segidx, reinterpret_cast<int32_t *>(ws + L.sp_single));
-    tr.mark();
+    la.mark();
     const int64_t nbig64 = a.N / (kLongRun + 1) * ((a.N + kWinBits - 1) / kWinBits);
     const int nbig = (int)(nbig64 < kGridCtas ? nbig64 : kGridCtas);
-    launch_k(k_sp_order, dim3(nbig + (int)((a.N + kOrderThreads - 1) / kOrderThreads)), dim3(kOrderThreads), 0, a.stream, tr.pdl(), placed, segidx, segoff,
+    la.launch(k_sp_order, dim3(nbig + (int)((a.N + kOrderThreads - 1) / kOrderThreads)), dim3(kOrderThreads), 0,
+              la.pdl(), placed, segidx, segoff,
              reinterpret_cast<int32_t *>(ws + L.sp_long),
              reinterpret_cast<int32_t *>(ws + L.sp_rng) + kScanCounters - 1, sc, a.N, nbig,
              reinterpret_cast<int32_t *>(ws + L.sp_perm), reinterpret_cast<int32_t *>(ws + L.sp_bounds),
              reinterpret_cast<int2 *>(ws + L.sp_cuts), nw1, rg);
-    tr.mark();
+    la.mark();
 }
 
 // Distinct ids, their counts and U to caller buffers.
@@ -1259,26 +1310,27 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     const SumMap map = sum_map(DV);
     const int NS = map.NS;
     const dim3 sum_threads(map.rg * map.tpb);
-    Tracer tr{a.trace, a.n_trace, 0, a.stream};
+    Launches la{a.trace, a.n_trace, 0, a.stream};
 
     auto *segsum = sum_threads.x > 192   ? k_sp_segsum<VEC, 256>
                    : sum_threads.x > 128 ? k_sp_segsum<VEC, 192>
                                          : k_sp_segsum<VEC, 128>;
-    // the ring and the static arrays together pass 48 KiB; asked for before the
-    // first launch, which leaves counts that only a whole step clears
-    const cudaError_t e = cudaFuncSetAttribute(segsum, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    // the ring and the static arrays together pass 48 KiB
+    cudaError_t e = cudaFuncSetAttribute(segsum, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    if (e == cudaSuccess)
+        e = begin(a);
     if (e != cudaSuccess)
         return e;
 
-    tr.mark();
+    la.mark();
     const int G = kSparseCtas;
     const StepConsts kc = make_consts(a.beta2, a.one_minus_beta2, a.V, a.D, a.inv_bc);
     if (a.N > 0 && a.N <= kSmallN) {
         const int nkey = (int)((a.N + kSpThreads / 32 - 1) / (kSpThreads / 32));
         auto go = [&](auto *ids) {
             using IdT = std::remove_const_t<std::remove_pointer_t<decltype(ids)>>;
-            launch_k(k_sp_dedup_small<IdT>, dim3(nkey + scan_ranges(a.V)), dim3(kSpThreads), 0, a.stream,
-                     tr.pdl() && small_first_pdl(a.N), ids,
+            la.launch(k_sp_dedup_small<IdT>, dim3(nkey + scan_ranges(a.V)), dim3(kSpThreads), 0,
+                      la.pdl() && small_first_pdl(a.N), ids,
                      (int)a.N, a.V, perm, segidx, uniq, single, bounds, cuts, G / NS, map.rg, sc, nkey, scan_len(a.V),
                      a.r, kc.ema, rsum_part);
         };
@@ -1286,20 +1338,20 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
             go(static_cast<const int64_t *>(a.ids));
         else
             go(static_cast<const int32_t *>(a.ids));
-        tr.mark();
+        la.mark();
     } else if (a.ids64) {
-        launch_count_scan<int64_t>(a, tr, a.r, kc.ema, rsum_part);
-        launch_place_order<int64_t>(a, tr, G / NS, map.rg);
+        launch_count_scan<int64_t>(a, la, a.r, kc.ema, rsum_part);
+        launch_place_order<int64_t>(a, la, G / NS, map.rg);
     } else {
-        launch_count_scan<int32_t>(a, tr, a.r, kc.ema, rsum_part);
-        launch_place_order<int32_t>(a, tr, G / NS, map.rg);
+        launch_count_scan<int32_t>(a, la, a.r, kc.ema, rsum_part);
+        launch_place_order<int32_t>(a, la, G / NS, map.rg);
     }
-    launch_k(segsum, dim3(G), sum_threads, kRingBytes, a.stream, tr.pdl(), a.rows, perm, segidx, sc, S, rowpart, carry,
+    la.launch(segsum, dim3(G), sum_threads, kRingBytes, la.pdl(), a.rows, perm, segidx, sc, S, rowpart, carry,
              colpart, bounds, D, map, reinterpret_cast<int32_t *>(ws + L.sp_rng), kScanCounters);
-    tr.mark();
-    launch_k(k_sp_carry<VEC>, dim3(G), sum_threads, 0, a.stream, tr.pdl(), cuts, sc, carry, S, rowpart,
+    la.mark();
+    la.launch(k_sp_carry<VEC>, dim3(G), sum_threads, 0, la.pdl(), cuts, sc, carry, S, rowpart,
              colpart, D, map);
-    tr.mark();
+    la.mark();
     // the touched rows' r and the column pass in one launch (a row per thread
     // for up to one CTA per SM: more would only wait for a place); the per-CTA
     // sums of r follow the scan CTAs' sums of the decayed rows
@@ -1308,9 +1360,10 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     const int GU = (int)(ub < kSms ? ub : kSms);
     const NormSource norm{rsum_part, nr + GU, csum_part, (D + kStateCols - 1) / kStateCols, nullptr, nullptr, D};
     // (segment-sum CTA b writes only the columns of its slice b % NS)
-    launch_state(colpart, G, rsum_part, a.c, csum_part, sc, a.V, D, kc, a.stream, tr.pdl(), a.r, slot,
-                 rowpart, NS, GU, uniq, nr, NS, map.tpb * VEC);
-    tr.mark();
+    if (la.err == cudaSuccess)
+        la.err = launch_state(colpart, G, rsum_part, a.c, csum_part, sc, a.V, D, kc, a.stream, la.pdl(), a.r, slot,
+                              rowpart, NS, GU, uniq, nr, NS, map.tpb * VEC);
+    la.mark();
     // one launch per column panel (one unless D is wider than a CTA's row)
     const int np = a.map.npanels, pw = a.map.pw;
     const size_t cs_bytes = (size_t)pw * sizeof(float);
@@ -1321,16 +1374,16 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
         void *Wq = static_cast<unsigned char *>(a.W) + c0 * (a.wbf16 ? 2 : 4);
         const float *rq = a.rows ? a.rows + c0 : nullptr;
         if (a.wbf16)
-            launch_k(k_sp_apply<VEC, CPT, R, true>, dim3(GA), dim3(kThreads), cs_bytes, a.stream, tr.pdl(), Wq,
+            la.launch(k_sp_apply<VEC, CPT, R, true>, dim3(GA), dim3(kThreads), cs_bytes, la.pdl(), Wq,
                      S + c0, rq, uniq, single, a.r, a.c + c0, sc, norm, dq, (int)a.D, a.map.tpr, kc, a.eps,
                      a.lr_signed, a.variant);
         else
-            launch_k(k_sp_apply<VEC, CPT, R, false>, dim3(GA), dim3(kThreads), cs_bytes, a.stream, tr.pdl(), Wq,
+            la.launch(k_sp_apply<VEC, CPT, R, false>, dim3(GA), dim3(kThreads), cs_bytes, la.pdl(), Wq,
                      S + c0, rq, uniq, single, a.r, a.c + c0, sc, norm, dq, (int)a.D, a.map.tpr, kc, a.eps,
                      a.lr_signed, a.variant);
     }
-    tr.mark();
-    return cudaGetLastError();
+    la.mark();
+    return finish(a, la);
 }
 
 }  // namespace
@@ -1358,11 +1411,14 @@ cudaError_t launch_sparse_step(const SparseArgs &a)
 cudaError_t launch_sparse_unique(const SparseArgs &a, int32_t *uniq_out, int32_t *counts_out,
                                  int32_t *n_unique_out)
 {
-    Tracer tr{nullptr, 0, 0, a.stream};
+    cudaError_t e = begin(a);
+    if (e != cudaSuccess)
+        return e;
+    Launches la{nullptr, 0, 0, a.stream};
     if (a.ids64)
-        launch_count_scan<int64_t>(a, tr, nullptr, EmaPair{}, nullptr);
+        launch_count_scan<int64_t>(a, la, nullptr, EmaPair{}, nullptr);
     else
-        launch_count_scan<int32_t>(a, tr, nullptr, EmaPair{}, nullptr);
+        launch_count_scan<int32_t>(a, la, nullptr, EmaPair{}, nullptr);
     const DevScalars *sc = reinterpret_cast<const DevScalars *>(a.ws + a.lay.scalars);
     const int32_t *uniq = reinterpret_cast<const int32_t *>(a.ws + a.lay.sp_uniq);
     const int32_t *segoff = reinterpret_cast<const int32_t *>(a.ws + a.lay.sp_segoff);
@@ -1371,12 +1427,12 @@ cudaError_t launch_sparse_unique(const SparseArgs &a, int32_t *uniq_out, int32_t
         nb = 1;
     if (nb > 4 * kGridCtas)
         nb = 4 * kGridCtas;
-    launch_k(k_sp_export, dim3((int)nb), dim3(kThreads), 0, a.stream, tr.pdl(), uniq, segoff, sc, a.N,
+    la.launch(k_sp_export, dim3((int)nb), dim3(kThreads), 0, la.pdl(), uniq, segoff, sc, a.N,
              uniq_out, counts_out, n_unique_out, reinterpret_cast<int32_t *>(a.ws + a.lay.sp_rng), kScanCounters);
     // the touched-row map must be all-zero again before the next step
-    int32_t *slot = reinterpret_cast<int32_t *>(a.ws + a.lay.sp_slot);
-    cudaMemsetAsync(slot, 0, sizeof(int32_t) * (size_t)a.V, a.stream);
-    return cudaGetLastError();
+    if (la.err == cudaSuccess)
+        la.err = cudaMemsetAsync(a.ws + a.lay.sp_slot, 0, sizeof(int32_t) * (size_t)a.V, a.stream);
+    return finish(a, la);
 }
 
 }  // namespace ember
