@@ -522,8 +522,6 @@ k_state_dense(ColSource src, float *__restrict__ rsum_part, float *__restrict__ 
             const int64_t U = sc->n_unique;
             for (int64_t u = (int64_t)rb * kStateThreads + threadIdx.x; u < U; u += stride) {
                 const int64_t i = rowp.uniq[u];
-                if (i < 0)
-                    continue;  // a small batch numbers its runs by position
                 float tot = 0.f;
                 for (int q = 0; q < rowp.nslices; ++q)
                     tot += rowp.rowpart[u * rowp.nslices + q];

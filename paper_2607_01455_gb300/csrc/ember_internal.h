@@ -61,8 +61,9 @@ constexpr int kScanCtas = kGridCtas;
 constexpr int kScanMin = 256;
 constexpr int kScanCounters = 2 * kScanCtas + 1;  // two per range, then the number of long runs
 constexpr int kLongRun = 128;
-// Batches of up to kSmallN occurrences are deduped by comparing all pairs.
-constexpr int kSmallN = 4096;
+// Batches of up to kSmallN occurrences are deduped in one launch (see
+// k_sp_dedup_small for both sides of the line).
+constexpr int kSmallN = 3072;
 
 // Workspace layout (byte offsets, each 256-byte aligned).
 struct Layout {

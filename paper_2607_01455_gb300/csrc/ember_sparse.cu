@@ -329,9 +329,12 @@ k_sp_place(const IdT *__restrict__ ids, int64_t N, const int32_t *__restrict__ s
 // one or two per position).  Worker w owns [first(w), first(w + 1)), where
 // first(w) is the smallest position whose cost reaches T(w) = w C / nw and
 // C = n_valid + U.
-__device__ __forceinline__ int64_t cost_target(int w, int nw, int64_t C)
+// I: int64_t, or int where 2 kSmallN times the number of workers fits it (64-bit
+// divisions take most of a microsecond of the one-launch dedup).
+template <typename I>
+__device__ __forceinline__ I cost_target(int w, int nw, I C)
 {
-    return ((int64_t)w * C) / nw;
+    return ((I)w * C) / nw;
 }
 
 // Workers in use, of the nw1 rg groups of a slice's CTAs (group g of CTA b is
@@ -350,15 +353,47 @@ __device__ __forceinline__ int workers_of(int n_valid, int nw1, int rg)
 }
 
 // Worker whose range holds sorted position p of run u.
-__device__ __forceinline__ int worker_of(int p, int u, int nw, int64_t C)
+template <typename I>
+__device__ __forceinline__ int worker_of(int p, int u, int nw, I C)
 {
-    const int64_t c = (int64_t)p + u;
+    const I c = (I)p + u;
     int w = (int)((c * nw) / C);
     while (w + 1 < nw && cost_target(w + 1, nw, C) <= c)
         ++w;
     while (w > 0 && cost_target(w, nw, C) > c)
         --w;
     return w;
+}
+
+// The workers that start at position p, of run u, which holds [s, e); `before`
+// is the run of position p - 1 (-1 for p = 0): those whose target lies above
+// the cost of the position before p and not above that of p, and, at the last
+// position, those above every cost, which own nothing.  cuts[q]: the run that
+// goes on at the start of worker q and began in worker q - 1's range, and the
+// worker it ends in, or (-1, 0).  Both forms of the dedup take the starts from
+// here: the sums of a batch do not depend on which one its length chooses.
+// Threads `first` of `step` share the workers.
+template <typename I>
+__device__ __forceinline__ void worker_starts(int p, int u, int before, int s, int e, int n_valid, int U, int nw1,
+                                              int rg, int32_t *__restrict__ bounds, int2 *__restrict__ cuts,
+                                              int first, int step)
+{
+    const int nw = workers_of(n_valid, nw1, rg);
+    const I C = (I)n_valid + U;
+    const I c1 = (I)p + u;
+    const I c0 = p > 0 ? (I)p - 1 + before : -1;
+    for (I q = ((c0 + 1) * nw + C - 1) / C + first; q < nw; q += step) {
+        const bool here = cost_target((int)q, nw, C) <= c1;
+        if (!here && p + 1 < n_valid)
+            break;
+        bounds[q] = here ? p : n_valid;
+        int2 cut = make_int2(-1, 0);
+        if (here && s < p && q > 0 && cost_target((int)q - 1, nw, C) <= (I)s + u)
+            cut = make_int2(u, worker_of(e - 1, u, nw, C));
+        cuts[q] = cut;
+    }
+    if (p + 1 == n_valid && first == 0)
+        bounds[nw] = n_valid;
 }
 
 // Each run's occurrences in increasing order, and the workers' bounds.
@@ -385,11 +420,11 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
     grid_dep_launch();
     if ((int)blockIdx.x >= nbig) {
         const int n_valid = sc->n_valid, U = sc->n_unique;
-        const int64_t p = (int64_t)((int)blockIdx.x - nbig) * kOrderThreads + tid;
+        const int p = ((int)blockIdx.x - nbig) * kOrderThreads + tid;  // N < 2^30
         if (p >= n_valid)
             return;
         const int u = segidx[p];
-        const int before = p > 0 ? segidx[p - 1] : 0;
+        const int before = p > 0 ? segidx[p - 1] : -1;
         const int x = placed[p];
         const int s = segoff[u], e = segoff[u + 1];
         if (e - s <= kLongRun) {
@@ -399,27 +434,7 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
                 below += placed[q] < x;
             perm[s + below] = x;
         }
-        // the workers whose target lies above the position before this one
-        // and not above this one start here (and those above the last
-        // position at the end); cuts[q]: the run that goes on at the start of
-        // worker q and began in worker q - 1's range, and the worker it ends
-        // in, or (-1, 0)
-        const int nw = workers_of(n_valid, nw1, rg);
-        const int64_t C = (int64_t)n_valid + U;
-        const int64_t c1 = p + u;
-        const int64_t c0 = p > 0 ? p - 1 + before : -1;
-        for (int64_t q = ((c0 + 1) * nw + C - 1) / C; q < nw; ++q) {
-            const bool here = cost_target((int)q, nw, C) <= c1;
-            if (!here && p + 1 < n_valid)
-                break;
-            bounds[q] = here ? (int)p : n_valid;
-            int2 cut = make_int2(-1, 0);
-            if (here && s < p && q > 0 && cost_target((int)q - 1, nw, C) <= (int64_t)s + u)
-                cut = make_int2(u, worker_of(e - 1, u, nw, C));
-            cuts[q] = cut;
-        }
-        if (p + 1 == n_valid)
-            bounds[nw] = n_valid;
+        worker_starts<int64_t>(p, u, before, s, e, n_valid, U, nw1, rg, bounds, cuts, 0, 1);
         return;
     }
     const int nwin = (int)((N + kWinBits - 1) / kWinBits);
@@ -483,129 +498,210 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
 }
 
 // ---------------------------------------------------------------------------
-// Dedup of a small batch (N <= kSmallN) in one launch: a warp per occurrence
-// compares its id with every other one in shared memory, which gives the
-// occurrence's sorted position at once.  Runs are numbered by their first
-// position (uniq holds -1 elsewhere, and n_unique is the number of
-// positions), so nothing has to be scanned.  N^2 comparisons: 1 us for 1024
-// occurrences; the four kernels above, a few trips to L2 and a launch each,
-// take 13.7 us.  The CTAs from `nkey` on decay r on the rows outside the
-// batch, kScanTile-sized ranges as in k_sp_scan, from a bitmap of the ids.
+// Dedup of a small batch (N <= kSmallN) in one launch.  Every CTA takes the
+// batch into shared memory, where a hash table picks one occurrence of every
+// id to stand for it; a warp per occurrence then counts the smaller
+// occurrences, those among them that stand for their id, and the earlier ones
+// of its own id, which gives its sorted position and the number of its run.
+// Nothing has to be scanned, and numbers, worker starts and the order in
+// which r is summed are those of the four kernels above, so that a batch gives
+// the same bits however many skipped ids it is padded with.
+//   Bound by the N^2 integer compares and adds, over the CTAs, so a skewed
+// batch takes no longer than a flat one.  50257 x 768, Zipf ids, us per step
+// with it and with the four kernels: 1024 ids 25.3 and 30.2, 1536 25.9 and
+// 29.4, 2048 29.2 and 30.9, 3000 30.8 and 31.7 (262144 x 2048: 38.3 and 38.0).
+// Without the table, runs numbered by their first position, 1024 ids took
+// 24.6, but the workers' shares and the sums of r depended on the padding.
+//   The CTAs from `nkey` on decay r on the rows outside the batch, the ranges
+// and tiles of k_sp_scan, from a bitmap of the ids.
 // ---------------------------------------------------------------------------
+constexpr int kSmallThreads = 512;
+constexpr int kBitmapWords = 2048;
+constexpr int small_pad(int N) { return (N + 127) / 128 * 128; }
+// 1 << log_slots entries of the hash table: at least half stay empty.
+constexpr int small_log_slots(int N)
+{
+    int log_slots = 7;
+    while (1 << log_slots < 2 * N)
+        ++log_slots;
+    return log_slots;
+}
+// The ids, their weights, the table (or the bitmap).  Never less than kSmallSmem: what a kernel asks for
+// decides how its SMs split shared memory and L1, and with the 12 KB that
+// 1024 occurrences needed at first the step took 26.5 us (50257 x 768), with
+// twice as much or more 25.4.
+constexpr size_t kSmallSmem = 46 << 10;
+constexpr size_t small_smem(int N)
+{
+    const size_t slots = (size_t)1 << small_log_slots(N);
+    const size_t b = sizeof(int) * (2 * (size_t)small_pad(N) + (slots > kBitmapWords ? slots : kBitmapWords));
+    return b > kSmallSmem ? b : kSmallSmem;
+}
 template <typename IdT>
-__global__ void __launch_bounds__(kSpThreads)
+__global__ void __launch_bounds__(kSmallThreads)
 k_sp_dedup_small(const IdT *__restrict__ ids, int N, int64_t V, int32_t *__restrict__ perm,
                  int32_t *__restrict__ segidx, int32_t *__restrict__ uniq, int32_t *__restrict__ single,
                  int32_t *__restrict__ bounds, int2 *__restrict__ cuts, int nw1, int rg, DevScalars *sc, int nkey,
-                 int64_t len, float *__restrict__ r, EmaPair ema, float *__restrict__ rsum_part)
+                 int npad, int log_slots, int64_t len, float *__restrict__ r, EmaPair ema,
+                 float *__restrict__ rsum_part)
 {
-    constexpr int kW = kSpThreads / 32;
+    constexpr int kW = kSmallThreads / 32;
     constexpr int kNone = 0x7fffffff;  // a skipped id: V < 2^31, so every valid one is below
-    constexpr int kBitWords = 2048;
-    __shared__ __align__(16) int sid[kSmallN];
-    __shared__ unsigned bits[kBitWords];
-    __shared__ float wr[kW];
+    constexpr int kFree = -1;
+    __shared__ int total[2];  // distinct ids, valid ones
+    __shared__ float wr[kSpThreads / 32];
+    extern __shared__ __align__(16) int sid[];  // the ids, npad of them
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int npad = (N + 127) / 128 * 128;
+    // 1, plus 1 << 16 where the occurrence stands for its id
+    unsigned *const weight = reinterpret_cast<unsigned *>(sid + npad);
+    int *const words = sid + 2 * npad;  // hash table of the ids, or a bitmap of a range's ids
+    const bool keys = (int)blockIdx.x < nkey;
+    if (keys) {
+        for (int q = tid; q < 1 << log_slots; q += kSmallThreads)
+            words[q] = kFree;
+        if (tid < 2)
+            total[tid] = 0;
+        __syncthreads();
+    }
     grid_dep_wait();  // whatever ran before on the stream
     grid_dep_launch();
     bool bad = false;
-    for (int q = tid; q < npad; q += kSpThreads) {
-        int x = kNone;
-        if (q < N) {
-            const int64_t id = (int64_t)ids[q];
-            if (id >= 0 && id < V)
-                x = (int)id;
-            else
-                bad = true;
+    int U = 0, valid = 0;
+    constexpr int kAtOnce = 4;
+    for (int q0 = tid; q0 < npad; q0 += kAtOnce * kSmallThreads) {
+        int64_t id[kAtOnce];
+#pragma unroll
+        for (int e = 0; e < kAtOnce; ++e)
+            id[e] = q0 + e * kSmallThreads < N ? (int64_t)ids[q0 + e * kSmallThreads] : 0;
+#pragma unroll
+        for (int e = 0; e < kAtOnce; ++e) {
+            const int q = q0 + e * kSmallThreads;
+            if (q >= npad)
+                break;  // whole warps: npad is a multiple of 32
+            const bool ok = q < N && id[e] >= 0 && id[e] < V;
+            bad |= q < N && !ok;
+            const int x = ok ? (int)id[e] : kNone;
+            sid[q] = x;
+            if (!keys)
+                continue;
+            // an entry holds the id that took it; whoever took it stands for the id
+            int was = x;
+            if (ok)
+                for (unsigned h = (unsigned)x * 2654435761u >> (32 - log_slots);;  // Fibonacci hashing
+                     h = (h + 1) & ((1u << log_slots) - 1)) {
+                    was = *(volatile int *)(words + h);
+                    if (was == kFree)
+                        was = atomicCAS(words + h, kFree, x);
+                    if (was == kFree || was == x)
+                        break;
+                }
+            weight[q] = was == kFree ? 1u + (1u << 16) : 1u;
+            U += __popc(__ballot_sync(0xffffffffu, was == kFree));
+            valid += __popc(__ballot_sync(0xffffffffu, ok));
         }
-        sid[q] = x;
     }
     if (bad && blockIdx.x == 0)
         atomicOr(&sc->flags, kFlagIdRange);
+    if (keys && lane == 0) {
+        atomicAdd(&total[0], U);
+        atomicAdd(&total[1], valid);
+    }
     __syncthreads();
-    if ((int)blockIdx.x < nkey) {
+    if (keys) {
+        U = total[0];
+        valid = total[1];
+        if (blockIdx.x == 0 && tid == 0) {
+            sc->n_unique = U;
+            sc->n_valid = valid;
+        }
         const int k = (int)blockIdx.x * kW + w;
         if (k >= N)
             return;
         const int x = sid[k];
-        int less = 0, before = 0, same = 0, valid = 0;
-        for (int q = lane * 4; q < npad; q += 128) {
-            const int4 v = *reinterpret_cast<const int4 *>(sid + q);
-            const int y[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                less += y[e] < x;
-                same += y[e] == x;
-                before += y[e] == x && q + e < k;
-                valid += y[e] != kNone;
-            }
-        }
-        less = __reduce_add_sync(0xffffffffu, less);
-        same = __reduce_add_sync(0xffffffffu, same);
-        before = __reduce_add_sync(0xffffffffu, before);
-        valid = __reduce_add_sync(0xffffffffu, valid);
-        if (k == 0 && lane == 0)
-            sc->n_unique = sc->n_valid = valid;
         if (x == kNone)
             return;
+        // smaller occurrences and, in the upper half, smaller distinct ids;
+        // occurrences of x before k and from k on
+        unsigned below = 0;
+        int before = 0, after = 0;
+        auto smaller = [&](const int4 &y, int q) {
+            const uint4 o = *reinterpret_cast<const uint4 *>(weight + q);
+            below += (y.x < x ? o.x : 0u) + (y.y < x ? o.y : 0u) + (y.z < x ? o.z : 0u) + (y.w < x ? o.w : 0u);
+        };
+        int q = lane * 4;
+        for (; q + 3 < k; q += 128) {
+            const int4 y = *reinterpret_cast<const int4 *>(sid + q);
+            smaller(y, q);
+            before += (y.x == x) + (y.y == x) + (y.z == x) + (y.w == x);
+        }
+        for (; q < npad; q += 128) {
+            const int4 y = *reinterpret_cast<const int4 *>(sid + q);
+            smaller(y, q);
+            after += (y.x == x) + (y.y == x) + (y.z == x) + (y.w == x);
+            if (q < k) {  // the four that hold k - 1 and k
+                const int some = (y.x == x) + (q + 1 < k && y.y == x) + (q + 2 < k && y.z == x);
+                before += some;
+                after -= some;
+            }
+        }
+        below = __reduce_add_sync(0xffffffffu, below);
+        before = __reduce_add_sync(0xffffffffu, before);
+        const int same = before + __reduce_add_sync(0xffffffffu, after);
+        const int less = below & 0xffffu, u = below >> 16;
         const int p = less + before;
         if (lane == 0) {
             perm[p] = k;
-            segidx[p] = less;
-            uniq[p] = before == 0 ? x : -1;
-            single[p] = same == 1 ? k : -1;
-        }
-        // the workers that start here (equal shares of the positions), and
-        // the run each start cuts, as in k_sp_order
-        const int nw = workers_of(valid, nw1, rg);
-        for (int q = (p * nw + valid - 1) / valid + lane; q < nw && q * valid / nw == p; q += 32) {
-            bounds[q] = p;
-            int2 cut = make_int2(-1, 0);
-            if (before > 0 && q > 0 && (q - 1) * valid / nw <= less) {
-                int to = (less + same - 1) * nw / valid;  // the worker whose range holds the run's last position
-                while (to + 1 < nw && (to + 1) * valid / nw <= less + same - 1)
-                    ++to;
-                cut = make_int2(less, to);
+            segidx[p] = u;
+            if (before == 0) {
+                uniq[u] = x;
+                single[u] = same == 1 ? k : -1;
             }
-            cuts[q] = cut;
         }
-        if (p + 1 == valid && lane == 0)
-            bounds[nw] = valid;
+        worker_starts<int>(p, u, before > 0 ? u : u - 1, less, less + same, valid, U, nw1, rg, bounds, cuts, lane, 32);
         return;
     }
+    constexpr int kBitmapIds = 32 * kBitmapWords;  // a multiple of kScanTile
     const int64_t b = (int)blockIdx.x - nkey;
     const int64_t i1 = (b + 1) * len < V ? (b + 1) * len : V;
     float rsum = 0.f;
-    for (int64_t c0 = b * len; c0 < i1; c0 += 32 * kBitWords) {
-        const int n = (int)(i1 - c0 < 32 * kBitWords ? i1 - c0 : 32 * kBitWords);
-        for (int q = tid; q < (n + 31) / 32; q += kSpThreads)
-            bits[q] = 0u;
+    for (int64_t c0 = b * len; c0 < i1; c0 += kBitmapIds) {
+        const int n = (int)(i1 - c0 < kBitmapIds ? i1 - c0 : kBitmapIds);
+        for (int q = tid; q < (n + 31) / 32; q += kSmallThreads)
+            words[q] = 0;
         __syncthreads();
-        for (int q = tid; q < N; q += kSpThreads) {
+        for (int q = tid; q < N; q += kSmallThreads) {
             const int64_t o = sid[q] - c0;
-            if (o >= 0 && o < n)
-                atomicOr(&bits[o >> 5], 1u << (o & 31));
+            // (a frequent id's bit is mostly there already)
+            if (o >= 0 && o < n && !((unsigned)*(volatile int *)(words + (o >> 5)) >> (o & 31) & 1u))
+                atomicOr(&words[o >> 5], (int)(1u << (o & 31)));
         }
         __syncthreads();
-#pragma unroll 4
-        for (int q = tid; q < n; q += kSpThreads)
-            if (!(bits[q >> 5] >> (q & 31) & 1u)) {
-                const float rn = ema_pair(ema, r[c0 + q], 0.f);
-                r[c0 + q] = rn;
-                rsum += rn;
-            }
+        // by the threads and in the order of k_sp_scan
+        for (int q = tid * kScanPer; tid < kSpThreads && q < n; q += kScanTile) {
+            float rr[kScanPer];
+            const unsigned in = (unsigned)words[q >> 5] >> (q & 31);
+#pragma unroll
+            for (int e = 0; e < kScanPer; ++e)
+                rr[e] = q + e < n ? r[c0 + q + e] : 0.f;
+#pragma unroll
+            for (int e = 0; e < kScanPer; ++e)
+                if (q + e < n && !(in >> e & 1u)) {
+                    const float rn = ema_pair(ema, rr[e], 0.f);
+                    r[c0 + q + e] = rn;
+                    rsum += rn;
+                }
+        }
         __syncthreads();
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1)
         rsum += __shfl_xor_sync(0xffffffffu, rsum, o);
-    if (lane == 0)
+    if (lane == 0 && w < kSpThreads / 32)
         wr[w] = rsum;
     __syncthreads();
     if (tid == 0) {
         float t = 0.f;
-        for (int q = 0; q < kW; ++q)
+        for (int q = 0; q < kSpThreads / 32; ++q)
             t += wr[q];
         rsum_part[b] = t;
     }
@@ -1326,13 +1422,17 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     const int G = kSparseCtas;
     const StepConsts kc = make_consts(a.beta2, a.one_minus_beta2, a.V, a.D, a.inv_bc);
     if (a.N > 0 && a.N <= kSmallN) {
-        const int nkey = (int)((a.N + kSpThreads / 32 - 1) / (kSpThreads / 32));
+        const int nkey = (int)((a.N + kSmallThreads / 32 - 1) / (kSmallThreads / 32));
+        const size_t sm = small_smem((int)a.N);
         auto go = [&](auto *ids) {
             using IdT = std::remove_const_t<std::remove_pointer_t<decltype(ids)>>;
-            la.launch(k_sp_dedup_small<IdT>, dim3(nkey + scan_ranges(a.V)), dim3(kSpThreads), 0,
-                      la.pdl() && small_first_pdl(a.N), ids,
-                     (int)a.N, a.V, perm, segidx, uniq, single, bounds, cuts, G / NS, map.rg, sc, nkey, scan_len(a.V),
-                     a.r, kc.ema, rsum_part);
+            if (sm > (size_t)47 << 10)  // with the static arrays up to 48 KiB need no leave
+                la.err = cudaFuncSetAttribute(k_sp_dedup_small<IdT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)sm);
+            la.launch(k_sp_dedup_small<IdT>, dim3(nkey + scan_ranges(a.V)), dim3(kSmallThreads), sm,
+                      la.pdl() && small_first_pdl(a.N), ids, (int)a.N, a.V, perm, segidx, uniq, single, bounds, cuts,
+                      G / NS, map.rg, sc, nkey, small_pad((int)a.N), small_log_slots((int)a.N), scan_len(a.V), a.r,
+                      kc.ema, rsum_part);
         };
         if (a.ids64)
             go(static_cast<const int64_t *>(a.ids));

@@ -80,7 +80,7 @@ class Fake:
         return st, self.log()
 
 
-KINDS = [("step", 1, 0), ("step", 1, 100), ("step", 0, 4096), ("step", 1, 5000), ("step", 0, 100000),
+KINDS = [("step", 1, 0), ("step", 1, 100), ("step", 0, 3072), ("step", 1, 5000), ("step", 0, 100000),
          ("unique", 1, 100), ("unique", 0, 70000)]
 
 

@@ -181,11 +181,18 @@ def test_sparse_edge_cases(cuda_device):
     assert ex.value.status == EMBER_ERR_WORKSPACE
 
 
-def test_skipped_ids_leave_the_step_bit_identical(cuda_device):
-    """The same batch, and the batch followed by 10000 skipped ids (id -1,
-    whose rows are never read), give bit-identical W and state: skipped ids
-    sort after every valid one, so the segment sums see the same order."""
-    V, D, N, Npad = 20000, 256, 30000, 40000
+@pytest.mark.parametrize("V,D,N,Npad", [
+    (20000, 256, 30000, 40000),
+    # batches that the padding takes from the one-launch dedup (up to 3072
+    # occurrences) to the counting one, and from its direct counts to the table
+    (20000, 256, 3000, 3900), (20000, 256, 3000, 6000), (500, 64, 3072, 3073), (70000, 2048, 1000, 4500),
+    (400000, 203, 3072, 70000), (3000, 1, 1, 5000), (20000, 64, 40000, 66000),
+])
+def test_skipped_ids_leave_the_step_bit_identical(cuda_device, V, D, N, Npad):
+    """The same batch, and the batch followed by skipped ids (id -1, whose
+    rows are never read), give bit-identical W and state: the order of the
+    occurrences, the workers' ranges and every sum are functions of the valid
+    ids alone, whichever form of the dedup the length chooses."""
     ids, rows = batch(V, D, N, 1, cuda_device, seed=11)
     ids_pad = torch.cat([ids, torch.full((Npad - N,), -1, dtype=ids.dtype, device=cuda_device)])
     rows_pad = torch.cat([rows, torch.full((Npad - N, D), float("nan"), device=cuda_device)])
