@@ -107,6 +107,25 @@ def test_sparse_parity(cuda_device, V, D, N, wdtype):
         gated_sparse_step(emb, W, ids, rows, 1e-3, t, opt)
 
 
+@pytest.mark.parametrize("V,D,N", [
+    # 4-byte accesses pass in batches of 24 rows: workers of 23, 24, 25 and 49
+    # rows (33 workers of 9 column slices), one long run over all of them, and
+    # windows of 128 indices (8 groups per CTA) that no batch divides
+    (4000, 2049, 33 * 23), (4000, 2049, 33 * 24), (4000, 2049, 33 * 25), (60000, 2049, 33 * 49), (1, 2049, 5000),
+    (50, 7, 40000), (3000, 131, 20000),
+])
+def test_sparse_parity_in_batches_of_4_byte_rows(cuda_device, V, D, N):
+    """Rows of one sign: a one-row table's c is the square of a single sum of N
+    values, whose relative error is up to 2^-24 sum |x| / |sum x| per rounding;
+    with both signs the smallest of 2049 such sums is 1e4 times smaller than
+    its terms together, with one sign the ratio is 1."""
+    emb = make(V, D, "bf16", N)
+    W = (torch.randn(V, D, device=cuda_device) * 0.02).to(torch.bfloat16)
+    for t in (1, 2):
+        ids, rows = batch(V, D, N, t, cuda_device, seed=D + N)
+        gated_sparse_step(emb, W, ids, rows.abs(), 1e-3, t, Opt())
+
+
 @pytest.mark.parametrize("opt", [Opt(maximize=True), Opt(variant="row"), Opt(variant="col"),
                                  Opt(bias_correction=False), Opt(beta2=0.9, eps=1e-6)],
                          ids=["maximize", "row_only", "col_only", "no_bc", "beta2_0.9"])
