@@ -405,6 +405,11 @@ __device__ __forceinline__ void worker_starts(int p, int u, int before, int s, i
 // run is bound by its trips to L2, so a thread has 16 occurrences in flight.
 constexpr int kWinWords = 2048;
 constexpr int kWinBits = 32 * kWinWords;
+// Runs from this length on are looked through for stretches of nothing but one
+// id (padding): read back a lane per word, 40000 equal ids take 42 us here,
+// and 28 a lane per bit.  Asking costs short runs (262144 Zipf ids have
+// hardly a full word) more than it gives.
+constexpr int kStretch = 4096;
 __global__ void __launch_bounds__(kOrderThreads)
 k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segidx,
            const int32_t *__restrict__ segoff, const int32_t *__restrict__ longrun,
@@ -487,9 +492,22 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
             const int n = __popc(m);
             const int x = warp_scan(n, lane);
             int o = at + x - n;
-            while (m) {
-                perm[o++] = (int)(k0 + (int64_t)(q + lane) * 32 + __ffs(m) - 1);
-                m &= m - 1;
+            if (e - s >= kStretch && __any_sync(0xffffffffu, m == 0xffffffffu)) {
+                // a stretch of nothing but this id (a batch of padding): a lane
+                // per bit, a word at a time, so that the warp's writes are
+                // adjacent
+#pragma unroll 4
+                for (int k = 0; k < 32; ++k) {
+                    const unsigned mk = __shfl_sync(0xffffffffu, m, k);
+                    const int ok = __shfl_sync(0xffffffffu, o, k);
+                    if (mk >> lane & 1u)
+                        perm[ok + __popc(mk & ((1u << lane) - 1u))] = (int)(k0 + (int64_t)(q + k) * 32 + lane);
+                }
+            } else {
+                while (m) {
+                    perm[o++] = (int)(k0 + (int64_t)(q + lane) * 32 + __ffs(m) - 1);
+                    m &= m - 1;
+                }
             }
             at += __shfl_sync(0xffffffffu, x, 31);
         }

@@ -53,3 +53,28 @@ def test_order_within_runs_is_deterministic(cuda_device):
     for W, st in outs[1:]:
         assert torch.equal(W.view(torch.int32), outs[0][0].view(torch.int32))
         assert torch.equal(st.view(torch.int32), outs[0][1].view(torch.int32))
+
+
+@pytest.mark.parametrize("lead,length", [(0, 5000), (17, 4095), (32, 4096), (5, 70001), (65530, 9000)])
+def test_stretches_of_one_id(cuda_device, lead, length):
+    """Stretches of one id (a padded batch): whole words of the bitmap, partial
+    ones at both ends, one window and several, other ids of the run around."""
+    V, D = 3000, 64
+    g = torch.Generator(device=cuda_device).manual_seed(length)
+    noise = torch.randint(0, V, (lead + 3000,), generator=g, device=cuda_device)
+    pad = torch.full((length,), 5, device=cuda_device)
+    mixed = torch.where(torch.rand(2000, generator=g, device=cuda_device) < 0.9, 5, 6)
+    ids = torch.cat([noise[:lead], pad, noise[lead:], mixed, pad])
+    N = ids.numel()
+    emb = Ember(V, D, wdtype="f32", max_sparse_N=N, device=cuda_device)
+    W = torch.randn(V, D, generator=g, device=cuda_device)
+    rows = torch.rand(N, D, generator=g, device=cuda_device) * 1e-4
+    gated_sparse_step(emb, W, ids, rows, 1e-3, 1, Opt())
+    # in increasing occurrence: the same bits as the batch sorted by id beforehand
+    order = torch.sort(ids, stable=True).indices
+    ref = Ember(V, D, wdtype="f32", max_sparse_N=N, device=cuda_device)
+    emb.state.zero_()
+    W1, W2 = W.clone(), W.clone()
+    emb.step_sparse(W1, ids, rows, 1e-3, 1)
+    ref.step_sparse(W2, ids[order], rows[order].contiguous(), 1e-3, 1)
+    assert torch.equal(W1, W2) and torch.equal(emb.state, ref.state)
