@@ -768,10 +768,31 @@ cudaError_t launch_apply_t(const ApplyArgs &a, const ApplyMap &m, bool bf16)
                     m.lpr, m.nseg, a.mis, a.kc, a.eps, a.lr_signed, a.variant, a.span);
 }
 
+// Whether rows of pw columns that start on no 16-byte boundary take shifted
+// 16-byte accesses in the update rather than 4-byte ones.  A row's two partial
+// accesses go element by element, which short rows (above all of bf16
+// weights) do not earn back, nor do widths just past a power of two, where the
+// shifted form covers the row with half as many lanes instead of a quarter.
+// Steps of 400000 rows, us shifted and 4-byte: fp32 7 columns 42.6 and 40.4, 9
+// 42.8 and 48.7, 61 95 and 106, 63 135 and 107, 127 186 and 174, 129 198 and
+// 256, 255 298 and 321; bf16 9 49.5 and 49.6, 41 114 and 97, 125 190 and 160,
+// 127 233 and 160, 129 243 and 244, 255 331 and 295, 257 359 and 510.
+bool shifted_pays(int pw, bool bf16)
+{
+    auto lanes = [&](bool rag) {
+        const ApplyMap m = apply_map(pw, rag ? 4 : 1, rag, bf16);
+        return m.lpr * m.k * m.nseg;
+    };
+    if (pw < (bf16 ? 128 : 8))
+        return false;
+    return pw >= (bf16 ? 256 : 128) || 2 * lanes(true) < lanes(false);
+}
+
 // vec 4: every row starts on a 16-byte boundary of G (and as many elements
 // of W); rag: only W and G themselves do; otherwise 4-byte accesses.
 cudaError_t launch_apply(const ApplyArgs &a, int vec, bool rag, bool bf16)
 {
+    rag = rag && shifted_pays(a.D, bf16);
     const ApplyMap m = apply_map(a.D, vec, rag, bf16);
     if (rag) {
         switch (m.k) {
