@@ -717,7 +717,9 @@ k_apply_dense(void *__restrict__ W, const float *__restrict__ G, const float *__
 // and unit, R row blocks per unit, segments of 32 K accesses chosen equal so
 // that few lanes are idle.  R K accesses of G and W are in flight per lane:
 // about 8 with bf16 weights and 4 to 6 with fp32 ones, 65 to 100 KB per SM
-// either way.  More makes the step slower, not only less: 32000 x 4096 fp32
+// either way, and 16 accesses of 4 bytes (of 8, 40 KB, the step takes 804 us on
+// 128256 x 2048 with bf16 weights off a 16-byte boundary, of 16 627, and after
+// the LM-head GEMM of 512 tokens 954 and 775).  More makes the step slower, not only less: 32000 x 4096 fp32
 // takes 326.5 us with 4 (66 KB) and 334 with 8 (131 KB); bf16 50257 x 768
 // takes 88 us with 6 (74 KB), 104 with 3 and 94 with three CTAs per SM.
 struct ApplyMap {
@@ -771,21 +773,23 @@ cudaError_t launch_apply_t(const ApplyArgs &a, const ApplyMap &m, bool bf16)
 // Whether rows of pw columns that start on no 16-byte boundary take shifted
 // 16-byte accesses in the update rather than 4-byte ones.  A row's two partial
 // accesses go element by element, which short rows (above all of bf16
-// weights) do not earn back, nor do widths just past a power of two, where the
-// shifted form covers the row with half as many lanes instead of a quarter.
-// Steps of 400000 rows, us shifted and 4-byte: fp32 7 columns 42.6 and 40.4, 9
-// 42.8 and 48.7, 61 95 and 106, 63 135 and 107, 127 186 and 174, 129 198 and
-// 256, 255 298 and 321; bf16 9 49.5 and 49.6, 41 114 and 97, 125 190 and 160,
-// 127 233 and 160, 129 243 and 244, 255 331 and 295, 257 359 and 510.
+// weights) do not earn back, nor do widths just past a power of two, where few
+// of the shifted form's lanes have anything to do.  Steps of 63e6 elements (of
+// 400000 rows below 157 columns), us shifted and 4-byte: fp32 7 columns 42.8
+// and 40.5, 9 42.9 and 48.7, 33 86.7 and 85.7, 61 95.8 and 95.0, 63 137 and 96,
+// 97 151 and 143, 129 199 and 220, 255 190 and 182, 257 210 and 286, 1023 184
+// and 182, 1119 194 and 217; bf16 29 66 and 68, 61 119 and 90, 129 247 and 211,
+// 253 181 and 164, 257 228 and 276, 511 169 and 163, 513 191 and 208, 1003 140
+// and 165, 1025 204 and 192, 2047 143 and 166.
 bool shifted_pays(int pw, bool bf16)
 {
     auto lanes = [&](bool rag) {
         const ApplyMap m = apply_map(pw, rag ? 4 : 1, rag, bf16);
         return m.lpr * m.k * m.nseg;
     };
-    if (pw < (bf16 ? 128 : 8))
-        return false;
-    return pw >= (bf16 ? 256 : 128) || 2 * lanes(true) < lanes(false);
+    if (bf16)
+        return pw >= 256 && 5 * lanes(true) < 2 * lanes(false);
+    return pw >= 256 || ((pw >= 128 || (pw >= 8 && pw < 64)) && 2 * lanes(true) < lanes(false));
 }
 
 // vec 4: every row starts on a 16-byte boundary of G (and as many elements
@@ -815,9 +819,9 @@ cudaError_t launch_apply(const ApplyArgs &a, int vec, bool rag, bool bf16)
     } else {
         switch (m.k) {
         case 1: return launch_apply_t<1, 1, 8, 8, false>(a, m, bf16);
-        case 2: return launch_apply_t<1, 2, 4, 4, false>(a, m, bf16);
-        case 4: return launch_apply_t<1, 4, 2, 2, false>(a, m, bf16);
-        case 8: return launch_apply_t<1, 8, 1, 1, false>(a, m, bf16);
+        case 2: return launch_apply_t<1, 2, 8, 8, false>(a, m, bf16);
+        case 4: return launch_apply_t<1, 4, 4, 4, false>(a, m, bf16);
+        case 8: return launch_apply_t<1, 8, 2, 2, false>(a, m, bf16);
         }
     }
     return cudaErrorInvalidValue;

@@ -21,7 +21,8 @@ def shifted(x, by):
 @pytest.mark.parametrize("V,D", [(5, 1), (9, 2), (300, 3), (700, 5), (305, 31), (306, 33), (1000, 61), (257, 127),
                                  (999, 130), (777, 253),
                                  # both sides of the widths from which shifted accesses are taken
-                                 (500, 7), (500, 9), (400, 63), (400, 65), (400, 129), (300, 255), (300, 257), (100, 511), (310, 509), (305, 1021), (306, 1025), (40, 2047),
+                                 (500, 7), (500, 9), (400, 63), (400, 65), (400, 129), (300, 255), (300, 257), (100, 511), (100, 513),
+                                 (60, 1027), (33, 2047), (310, 509), (305, 1021), (306, 1025), (40, 2047),
                                  (33, 2049), (21, 3001)])
 @pytest.mark.parametrize("wdtype", ["bf16", "f32"])
 @pytest.mark.parametrize("variant", ["full", "col"])
