@@ -184,10 +184,54 @@ k_sp_count(const IdT *__restrict__ ids, int64_t N, int64_t V, int32_t *__restric
 // number.  Runs longer than kLongRun are listed for k_sp_order (in any
 // order).  With r: the rows outside the batch decay, r_i <- beta2 r_i (their
 // g is 0), and the CTA's fp32 sum of them goes to rsum_part[b]; the touched
-// rows are left to the state pass.  A CTA's loads are one trip to L2 when
-// its range is one tile (V up to kScanCtas x kScanTile).
+// rows are left to the state pass.
+//   A range of one tile (V up to kScanCtas x kScanTile) is one trip to L2.
+// The ranges of taller tables are bound by bandwidth: TILES tiles are loaded
+// at once, and batches of tiles that no id is in, most of them, are not
+// numbered.  With one tile at a time and 4-byte accesses of r, 8192 ids over
+// 2^24 x 16 took 126 us and over 2^26 x 8 368; now 87 and 188 (4 tiles 89 and
+// 194).
 constexpr int kScanPer = 4;                        // ids per thread of a tile
 constexpr int kScanTile = kSpThreads * kScanPer;
+
+// r_i .. r_{i+3} below i1 (0 past it), in one access where r allows it.
+__device__ __forceinline__ void load_r4(const float *r, bool aligned, int64_t i, int64_t i1,
+                                        float (&x)[kScanPer])
+{
+    if (aligned && i + 3 < i1) {
+        const float4 v = *reinterpret_cast<const float4 *>(r + i);
+        x[0] = v.x;
+        x[1] = v.y;
+        x[2] = v.z;
+        x[3] = v.w;
+    } else {
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e)
+            x[e] = i + e < i1 ? r[i + e] : 0.f;
+    }
+}
+
+// The rows of i .. i + 3 that `touched` does not mark decay, r_i <- beta2 r_i
+// (their g is 0); their new r is added to rsum in order.
+__device__ __forceinline__ void decay_r4(float *r, bool aligned, int64_t i, int64_t i1,
+                                         const EmaPair &ema, unsigned touched, float (&x)[kScanPer], float &rsum)
+{
+#pragma unroll
+    for (int e = 0; e < kScanPer; ++e)
+        if (i + e < i1 && !(touched >> e & 1u)) {
+            x[e] = ema_pair(ema, x[e], 0.f);
+            rsum += x[e];
+        }
+    if (aligned && i + 3 < i1 && (touched & 15u) == 0)
+        *reinterpret_cast<float4 *>(r + i) = make_float4(x[0], x[1], x[2], x[3]);
+    else
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e)
+            if (i + e < i1 && !(touched >> e & 1u))
+                r[i + e] = x[e];
+}
+
+template <int TILES>
 __global__ void __launch_bounds__(kSpThreads)
 k_sp_scan(int32_t *__restrict__ slot, int64_t V, int64_t len, const int32_t *__restrict__ rng,
           int32_t *__restrict__ uniq, int32_t *__restrict__ segoff, int32_t *__restrict__ longrun,
@@ -195,7 +239,8 @@ k_sp_scan(int32_t *__restrict__ slot, int64_t V, int64_t len, const int32_t *__r
           float *__restrict__ rsum_part)
 {
     constexpr int kW = kSpThreads / 32;
-    __shared__ int wh[2][kW], wv[2][kW];
+    __shared__ int bh[kW], bv[kW];  // of the ranges before this one, per warp of the sum
+    __shared__ int wh[TILES][kW], wv[TILES][kW];
     __shared__ float wr[kW];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int64_t i0 = (int64_t)blockIdx.x * len;
@@ -211,72 +256,96 @@ k_sp_scan(int32_t *__restrict__ slot, int64_t V, int64_t len, const int32_t *__r
     h = __reduce_add_sync(0xffffffffu, h);
     v = __reduce_add_sync(0xffffffffu, v);
     if (lane == 0) {
-        wh[1][w] = h;
-        wv[1][w] = v;
+        bh[w] = h;
+        bv[w] = v;
     }
     float rsum = 0.f;
-    int run = 0, pos = 0;  // of the next tile (tile 0: added from wh[1] and wv[1])
-    int buf = 0;
-    for (int64_t t0 = i0; t0 < i1; t0 += kScanTile) {
-        const int64_t i = t0 + (int64_t)tid * kScanPer;  // len and kScanPer are multiples of 4
-        int c[kScanPer];
-        float rr[kScanPer];
-        const int4 c4 = (i + 3 < i1) ? __ldcg(reinterpret_cast<const int4 *>(slot + i)) : make_int4(0, 0, 0, 0);
-        c[0] = c4.x;
-        c[1] = c4.y;
-        c[2] = c4.z;
-        c[3] = c4.w;
+    const bool aligned = (uintptr_t)r % 16 == 0;  // len is a multiple of 4
+    int run = 0, pos = 0;  // of the next tile
+    for (int64_t tb = i0; tb < i1; tb += TILES * kScanTile) {
+        int c[TILES][kScanPer];
+        float rr[TILES][kScanPer];
 #pragma unroll
-        for (int e = 0; e < kScanPer; ++e) {
-            if (i + 3 >= i1)
-                c[e] = (i + e < i1) ? __ldcg(slot + i + e) : 0;
-            rr[e] = (r && i + e < i1) ? r[i + e] : 0.f;
-        }
-        int nh = 0, nv = 0;
+        for (int d = 0; d < TILES; ++d) {
+            const int64_t i = tb + d * kScanTile + (int64_t)tid * kScanPer;  // a multiple of 4, as len is
+            if (i + 3 < i1) {
+                const int4 v = __ldcg(reinterpret_cast<const int4 *>(slot + i));
+                c[d][0] = v.x;
+                c[d][1] = v.y;
+                c[d][2] = v.z;
+                c[d][3] = v.w;
+            } else {
 #pragma unroll
-        for (int e = 0; e < kScanPer; ++e) {
-            nh += c[e] > 0;
-            nv += c[e];
+                for (int e = 0; e < kScanPer; ++e)
+                    c[d][e] = (i + e < i1) ? __ldcg(slot + i + e) : 0;
+            }
+            if (r)
+                load_r4(r, aligned, i, i1, rr[d]);
         }
-        const int xh = warp_scan(nh, lane), xv = warp_scan(nv, lane);
-        if (lane == 31) {
-            wh[buf][w] = xh;
-            wv[buf][w] = xv;
+        // distinct ids and occurrences before this thread's, within its warp
+        int xh[TILES], xv[TILES];
+        bool any = false;
+#pragma unroll
+        for (int d = 0; d < TILES; ++d) {
+            int nh = 0, nv = 0;
+#pragma unroll
+            for (int e = 0; e < kScanPer; ++e) {
+                nh += c[d][e] > 0;
+                nv += c[d][e];
+            }
+            xh[d] = xv[d] = 0;
+            int th = 0, tv = 0;  // of the warp
+            if (TILES == 1 || __any_sync(0xffffffffu, nv)) {  // (a tall table has mostly empty stretches)
+                th = warp_scan(nh, lane);
+                tv = warp_scan(nv, lane);
+                xh[d] = th - nh;
+                xv[d] = tv - nv;
+                any = true;
+            }
+            if (lane == 31) {
+                wh[d][w] = th;
+                wv[d][w] = tv;
+            }
         }
-        __syncthreads();
-        if (t0 == i0) {
+        any = __syncthreads_or(any);
+        if (tb == i0) {
 #pragma unroll
             for (int q = 0; q < kW; ++q) {
-                run += wh[1][q];
-                pos += wv[1][q];
-            }
-            __syncthreads();  // before the next tile writes wh[1]
-        }
-        int u = run + xh - nh, p = pos + xv - nv;
-#pragma unroll
-        for (int q = 0; q < kW; ++q) {
-            u += q < w ? wh[buf][q] : 0;
-            p += q < w ? wv[buf][q] : 0;
-            run += wh[buf][q];
-            pos += wv[buf][q];
-        }
-#pragma unroll
-        for (int e = 0; e < kScanPer; ++e) {
-            if (c[e] > 0) {
-                uniq[u] = (int)(i + e);
-                segoff[u] = p;
-                if (c[e] > kLongRun)
-                    longrun[atomicAdd(nlong, 1)] = u;
-                ++u;
-                slot[i + e] = u;
-                p += c[e];
-            } else if (r && i + e < i1) {
-                const float rn = ema_pair(ema, rr[e], 0.f);
-                r[i + e] = rn;
-                rsum += rn;
+                run += bh[q];
+                pos += bv[q];
             }
         }
-        buf ^= 1;
+#pragma unroll
+        for (int d = 0; d < TILES; ++d) {
+            const int64_t i = tb + d * kScanTile + (int64_t)tid * kScanPer;
+            unsigned touched = 0;
+            if (any) {
+                int u = run + xh[d], p = pos + xv[d];
+#pragma unroll
+                for (int q = 0; q < kW; ++q) {
+                    u += q < w ? wh[d][q] : 0;
+                    p += q < w ? wv[d][q] : 0;
+                    run += wh[d][q];
+                    pos += wv[d][q];
+                }
+#pragma unroll
+                for (int e = 0; e < kScanPer; ++e)
+                    if (c[d][e] > 0) {
+                        uniq[u] = (int)(i + e);
+                        segoff[u] = p;
+                        if (c[d][e] > kLongRun)
+                            longrun[atomicAdd(nlong, 1)] = u;
+                        ++u;
+                        slot[i + e] = u;
+                        p += c[d][e];
+                        touched |= 1u << e;
+                    }
+            }
+            if (r)
+                decay_r4(r, aligned, i, i1, ema, touched, rr[d], rsum);
+        }
+        if (TILES > 1 && any)
+            __syncthreads();  // before the next batch writes wh
     }
     if (blockIdx.x == gridDim.x - 1 && tid == 0) {
         sc->n_unique = run;
@@ -679,6 +748,7 @@ k_sp_dedup_small(const IdT *__restrict__ ids, int N, int64_t V, int32_t *__restr
         return;
     }
     constexpr int kBitmapIds = 32 * kBitmapWords;  // a multiple of kScanTile
+    const bool aligned = (uintptr_t)r % 16 == 0;
     const int64_t b = (int)blockIdx.x - nkey;
     const int64_t i1 = (b + 1) * len < V ? (b + 1) * len : V;
     float rsum = 0.f;
@@ -697,17 +767,8 @@ k_sp_dedup_small(const IdT *__restrict__ ids, int N, int64_t V, int32_t *__restr
         // by the threads and in the order of k_sp_scan
         for (int q = tid * kScanPer; tid < kSpThreads && q < n; q += kScanTile) {
             float rr[kScanPer];
-            const unsigned in = (unsigned)words[q >> 5] >> (q & 31);
-#pragma unroll
-            for (int e = 0; e < kScanPer; ++e)
-                rr[e] = q + e < n ? r[c0 + q + e] : 0.f;
-#pragma unroll
-            for (int e = 0; e < kScanPer; ++e)
-                if (q + e < n && !(in >> e & 1u)) {
-                    const float rn = ema_pair(ema, rr[e], 0.f);
-                    r[c0 + q + e] = rn;
-                    rsum += rn;
-                }
+            load_r4(r, aligned, c0 + q, c0 + n, rr);
+            decay_r4(r, aligned, c0 + q, c0 + n, ema, (unsigned)words[q >> 5] >> (q & 31), rr, rsum);
         }
         __syncthreads();
     }
@@ -1354,6 +1415,17 @@ int64_t scan_len(int64_t V)
 }
 int scan_ranges(int64_t V) { return (int)((V + scan_len(V) - 1) / scan_len(V)); }
 
+// Tiles in flight in a CTA of the scan of a tall table.
+constexpr int kTallTiles = 8;
+
+// Whether the kernels that read a range of the table per CTA are launched
+// early.  Of a tall table that loses more than the launch latency it gains:
+// 8 ids over 2^24 x 16 49 us early and 37 not, 8192 ids over 2^22 x 64 52.7
+// and 50.9; over 2^20 x 64 22.2 and 23.9, 45.3 and 46.4.  (CTAs launched onto
+// SMs that are still busy are spread unevenly, likely, and a long range is
+// bound by bandwidth.)
+bool early_ranges(int64_t V) { return V <= int64_t(1) << 22; }
+
 // Count the ids and number the distinct ones; with r also decay the rows
 // outside the batch (their sums to rsum_part[0 .. scan_ranges)).
 template <typename IdT>
@@ -1375,7 +1447,8 @@ void launch_count_scan(const SparseArgs &a, Launches &la, float *r, const EmaPai
                  (unsigned)len, nr, sc);
         la.mark();
     }
-    la.launch(k_sp_scan, dim3(nr), dim3(kSpThreads), 0, la.pdl(), slot, a.V, len, rng,
+    la.launch(len > kScanTile ? k_sp_scan<kTallTiles> : k_sp_scan<1>, dim3(nr), dim3(kSpThreads), 0,
+              la.pdl() && early_ranges(a.V), slot, a.V, len, rng,
              reinterpret_cast<int32_t *>(ws + L.sp_uniq), reinterpret_cast<int32_t *>(ws + L.sp_segoff),
              reinterpret_cast<int32_t *>(ws + L.sp_long), rng + kScanCounters - 1, sc, r, ema, rsum_part);
     la.mark();
@@ -1410,11 +1483,12 @@ void launch_place_order(const SparseArgs &a, Launches &la, int nw1, int rg)
     la.mark();
 }
 
-// Distinct ids, their counts and U to caller buffers.
+// Distinct ids, their counts and U to caller buffers; the map and the counters
+// cleared for the next call.
 __global__ void k_sp_export(const int32_t *__restrict__ uniq, const int32_t *__restrict__ segoff,
                             const DevScalars *__restrict__ sc, int64_t N, int32_t *__restrict__ uniq_out,
                             int32_t *__restrict__ counts_out, int32_t *__restrict__ n_unique_out,
-                            int32_t *__restrict__ counters, int ncounters)
+                            int32_t *__restrict__ slot, int32_t *__restrict__ counters, int ncounters)
 {
     grid_dep_wait();
     if (blockIdx.x == 0)
@@ -1424,7 +1498,9 @@ __global__ void k_sp_export(const int32_t *__restrict__ uniq, const int32_t *__r
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < N;
          u += (int64_t)gridDim.x * blockDim.x) {
         if (u < U) {
-            uniq_out[u] = uniq[u];
+            const int id = uniq[u];
+            uniq_out[u] = id;
+            slot[id] = 0;  // the map is all zero again for the next call
             counts_out[u] = segoff[u + 1] - segoff[u];
         }
     }
@@ -1489,7 +1565,7 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
                 la.err = cudaFuncSetAttribute(k_sp_dedup_small<IdT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)sm);
             la.launch(k_sp_dedup_small<IdT>, dim3(nkey + scan_ranges(a.V)), dim3(kSmallThreads), sm,
-                      la.pdl() && small_first_pdl(a.N), ids, (int)a.N, a.V, perm, segidx, uniq, single, bounds, cuts,
+                      la.pdl() && small_first_pdl(a.N) && early_ranges(a.V), ids, (int)a.N, a.V, perm, segidx, uniq, single, bounds, cuts,
                       G / NS, map.rg, sc, nkey, small_pad((int)a.N), small_log_slots((int)a.N), scan_len(a.V), a.r,
                       kc.ema, rsum_part);
         };
@@ -1587,10 +1663,8 @@ cudaError_t launch_sparse_unique(const SparseArgs &a, int32_t *uniq_out, int32_t
     if (nb > 4 * kGridCtas)
         nb = 4 * kGridCtas;
     la.launch(k_sp_export, dim3((int)nb), dim3(kThreads), 0, la.pdl(), uniq, segoff, sc, a.N,
-             uniq_out, counts_out, n_unique_out, reinterpret_cast<int32_t *>(a.ws + a.lay.sp_rng), kScanCounters);
-    // the touched-row map must be all-zero again before the next step
-    if (la.err == cudaSuccess)
-        la.err = cudaMemsetAsync(a.ws + a.lay.sp_slot, 0, sizeof(int32_t) * (size_t)a.V, a.stream);
+             uniq_out, counts_out, n_unique_out, reinterpret_cast<int32_t *>(a.ws + a.lay.sp_slot),
+             reinterpret_cast<int32_t *>(a.ws + a.lay.sp_rng), kScanCounters);
     return finish(a, la);
 }
 

@@ -4,6 +4,7 @@ tables that fill one id range, its neighbours and more than one scan tile."""
 import pytest
 import torch
 
+from paper_2607_01455_gb300 import ember
 from paper_2607_01455_gb300.ember import Ember
 from parity import Opt
 from test_sparse_gpu import check_dedup, gated_sparse_step
@@ -78,3 +79,32 @@ def test_stretches_of_one_id(cuda_device, lead, length):
     emb.step_sparse(W1, ids, rows, 1e-3, 1)
     ref.step_sparse(W2, ids[order], rows[order].contiguous(), 1e-3, 1)
     assert torch.equal(W1, W2) and torch.equal(emb.state, ref.state)
+
+
+@pytest.mark.parametrize("V", [311296, 311297, 304 * 8192, 304 * 8192 + 5, 5000001])
+@pytest.mark.parametrize("N", [9, 3500])
+def test_tall_tables(cuda_device, V, N):
+    """Ranges of one tile, of one and a bit, of a whole batch of tiles, of more;
+    mostly empty ones, ids in the first and last rows; r on a 16-byte boundary
+    and off it give the same bits, and the dedup clears its map each time."""
+    D = 4
+    g = torch.Generator(device=cuda_device).manual_seed(V + N)
+    ids = torch.randint(0, V, (N,), generator=g, device=cuda_device)
+    ids[:6] = torch.tensor([0, V - 1, V - 1, 1024, 8191, 8192], device=cuda_device)
+    ids[N // 2:] = ids[N // 2:] % 3000 + V // 2
+    emb = Ember(V, D, wdtype="f32", max_sparse_N=N, device=cuda_device)
+    check_dedup(emb, ids)
+    check_dedup(emb, ids.flip(0))
+    W = torch.randn(V, D, generator=g, device=cuda_device)
+    W0 = W.clone()
+    emb.state.copy_(torch.rand(V + D, generator=g, device=cuda_device) * 1e-6)
+    st0 = emb.state.clone()
+    rows = torch.randn(N, D, generator=g, device=cuda_device) * 1e-3
+    gated_sparse_step(emb, W, ids, rows, 1e-3, 3, Opt())
+    buf = torch.empty(V + D + 3, device=cuda_device)
+    for off in (1, 2, 3):
+        st = buf[off:off + V + D]
+        st.copy_(st0)
+        W1 = W0.clone()
+        ember.ember_step_sparse(emb.handle, W1, ids, ember.EMBER_I64, N, rows, st, 1e-3, 3)
+        assert torch.equal(st, emb.state) and torch.equal(W1, W)
