@@ -25,7 +25,7 @@ Layout make_layout(int64_t V, int64_t D, int64_t max_sparse_N)
     const size_t nstate = (size_t)((D + kStateCols - 1) / kStateCols);
     L.scalars = take(sizeof(DevScalars));
     L.rsum_part = take(sizeof(float) * kRsumParts);
-    L.csum_part = take(sizeof(double) * nstate);
+    L.csum_part = take(sizeof(float) * nstate);
     L.colpart = take(sizeof(float) * (size_t)kPartRows * (size_t)D);
     if (max_sparse_N > 0) {
         const size_t N = (size_t)max_sparse_N;

@@ -517,8 +517,8 @@ k_state_dense(ColSource src, float *__restrict__ rsum_part, float *__restrict__ 
             }
             rsum = tsum;
         } else {
-            // sparse step: the touched rows only (the segment-sum kernel has
-            // decayed every other row): each adds its sums of g^2 per slice
+            // sparse step: the touched rows only (the dedup has decayed every
+            // other row): each adds its sums of g^2 per slice
             const int64_t U = sc->n_unique;
             for (int64_t u = (int64_t)rb * kStateThreads + threadIdx.x; u < U; u += stride) {
                 const int64_t i = rowp.uniq[u];
@@ -878,7 +878,7 @@ struct SmallArgs {
 // (one 16- or 8-byte slot per thread, per row and access of each reduce
 // iteration), then D floats of the column partial, (256 / tpr) x D floats of
 // the row groups' sums, D floats each of the old c and the new c (then the
-// column scales), ceil(D/32) floats, and the new r of the CTA's rows.
+// column scales), ceil(D/8) floats, and the new r of the CTA's rows.
 template <int CPT, int R, bool BF16>
 __host__ __device__ constexpr size_t small_slots(int nits) { return (size_t)nits * R * CPT * kThreads; }
 
@@ -1019,7 +1019,7 @@ k_dense_cluster(SmallArgs a)
         for (int j = tid; j < D; j += kThreads)
             a.c[j] = cnew[j];
 
-    // the update, as apply_rows forms it, from the kept G and W
+    // the update, by the arithmetic of k_apply_dense, from the kept G and W
     const float inv_bc = a.kc.inv_bc;
     const float inv_s = (a.variant == EMBER_VARIANT_FULL) ? norm : 1.f;
     float *cs = cnew;  // the column scales replace the new c (already written out)
@@ -1159,8 +1159,8 @@ k_rowonly_dense(void *__restrict__ W, const float *__restrict__ G, float *__rest
     // the old r of the row that this thread finishes, an iteration ahead: a
     // trip to L2 between the two barriers of every iteration otherwise (50304 x
     // 2048: 132 us per step against 151).  Not with eight accesses per row,
-    // whose 128 registers have no room for it (128256 x 8192: 1226 us without,
-    // 1251 with it).
+    // whose 128 registers have no room for it (128256 x 8192: 1200 us without,
+    // 1235 with it).
     constexpr bool kAhead = CPT <= 4;
     auto old_r = [&](int64_t base) {
         const int64_t i = base + (int64_t)g * R + l;

@@ -216,15 +216,15 @@ inline int reduce_rows_per_thread(int64_t V, int64_t D, const ColMap &m)
     return rows <= (int64_t)(kThreads / m.tpr) * (r / 2) ? r / 2 : r;
 }
 
-// Default limit of a bounded wait inside a kernel (grid barriers, mbarrier
-// waits): 2 s of wall time.
+// Default limit of a bounded wait inside a kernel (the LM-head kernel's
+// mbarrier waits): 2 s of wall time.
 constexpr uint64_t kDefaultWaitNs = 2000000000ull;
 
 cudaError_t launch_dense_step(const DenseArgs &a);
 
 // beta2 r + (1 - beta2) m is formed in fp32 with each coefficient carried as
 // a float pair hi + lo (hi the coefficient rounded to fp32, lo the rest),
-// computed once on the host.  See ema_pair() in ember_dense.cu.
+// computed once on the host (see ema_pair()).
 struct EmaPair {
     float bh, bl, ah, al;
 };
@@ -279,7 +279,7 @@ struct NormSource {
 // Column totals are exact fixed-point sums of the nparts partial rows
 // (ember_device.cuh).
 // For the sparse step (slot set) the row pass covers only the U touched rows
-// uniq[0..U) (the segment-sum kernel decays the others) and writes its
+// uniq[0..U) (the dedup decays the others) and writes its
 // per-CTA sums of r from rsum_part[rsum_base] on.
 cudaError_t launch_state(const float *colpart, int nparts, float *rsum_part, float *c,
                          float *csum_part, const DevScalars *sc, int64_t V, int D, const StepConsts &k,

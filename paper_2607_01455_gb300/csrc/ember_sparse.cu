@@ -12,7 +12,8 @@
 //   - only the touched rows of W change.
 //
 // Kernels, in launch order:
-//   dedup     a counting sort by id, linear in N and V, in integer atomics:
+//   dedup     a counting sort by id, in integer atomics, linear in N and V but
+//             for runs of more than 128 occurrences (see k_sp_order):
 //             k_sp_count counts each id's occurrences in the V-entry map and
 //             hands every occurrence an arrival number; k_sp_scan turns the
 //             counts into the distinct ids (ascending) and where each id's run
@@ -38,7 +39,7 @@
 //             column panel for tables wider than a CTA holds).
 //
 // Every kernel is launched with programmatic dependent launch (but see
-// small_first_pdl) and waits (griddepcontrol.wait) before it reads anything.
+// small_first_pdl and early_ranges) and waits (griddepcontrol.wait) before it reads anything.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -472,6 +473,11 @@ __device__ __forceinline__ void worker_starts(int p, int u, int before, int s, i
 // window of kWinBits are bits of a bitmap in shared memory, read back in
 // order; the first `nbig` CTAs take the (long run, window) pairs.  A long
 // run is bound by its trips to L2, so a thread has 16 occurrences in flight.
+//   Every window reads its whole run, so a long run of L occurrences costs
+// L ceil(N / kWinBits) reads and as many bitmaps of kWinWords: linear in N
+// while one window holds the batch, then with its square (1M uniform ids over
+// 4000 rows, 4000 long runs and 16 windows: 0.70 ms here; the tile sort and
+// ranks before took 4.6).
 constexpr int kWinWords = 2048;
 constexpr int kWinBits = 32 * kWinWords;
 // Runs from this length on are looked through for stretches of nothing but one
@@ -1400,8 +1406,11 @@ cudaError_t finish(const SparseArgs &a, const Launches &la)
 
 // Fewest occurrences that are counted through the hash table: below, at most
 // 3.3 ns of atomics queue on one address per 32 occurrences of one id, and
-// the direct form's one trip to L2 ends sooner (32768 Zipf ids: 5.6 us
-// against 7.2; 262144: 27.8 against 14.4).
+// the direct form's one trip to L2 ends sooner.  Zipf ids over 50257 x 256, us
+// per step through the table and directly: 32768 48.5 and 45.0, 49152 53.0
+// and 52.9, 65536 59.1 and 59.6, 131072 74.1 and 79.8, 262144 113.3 and 130.1
+// (uniform ids, where no address queues: 53.9 and 51.7, 58.5 and 56.1, 76.1 and
+// 74.6, 105.3 and 107.8 from 49152 on).
 constexpr int64_t kTableMinN = 65536;
 
 // Ids per range of k_sp_count and k_sp_scan, and the number of ranges: a
@@ -1509,11 +1518,15 @@ __global__ void k_sp_export(const int32_t *__restrict__ uniq, const int32_t *__r
 }
 
 // Whether the one dedup kernel of a small batch may be launched while the
-// kernel before it on the stream is still running.  With few CTAs it gains
-// its launch latency, 128 ids over 67019 x 480: 22.7 us per step against 24.0.
-// With many, its waiting CTAs cost the kernel before it more: 1024 ids over
-// 50257 x 768 take 28.6 us with it and 26.6 without, 1384 over 5656 x 96 31.6
-// and 27.9.
+// kernel before it on the stream is still running.  Early, it gains a launch
+// latency; the CTAs that then wait hold SMs which the kernel before, the update
+// of the step before in a run of steps, still wants, and their number grows
+// with N.  us per step early and not: 50257 x 768, 64 Zipf ids 18.9 and 20.8,
+// 128 21.0 and 22.8, 256 22.9 and 23.1, 384 24.2 and 24.8, 512 26.1 and 24.8,
+// 1024 27.9 and 25.5.  The line does not move with V: 128 ids of 256 columns
+// 20.5 and 21.0 over 2000 rows, 19.2 and 20.7 over 16384, 21.5 and 22.8 over
+// 262144, 22.3 and 23.1 over 1000000; 1024 ids 25.7 and 23.0, 25.2 and 23.0,
+// 25.5 and 23.9, 26.5 and 24.8.
 bool small_first_pdl(int64_t N) { return N <= 256; }
 
 template <int VEC, int CPT>
@@ -1543,9 +1556,8 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     const dim3 sum_threads(map.rg * map.tpb);
     Launches la{a.trace, a.n_trace, 0, a.stream};
 
-    auto *segsum = sum_threads.x > 192   ? k_sp_segsum<VEC, 256>
-                   : sum_threads.x > 128 ? k_sp_segsum<VEC, 192>
-                                         : k_sp_segsum<VEC, 128>;
+    // (a CTA has 160, 192, 224 or 256 threads: see sum_map)
+    auto *segsum = sum_threads.x > 192 ? k_sp_segsum<VEC, 256> : k_sp_segsum<VEC, 192>;
     // the ring and the static arrays together pass 48 KiB
     cudaError_t e = cudaFuncSetAttribute(segsum, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
     if (e == cudaSuccess)
