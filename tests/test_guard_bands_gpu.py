@@ -43,7 +43,8 @@ def test_dense_steps_stay_in_bounds(cuda_device, V, D, wdtype, variant):
     assert emb.device_status() == 0
 
 
-@pytest.mark.parametrize("V,D,N", [(1000, 33, 3001), (5000, 127, 1025), (300, 2048, 4097)])
+@pytest.mark.parametrize("V,D,N", [(1000, 33, 3001), (5000, 127, 1025), (300, 2048, 4097), (1000, 33, 5001),
+                                    (5000, 127, 3073), (40, 1100, 9001)])
 def test_sparse_steps_stay_in_bounds(cuda_device, V, D, N):
     emb = Ember(V, D, wdtype="bf16", max_sparse_N=N, device=cuda_device)
     wbuf, W = guarded(V * D, torch.bfloat16, cuda_device, -7.0)

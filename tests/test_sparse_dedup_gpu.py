@@ -1,6 +1,7 @@
-"""Edges of the sparse step's counting dedup: runs as long as a thread orders
-(128) and longer, occurrences on both sides of a bitmap window (65536), and
-tables that fill one id range, its neighbours and more than one scan tile."""
+"""Edges of the sparse step's dedup, both of its forms (one launch up to 3072
+occurrences, a counting sort above): runs as long as a thread orders (128) and
+longer, occurrences on both sides of a bitmap window (65536), and tables that
+fill one id range, its neighbours and more than one scan tile."""
 import pytest
 import torch
 
@@ -13,12 +14,18 @@ pytestmark = pytest.mark.gpu
 
 
 def ids_of(V, counts, N, device, seed):
-    """N shuffled ids: counts[i] times id i * (V - 1) / len, the rest uniform."""
+    """N shuffled ids: exactly counts[i] times id i * (V - 1) / len, the rest
+    uniform over the other ids."""
     g = torch.Generator(device=device).manual_seed(seed)
     k = len(counts)
-    parts = [torch.full((c,), i * (V - 1) // max(1, k - 1), device=device, dtype=torch.int64)
-             for i, c in enumerate(counts)]
-    ids = torch.cat(parts + [torch.randint(0, V, (N - sum(counts),), generator=g, device=device)])
+    at = [i * (V - 1) // max(1, k - 1) for i in range(k)]
+    parts = [torch.full((c,), i, device=device, dtype=torch.int64) for i, c in zip(at, counts)]
+    others = torch.ones(V, dtype=torch.bool, device=device)
+    others[at] = False
+    others = others.nonzero().flatten()
+    if N > sum(counts):
+        parts.append(others[torch.randint(0, others.numel(), (N - sum(counts),), generator=g, device=device)])
+    ids = torch.cat(parts)
     return ids[torch.randperm(N, generator=g, device=device)]
 
 
@@ -26,6 +33,10 @@ def ids_of(V, counts, N, device, seed):
     (300, 1100, (127, 128, 129)), (256, 129, (129,)), (257, 600, (300, 130)), (77824, 3000, (130, 1, 2)),
     (77825, 5000, (1000, 1000, 1000)), (400000, 2000, (129, 500)),
     (1000, 65536, (65536,)), (1000, 65537, (65537,)), (50000, 270000, (140000, 300, 90000)),
+    # either side of the line between the two forms, and of the longest run a
+    # thread of the counting form orders
+    (1000, 3072, (127, 128, 129)), (1000, 3073, (127, 128, 129)), (70000, 3500, (129,)), (70000, 3500, (128,)),
+    (9000, 9000, (128, 129) * 20), (60000, 140000, (129, 128, 127, 70000)),
 ])
 @pytest.mark.parametrize("idtype", [torch.int64, torch.int32])
 def test_dedup_edges(cuda_device, V, N, counts, idtype):
@@ -37,6 +48,31 @@ def test_dedup_edges(cuda_device, V, N, counts, idtype):
     for t in (1, 2):
         rows = torch.randn(N, D, device=cuda_device, generator=torch.Generator(device=cuda_device).manual_seed(t)) * 1e-4
         gated_sparse_step(emb, W, ids, rows, 1e-3, t, Opt())
+
+
+@pytest.mark.parametrize("V,N,counts", [
+    (5000, 900, (127, 128, 129)), (5000, 3072, (5, 300)), (5000, 3073, (5, 300)), (70000, 9000, (128, 129) * 20),
+    (5000, 40000, (127, 128, 129, 20000)), (5000, 140000, (128, 129, 70000)), (3, 5000, (1700, 1700, 1600)),
+])
+def test_runs_are_summed_in_increasing_occurrence(cuda_device, V, N, counts):
+    """The bits of a batch are those of the same batch sorted by id beforehand
+    (stably): every run is added in increasing occurrence.  The values span
+    eight decades, so that another order shows: of 64 columns, swapping two of
+    2, 3, 5 or 129 occurrences changes 1, 8, 7 or 20 compensated sums."""
+    D = 64
+    ids = ids_of(V, counts, N, cuda_device, N)
+    g = torch.Generator(device=cuda_device).manual_seed(N)
+    rows = torch.randn(N, D, generator=g, device=cuda_device) * 1e-4
+    rows *= 10 ** (torch.rand(N, D, generator=g, device=cuda_device) * 8 - 4)
+    order = torch.sort(ids, stable=True).indices
+    outs = []
+    for i, x in ((ids, rows), (ids[order], rows[order].contiguous())):
+        emb = Ember(V, D, wdtype="f32", max_sparse_N=N, device=cuda_device)
+        W = torch.zeros(V, D, device=cuda_device)
+        for t in (1, 2):
+            emb.step_sparse(W, i, x, 1e-3, t)
+        outs.append((W, emb.state))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
 
 
 def test_order_within_runs_is_deterministic(cuda_device):

@@ -67,8 +67,8 @@ def check_dedup(emb, ids):
     np.testing.assert_array_equal(counts.cpu().numpy(), want_c)
 
 
-# 1024-key sort tiles: 4096, 4097, 32768, 32769, 65536 and 65537 sit on tile
-# edges; the largest batch spans 98 tiles.
+# Batches of one launch (up to 3072 ids), of direct counts (up to 65535) and of
+# counts through the hash table; 65536 ids fill one bitmap window.
 @pytest.mark.parametrize("V,D,N", [
     (50, 8, 1), (50, 8, 37), (1000, 64, 4096), (1000, 64, 4097), (5000, 200, 9000),
     (3000, 203, 5000), (262144, 128, 12288), (100, 2048, 3000), (20000, 8192, 700),
@@ -92,7 +92,7 @@ def test_dedup_bit_exact(cuda_device, V, D, N, idtype):
     # two column slices of the segment sums, the second 8 columns wide
     # (1032 = 1024 + 8), and bf16 rows that do not start on 16-byte
     # boundaries (1100 = 8 * 137 + 4)
-    (1500, 1032, 2500), (3000, 1100, 4000),
+    (1500, 1032, 2500), (3000, 1100, 4000), (1500, 1032, 4500),
 ])
 @pytest.mark.parametrize("wdtype", ["bf16", "f32"])
 def test_sparse_parity(cuda_device, V, D, N, wdtype):

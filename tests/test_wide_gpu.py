@@ -132,7 +132,7 @@ def test_wide_from_host_matches_device_step(cuda_device):
         assert torch.equal(a.state, b.state)
 
 
-@pytest.mark.parametrize("V,D,N", [(2000, 16384, 3000), (2000, 10001, 1500)])
+@pytest.mark.parametrize("V,D,N", [(2000, 16384, 3000), (2000, 10001, 1500), (2000, 16384, 3500), (2000, 10001, 3500)])
 def test_wide_sparse_parity(cuda_device, V, D, N):
     opt = Opt()
     emb = make(V, D, "bf16", opt, max_sparse_N=N)
