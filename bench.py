@@ -63,13 +63,13 @@ class L2Flush:
 # it came from.  A kernel that changes gets None here until it is captured
 # again.
 TRAFFIC = {
-    # the 32768 x 8192 quarter table measured 2.1147 GB per launch (mean of
-    # three launches); every row of G and W is read once and W written once,
+    # the 32768 x 8192 quarter table measured 2.1159 GB per launch (mean of
+    # two launches); every row of G and W is read once and W written once,
     # so the traffic is scaled by rows
     ("k_apply_dense", "dense_lmhead_v128256_d8192_bf16"): (
-        int(2.1147e9 * 128256 / 32768),
+        int(2.1159e9 * 128256 / 32768),
         "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_apply_dense on the 32768 x 8192 table, "
-        "2.1147 GB per launch, scaled by rows (2026-12-04, update by warp units)"),
+        "2.1159 GB per launch, scaled by rows (2026-12-05, update by warp units)"),
     ("k_sp_segsum", "sparse_v262144_d2048_bf16_n32768"): (
         269392213, "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_sp_segsum on this workload "
                    "(2026-12-04, ring of rows)"),
