@@ -772,24 +772,26 @@ cudaError_t launch_apply_t(const ApplyArgs &a, const ApplyMap &m, bool bf16)
 
 // Whether rows of pw columns that start on no 16-byte boundary take shifted
 // 16-byte accesses in the update rather than 4-byte ones.  A row's two partial
-// accesses go element by element, which short rows (above all of bf16
-// weights) do not earn back, nor do widths just past a power of two, where few
-// of the shifted form's lanes have anything to do.  Steps of 63e6 elements (of
-// 400000 rows below 157 columns), us shifted and 4-byte: fp32 7 columns 42.8
-// and 40.5, 9 42.9 and 48.7, 33 86.7 and 85.7, 61 95.8 and 95.0, 63 137 and 96,
-// 97 151 and 143, 129 199 and 220, 255 190 and 182, 257 210 and 286, 1023 184
-// and 182, 1119 194 and 217; bf16 29 66 and 68, 61 119 and 90, 129 247 and 211,
-// 253 181 and 164, 257 228 and 276, 511 169 and 163, 513 191 and 208, 1003 140
-// and 165, 1025 204 and 192, 2047 143 and 166.
+// accesses go element by element, which rows of 32 columns and more (above all
+// of bf16 weights) have to earn back, and widths just past a power of two
+// leave most of the shifted form's lanes idle.  Steps of 63e6 elements (of
+// 400000 rows below 157 columns), us shifted and 4-byte: fp32 5 columns 37.6
+// and 40.2, 7 42.8 and 40.5, 9 42.9 and 48.7, 33 86.7 and 85.7, 61 95.8 and
+// 95.0, 63 137 and 96, 97 151 and 143, 129 199 and 220, 255 190 and 182, 257
+// 210 and 286, 1023 184 and 182, 1119 194 and 217; bf16 9 49.2 and 49.5
+// (2^20 rows 101.7 and 105.7), 29 66 and 68, 33 105 and 82, 61 119 and 90, 129
+// 247 and 211, 253 181 and 164, 257 228 and 276, 511 169 and 163, 513 191 and
+// 208, 1003 140 and 165, 1025 204 and 192, 2047 143 and 166.
 bool shifted_pays(int pw, bool bf16)
 {
     auto lanes = [&](bool rag) {
         const ApplyMap m = apply_map(pw, rag ? 4 : 1, rag, bf16);
         return m.lpr * m.k * m.nseg;
     };
+    const int shifted = lanes(true), narrow = lanes(false);
     if (bf16)
-        return pw >= 256 && 5 * lanes(true) < 2 * lanes(false);
-    return pw >= 256 || ((pw >= 128 || (pw >= 8 && pw < 64)) && 2 * lanes(true) < lanes(false));
+        return pw < 32 ? 2 * shifted < narrow : pw >= 256 && 5 * shifted < 2 * narrow;
+    return pw >= 256 || ((pw >= 128 || pw < 64) && 2 * shifted < narrow);
 }
 
 // vec 4: every row starts on a 16-byte boundary of G (and as many elements
