@@ -64,6 +64,7 @@ constexpr int kLongRun = 128;
 // Batches of up to kSmallN occurrences are deduped in one launch (see
 // k_sp_dedup_small for both sides of the line).
 constexpr int kSmallN = 3072;
+constexpr int kSmallTallN = 4096;
 
 // Workspace layout (byte offsets, each 256-byte aligned).
 struct Layout {

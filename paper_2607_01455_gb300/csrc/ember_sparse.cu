@@ -603,13 +603,17 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
 // batch takes no longer than a flat one.  50257 x 768, Zipf ids, us per step
 // with it and with the four kernels: 1024 ids 25.3 and 30.2, 1536 25.9 and
 // 29.4, 2048 29.2 and 30.9, 3000 30.8 and 31.7 (262144 x 2048: 38.3 and 38.0).
+// 2^24 x 8, where the four kernels scan a map of 64 MB: 3500 ids 51.7 and
+// 78.5, 4096 57.9 and 80.3; 10^7 x 8 43.8 and 56.9, 49.5 and 57.8.
 // Without the table, runs numbered by their first position, 1024 ids took
 // 24.6, but the workers' shares and the sums of r depended on the padding.
 //   The CTAs from `nkey` on decay r on the rows outside the batch, the ranges
-// and tiles of k_sp_scan, from a bitmap of the ids.
+// and tiles of k_sp_scan, from a bitmap of the ids, kDecayTiles tiles at once
+// (1024 ids over 2^23 x 8 31.1 us per step, one at a time 37; eight 33.1).
 // ---------------------------------------------------------------------------
 constexpr int kSmallThreads = 512;
 constexpr int kBitmapWords = 2048;
+constexpr int kDecayTiles = 4;  // in flight per CTA
 constexpr int small_pad(int N) { return (N + 127) / 128 * 128; }
 // 1 << log_slots entries of the hash table: at least half stay empty.
 constexpr int small_log_slots(int N)
@@ -771,10 +775,18 @@ k_sp_dedup_small(const IdT *__restrict__ ids, int N, int64_t V, int32_t *__restr
         }
         __syncthreads();
         // by the threads and in the order of k_sp_scan
-        for (int q = tid * kScanPer; tid < kSpThreads && q < n; q += kScanTile) {
-            float rr[kScanPer];
-            load_r4(r, aligned, c0 + q, c0 + n, rr);
-            decay_r4(r, aligned, c0 + q, c0 + n, ema, (unsigned)words[q >> 5] >> (q & 31), rr, rsum);
+        for (int q0 = tid * kScanPer; tid < kSpThreads && q0 < n; q0 += kDecayTiles * kScanTile) {
+            float rr[kDecayTiles][kScanPer];
+#pragma unroll
+            for (int d = 0; d < kDecayTiles; ++d)
+                if (q0 + d * kScanTile < n)
+                    load_r4(r, aligned, c0 + q0 + d * kScanTile, c0 + n, rr[d]);
+#pragma unroll
+            for (int d = 0; d < kDecayTiles; ++d) {
+                const int q = q0 + d * kScanTile;
+                if (q < n)
+                    decay_r4(r, aligned, c0 + q, c0 + n, ema, (unsigned)words[q >> 5] >> (q & 31), rr[d], rsum);
+            }
         }
         __syncthreads();
     }
@@ -1529,6 +1541,14 @@ __global__ void k_sp_export(const int32_t *__restrict__ uniq, const int32_t *__r
 // 25.5 and 23.9, 26.5 and 24.8.
 bool small_first_pdl(int64_t N) { return N <= 256; }
 
+// Whether a batch takes the one-launch dedup: up to kSmallN occurrences, and,
+// of a table so tall that the counting form's scan of the map shows, up to
+// kSmallTallN (see k_sp_dedup_small for both sides of the lines).
+bool one_launch_dedup(int64_t N, int64_t V)
+{
+    return N > 0 && (N <= kSmallN || (N <= kSmallTallN && V >= int64_t(1) << 23));
+}
+
 template <int VEC, int CPT>
 cudaError_t launch_sparse_t(const SparseArgs &a)
 {
@@ -1568,7 +1588,7 @@ cudaError_t launch_sparse_t(const SparseArgs &a)
     la.mark();
     const int G = kSparseCtas;
     const StepConsts kc = make_consts(a.beta2, a.one_minus_beta2, a.V, a.D, a.inv_bc);
-    if (a.N > 0 && a.N <= kSmallN) {
+    if (one_launch_dedup(a.N, a.V)) {
         const int nkey = (int)((a.N + kSmallThreads / 32 - 1) / (kSmallThreads / 32));
         const size_t sm = small_smem((int)a.N);
         auto go = [&](auto *ids) {

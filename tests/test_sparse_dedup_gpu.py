@@ -117,7 +117,7 @@ def test_stretches_of_one_id(cuda_device, lead, length):
     assert torch.equal(W1, W2) and torch.equal(emb.state, ref.state)
 
 
-@pytest.mark.parametrize("V", [311296, 311297, 304 * 8192, 304 * 8192 + 5, 5000001])
+@pytest.mark.parametrize("V", [311296, 311297, 304 * 8192, 304 * 8192 + 5, 5000001, (1 << 23) + 3])
 @pytest.mark.parametrize("N", [9, 3500])
 def test_tall_tables(cuda_device, V, N):
     """Ranges of one tile, of one and a bit, of a whole batch of tiles, of more;

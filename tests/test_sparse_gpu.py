@@ -206,6 +206,7 @@ def test_sparse_edge_cases(cuda_device):
     # occurrences) to the counting one, and from its direct counts to the table
     (20000, 256, 3000, 3900), (20000, 256, 3000, 6000), (500, 64, 3072, 3073), (70000, 2048, 1000, 4500),
     (400000, 203, 3072, 70000), (3000, 1, 1, 5000), (20000, 64, 40000, 66000),
+    (9000001, 8, 3500, 4200),
 ])
 def test_skipped_ids_leave_the_step_bit_identical(cuda_device, V, D, N, Npad):
     """The same batch, and the batch followed by skipped ids (id -1, whose
