@@ -398,14 +398,8 @@ k_sp_place(const IdT *__restrict__ ids, int64_t N, const int32_t *__restrict__ s
 // per summed row written (runs are numbered in order, so the cost rises by
 // one or two per position).  Worker w owns [first(w), first(w + 1)), where
 // first(w) is the smallest position whose cost reaches T(w) = w C / nw and
-// C = n_valid + U.
-// I: int64_t, or int where 2 kSmallN times the number of workers fits it (64-bit
-// divisions take most of a microsecond of the one-launch dedup).
-template <typename I>
-__device__ __forceinline__ I cost_target(int w, int nw, I C)
-{
-    return ((I)w * C) / nw;
-}
+// C = n_valid + U.  T(w) <= c where w C < (c + 1) nw: the tests below multiply
+// instead of dividing.
 
 // Workers in use, of the nw1 rg groups of a slice's CTAs (group g of CTA b is
 // worker g nw1 + b): nw1 times as many groups as have kMinRows occurrences
@@ -422,19 +416,6 @@ __device__ __forceinline__ int workers_of(int n_valid, int nw1, int rg)
     return nw1 * (most < 1 ? 1 : most < rg ? most : rg);
 }
 
-// Worker whose range holds sorted position p of run u.
-template <typename I>
-__device__ __forceinline__ int worker_of(int p, int u, int nw, I C)
-{
-    const I c = (I)p + u;
-    int w = (int)((c * nw) / C);
-    while (w + 1 < nw && cost_target(w + 1, nw, C) <= c)
-        ++w;
-    while (w > 0 && cost_target(w, nw, C) > c)
-        --w;
-    return w;
-}
-
 // The workers that start at position p, of run u, which holds [s, e); `before`
 // is the run of position p - 1 (-1 for p = 0): those whose target lies above
 // the cost of the position before p and not above that of p, and, at the last
@@ -443,6 +424,7 @@ __device__ __forceinline__ int worker_of(int p, int u, int nw, I C)
 // worker it ends in, or (-1, 0).  Both forms of the dedup take the starts from
 // here: the sums of a batch do not depend on which one its length chooses.
 // Threads `first` of `step` share the workers.
+// I: int64_t, or int where 2 kSmallTallN times the number of workers fits it.
 template <typename I>
 __device__ __forceinline__ void worker_starts(int p, int u, int before, int s, int e, int n_valid, int U, int nw1,
                                               int rg, int32_t *__restrict__ bounds, int2 *__restrict__ cuts,
@@ -453,13 +435,15 @@ __device__ __forceinline__ void worker_starts(int p, int u, int before, int s, i
     const I c1 = (I)p + u;
     const I c0 = p > 0 ? (I)p - 1 + before : -1;
     for (I q = ((c0 + 1) * nw + C - 1) / C + first; q < nw; q += step) {
-        const bool here = cost_target((int)q, nw, C) <= c1;
+        const bool here = q * C < (c1 + 1) * nw;
         if (!here && p + 1 < n_valid)
             break;
         bounds[q] = here ? p : n_valid;
         int2 cut = make_int2(-1, 0);
-        if (here && s < p && q > 0 && cost_target((int)q - 1, nw, C) <= (I)s + u)
-            cut = make_int2(u, worker_of(e - 1, u, nw, C));
+        if (here && s < p && q > 0 && (q - 1) * C < ((I)s + u + 1) * nw) {
+            const I to = (((I)e + u) * nw - 1) / C;  // the last whose target is not above the cost of e - 1
+            cut = make_int2(u, (int)(to < nw ? to : nw - 1));
+        }
         cuts[q] = cut;
     }
     if (p + 1 == n_valid && first == 0)
@@ -599,14 +583,15 @@ k_sp_order(const int32_t *__restrict__ placed, const int32_t *__restrict__ segid
 // Nothing has to be scanned, and numbers, worker starts and the order in
 // which r is summed are those of the four kernels above, so that a batch gives
 // the same bits however many skipped ids it is padded with.
-//   Bound by the N^2 integer compares and adds, over the CTAs, so a skewed
-// batch takes no longer than a flat one.  50257 x 768, Zipf ids, us per step
-// with it and with the four kernels: 1024 ids 25.3 and 30.2, 1536 25.9 and
-// 29.4, 2048 29.2 and 30.9, 3000 30.8 and 31.7 (262144 x 2048: 38.3 and 38.0).
+//   Bound by the N^2 integer compares and adds, over the CTAs, and by the tries
+// that a CTA's last lane needs for its entry of the table.  50257 x 768, Zipf
+// ids, us per step with it and with the four kernels: 1024 ids 25.3 and 30.2,
+// 1536 25.8 and 29.4, 2048 29.1 and 30.9, 3000 29.5 and 31.7 (262144 x 2048:
+// 38.3 and 38.0).
 // 2^24 x 8, where the four kernels scan a map of 64 MB: 3500 ids 51.7 and
 // 78.5, 4096 57.9 and 80.3; 10^7 x 8 43.8 and 56.9, 49.5 and 57.8.
-// Without the table, runs numbered by their first position, 1024 ids took
-// 24.6, but the workers' shares and the sums of r depended on the padding.
+// Without the table, runs numbered by their first position, 1024 Zipf ids took
+// 24.6 to 24.9 and as many uniform ones 24.2 (27.1 with it), but the workers' shares and the sums of r depended on the padding.
 //   The CTAs from `nkey` on decay r on the rows outside the batch, the ranges
 // and tiles of k_sp_scan, from a bitmap of the ids, kDecayTiles tiles at once
 // (1024 ids over 2^23 x 8 31.1 us per step, one at a time 37; eight 33.1).
@@ -615,11 +600,13 @@ constexpr int kSmallThreads = 512;
 constexpr int kBitmapWords = 2048;
 constexpr int kDecayTiles = 4;  // in flight per CTA
 constexpr int small_pad(int N) { return (N + 127) / 128 * 128; }
-// 1 << log_slots entries of the hash table: at least half stay empty.
+// 1 << log_slots entries of the hash table: at least three quarters stay empty,
+// so that the last lane of a warp takes its entry at the second try, not the
+// fourth (2048 uniform ids: 33.3 us per step with half as many entries).
 constexpr int small_log_slots(int N)
 {
     int log_slots = 7;
-    while (1 << log_slots < 2 * N)
+    while (1 << log_slots < 4 * N)
         ++log_slots;
     return log_slots;
 }
@@ -653,23 +640,28 @@ k_sp_dedup_small(const IdT *__restrict__ ids, int N, int64_t V, int32_t *__restr
     unsigned *const weight = reinterpret_cast<unsigned *>(sid + npad);
     int *const words = sid + 2 * npad;  // hash table of the ids, or a bitmap of a range's ids
     const bool keys = (int)blockIdx.x < nkey;
+    grid_dep_wait();  // whatever ran before on the stream
+    grid_dep_launch();
+    constexpr int kAtOnce = 4;
+    int64_t id[kAtOnce];
+    auto load = [&](int q0) {
+#pragma unroll
+        for (int e = 0; e < kAtOnce; ++e)
+            id[e] = q0 + e * kSmallThreads < N ? (int64_t)ids[q0 + e * kSmallThreads] : 0;
+    };
+    load(tid);  // in flight while the table is cleared
     if (keys) {
-        for (int q = tid; q < 1 << log_slots; q += kSmallThreads)
-            words[q] = kFree;
+        for (int q = tid; q < 1 << (log_slots - 2); q += kSmallThreads)
+            reinterpret_cast<int4 *>(words)[q] = make_int4(kFree, kFree, kFree, kFree);
         if (tid < 2)
             total[tid] = 0;
         __syncthreads();
     }
-    grid_dep_wait();  // whatever ran before on the stream
-    grid_dep_launch();
     bool bad = false;
     int U = 0, valid = 0;
-    constexpr int kAtOnce = 4;
     for (int q0 = tid; q0 < npad; q0 += kAtOnce * kSmallThreads) {
-        int64_t id[kAtOnce];
-#pragma unroll
-        for (int e = 0; e < kAtOnce; ++e)
-            id[e] = q0 + e * kSmallThreads < N ? (int64_t)ids[q0 + e * kSmallThreads] : 0;
+        if (q0 != tid)
+            load(q0);
 #pragma unroll
         for (int e = 0; e < kAtOnce; ++e) {
             const int q = q0 + e * kSmallThreads;
@@ -686,9 +678,7 @@ k_sp_dedup_small(const IdT *__restrict__ ids, int N, int64_t V, int32_t *__restr
             if (ok)
                 for (unsigned h = (unsigned)x * 2654435761u >> (32 - log_slots);;  // Fibonacci hashing
                      h = (h + 1) & ((1u << log_slots) - 1)) {
-                    was = *(volatile int *)(words + h);
-                    if (was == kFree)
-                        was = atomicCAS(words + h, kFree, x);
+                    was = atomicCAS(words + h, kFree, x);
                     if (was == kFree || was == x)
                         break;
                 }
